@@ -404,6 +404,10 @@ struct dg_ctx {
     bool marks_dirty = false;  // marks or levels may be non-zero
     // x3 at order 3: tcgen05 kernels (volume, faces, projection)
     bool tc5 = false;
+    // the sum-factorised kernels: a stage is a volume and a face launch (the volume
+    // kernel of the stages after the first projects its own input), and one
+    // projection launch ends the step
+    bool sf = false;
     void* t5tab = nullptr;
     T5Maps t5maps{};  // tiled TMA descriptors of the state registers, rvol and a_h (tcgen05 kernels)
     void* rvol = nullptr;
@@ -663,9 +667,24 @@ cudaError_t tile_tc5(dg_ctx* c, const TileLaunch& t)
 cudaError_t tile(dg_ctx* c, const TileLaunch& t)
 {
     if (c->tc5) return tile_tc5(c, t);
-    Timed tm(c, t.mode == 0 ? KIND_PROJECT : KIND_RHS);
-    Launch L = make_launch(c);
-    return (c->prec == DG_PREC_F64) ? launch_tile<double>(L, t) : launch_tile<float>(L, t);
+    const Launch L = make_launch(c);
+    auto go = [&](const TileLaunch& x) {
+        Timed tm(c, x.mode == TM_PROJECT ? KIND_PROJECT : KIND_RHS);
+        return (c->prec == DG_PREC_F64) ? launch_tile<double>(L, x) : launch_tile<float>(L, x);
+    };
+    const cudaError_t e = go(t);
+    if (e != cudaSuccess || !c->sf || t.mode == TM_PROJECT || t.mode == TM_RHS || !(t.flags & F_NEXTPROJ)) return e;
+    // the projection of the stage's output, with the CFL bound
+    TileLaunch p{};
+    p.mode = TM_PROJECT;
+    p.u_in = t.out;
+    p.vh_out = t.vh_out;
+    p.vabs_out = t.vabs_out;
+    p.ahat = t.ahat;
+    p.flags = t.flags & (F_FORCE | F_DT);
+    p.abar_out = t.abar_out;
+    p.trouble = t.trouble;
+    return go(p);
 }
 
 // projection of u into vhat (+ forcing sums into abar slot, + CFL dt)
@@ -725,15 +744,13 @@ int upload_weights(dg_ctx* ctx, const float* w_host)
 
 // learned mode: the per-cell coefficient nu = cs h/p exp(net(x)) from u and
 // the projection of |v| already in c->vabs
-cudaError_t learned_infer(dg_ctx* c, const void* u)
+cudaError_t learned_infer(dg_ctx* c, const void* u, float* nu)
 {
     Timed tm(c, KIND_OTHER);
     Launch L = make_launch(c);
     return (c->prec == DG_PREC_F64)
-               ? mlp_infer<double>(L, (const double*)u, (const double*)c->vabs, nullptr, c->ncell, c->mpack, c->nu_cell,
-                                   nullptr)
-               : mlp_infer<float>(L, (const float*)u, (const float*)c->vabs, nullptr, c->ncell, c->mpack, c->nu_cell,
-                                  nullptr);
+               ? mlp_infer<double>(L, (const double*)u, (const double*)c->vabs, nullptr, c->ncell, c->mpack, nu, nullptr)
+               : mlp_infer<float>(L, (const float*)u, (const float*)c->vabs, nullptr, c->ncell, c->mpack, nu, nullptr);
 }
 
 // learned mode: projection of |v| of u (v-hat into the scratch slot 1), then the coefficient
@@ -748,7 +765,7 @@ cudaError_t learned_nu(dg_ctx* c, const void* u)
     t.abar_out = 1;
     cudaError_t e = tile(c, t);
     if (e != cudaSuccess) return e;
-    return learned_infer(c, u);
+    return learned_infer(c, u, c->nu_cell);
 }
 
 int upload_forcing(dg_ctx* ctx)
@@ -887,6 +904,7 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
     // order-3 x3 on the tcgen05 kernels (the learned sensor's in-step evaluation,
     // fused_infer, runs in their last projection)
     ctx->tc5 = ctx->prec == DG_PREC_X3 && order == 3 && nu->diffusion == 0.0 && opts->x3_backend == 0;
+    ctx->sf = ctx->prec != DG_PREC_X3 && nu->diffusion == 0.0;
     ctx->mlp_D = 2 * ctx->b;
     ctx->mlp_P = mlp_params(ctx->mlp_D);
 
@@ -1151,7 +1169,7 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
                 if (use_carry && fused)
                     std::swap(ctx->nu_cell, ctx->nu_next);
                 else
-                    CK(use_carry ? learned_infer(ctx, ctx->reg[A]) : learned_nu(ctx, ctx->reg[A]));
+                    CK(use_carry ? learned_infer(ctx, ctx->reg[A], ctx->nu_cell) : learned_nu(ctx, ctx->reg[A]));
             }
             if (!use_carry) CK(project(ctx, ctx->reg[A], vh_buf(ctx, pb), force ? ctx->ahat : nullptr, true, pb));
             for (int s = 0; s < ctx->rk; ++s) {
@@ -1160,7 +1178,7 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
                 t.nu = learned ? ctx->nu_cell : nullptr;
                 t.mode = (learned && last) ? 3 : 2;
                 t.nu_next = (learned && last && fused) ? ctx->nu_next : nullptr;
-                t.vabs_out = (learned && last && !fused) ? ctx->vabs : nullptr;
+                t.vabs_out = (learned && last && (!fused || ctx->sf)) ? ctx->vabs : nullptr;
                 t.mlp = ctx->mpack;
                 t.u_in = ctx->reg[in[s]];
                 t.u_n = ctx->reg[A];
@@ -1174,13 +1192,16 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
                 // the stages after the first project their own input in the volume
                 // kernel instead (driven: with the forcing sums), so only the last
                 // stage's output gets a projection launch
-                const bool fold = ctx->tc5;
+                const bool fold = ctx->tc5 || ctx->sf;
                 t.flags = (force ? F_FORCE : 0) | ((fold && !last) ? 0 : F_NEXTPROJ) | (last ? F_DT : 0) |
                           ((fold && s > 0) ? F_SELFPROJ : 0);
                 t.abar_in = (pb + s) & 1;
                 t.abar_out = (pb + s + 1) & 1;
                 t.trouble = marks;
                 CK(tile(ctx, t));
+                // fused_infer on the sum-factorised kernels: the next step's coefficient
+                // from the |v| projection the stage has just left
+                if (ctx->sf && t.nu_next) CK(learned_infer(ctx, t.out, ctx->nu_next));
             }
             struct {
                 unsigned int status;
@@ -1437,7 +1458,7 @@ int dg_av_nu_carried(dg_ctx* ctx, float* nu_out)
     if (!nu_out) return fail(ctx, DG_EINVAL, "dg_av_nu_carried: null buffer");
     if (ctx->nu.mode != DG_AV_LEARNED || !ctx->carry)
         return fail(ctx, DG_ESTATE, "dg_av_nu_carried: no coefficient carried from a learned step");
-    if (!ctx->nu.fused_infer) CK(learned_infer(ctx, ctx->reg[ctx->cur]));
+    if (!ctx->nu.fused_infer) CK(learned_infer(ctx, ctx->reg[ctx->cur], ctx->nu_cell));
     const float* src = ctx->nu.fused_infer ? ctx->nu_next : ctx->nu_cell;
     CK(cudaMemcpyAsync(nu_out, src, sizeof(float) * ctx->ncell, cudaMemcpyDeviceToDevice, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));

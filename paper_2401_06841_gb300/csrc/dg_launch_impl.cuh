@@ -8,6 +8,14 @@
 
 namespace dg {
 
+// the sum-factorised kernels (dg_sf_impl.cuh, instantiated in dg_sf_*.cu)
+namespace sf {
+template <typename T, int K>
+cudaError_t setup();
+template <typename T, int K>
+cudaError_t launch(const Launch& L, const TileLaunch& t);
+}  // namespace sf
+
 template <typename T, int K>
 struct Occ {
     static int tile[2][2][4], force, diag;  // [diffusion][back end][mode]
@@ -34,10 +42,12 @@ template <typename T, int K, int BK>
 static cudaError_t setup_modes()
 {
     cudaError_t e;
-    if ((e = setup_tile<T, K, TM_PROJECT, BK>()) != cudaSuccess) return e;
-    if ((e = setup_tile<T, K, TM_RHS, BK>()) != cudaSuccess) return e;
-    if ((e = setup_tile<T, K, TM_STAGE, BK>()) != cudaSuccess) return e;
-    if ((e = setup_tile<T, K, TM_STAGE_VABS, BK>()) != cudaSuccess) return e;
+    if constexpr (BK == BK_X3) {
+        if ((e = setup_tile<T, K, TM_PROJECT, BK>()) != cudaSuccess) return e;
+        if ((e = setup_tile<T, K, TM_RHS, BK>()) != cudaSuccess) return e;
+        if ((e = setup_tile<T, K, TM_STAGE, BK>()) != cudaSuccess) return e;
+        if ((e = setup_tile<T, K, TM_STAGE_VABS, BK>()) != cudaSuccess) return e;
+    }
     if ((e = setup_tile<T, K, TM_RHS, BK, true>()) != cudaSuccess) return e;
     if ((e = setup_tile<T, K, TM_STAGE, BK, true>()) != cudaSuccess) return e;
     return setup_tile<T, K, TM_STAGE_VABS, BK, true>();
@@ -50,6 +60,7 @@ cudaError_t setup_tiles()
 {
     cudaError_t e;
     if ((e = setup_modes<T, K, BK_FMA>()) != cudaSuccess) return e;
+    if ((e = sf::setup<T, K>()) != cudaSuccess) return e;
     if constexpr (sizeof(T) == 4) {
         if ((e = setup_modes<T, K, BK_X3>()) != cudaSuccess) return e;
     }
@@ -131,7 +142,16 @@ static cudaError_t tile_kb(const Launch& L, const TileLaunch& t)
     const size_t sm = sizeof(T) * Cf::total;
     const bool dif = L.ph.eps > 0.0 && t.mode != TM_PROJECT;
     const int g = grid_for(ntile, Occ<T, K>::tile[dif][BK][t.mode], L.nsm);
-    if (t.mode == TM_PROJECT)
+    if constexpr (BK == BK_FMA) {
+        // the CUDA-core products remain for the diffusion operator's stages
+        if (!dif) return cudaErrorInvalidValue;
+        if (t.mode == TM_RHS)
+            k_tile<T, K, TM_RHS, BK, true><<<g, Cf::NT, sm, L.st>>>(a);
+        else if (t.mode == TM_STAGE)
+            k_tile<T, K, TM_STAGE, BK, true><<<g, Cf::NT, sm, L.st>>>(a);
+        else
+            k_tile<T, K, TM_STAGE_VABS, BK, true><<<g, Cf::NT, sm, L.st>>>(a);
+    } else if (t.mode == TM_PROJECT)
         k_tile<T, K, TM_PROJECT, BK><<<g, Cf::NT, sm, L.st>>>(a);
     else if (t.mode == TM_RHS)
         dif ? k_tile<T, K, TM_RHS, BK, true><<<g, Cf::NT, sm, L.st>>>(a)
@@ -152,7 +172,8 @@ cudaError_t tile_k(const Launch& L, const TileLaunch& t)
         if (L.bk == BK_X3) return tile_kb<T, K, BK_X3>(L, t);
     }
     if (L.bk != BK_FMA) return cudaErrorInvalidValue;
-    return tile_kb<T, K, BK_FMA>(L, t);
+    if (L.ph.eps > 0.0 && t.mode != TM_PROJECT) return tile_kb<T, K, BK_FMA>(L, t);
+    return sf::launch<T, K>(L, t);
 }
 
 template <typename T, int K>

@@ -1,0 +1,5 @@
+// sum-factorised kernels, f32, degree 2
+#include "dg_sf_impl.cuh"
+namespace dg {
+DG_SF_INSTANTIATE(float, 2)
+}
