@@ -16,8 +16,8 @@
 //
 // Layout of the work: a block takes 32 consecutive cells, lane = cell, so that
 // everything a warp branches on is uniform and shared-memory accesses of
-// consecutive lanes never conflict (state rows are padded by 16 bytes: 8 lanes of
-// a 16-byte load then fall on 8 distinct groups of banks).  In k_sf_vol warp c
+// consecutive lanes never conflict (rows are padded to an odd number of 16-byte
+// units: 8 lanes of a 16-byte load then fall on 8 distinct groups of banks).  In k_sf_vol warp c
 // owns the plane c of Gauss points along z (K+1 warps): it contracts the modes
 // along z with its plane's basis values, then walks the rows of points, whose
 // fields, fluxes and partial sums along x and y stay in registers; the sums along
@@ -173,35 +173,57 @@ __device__ __forceinline__ void line_proj(const T* f, T* t)
     });
 }
 
-// contraction of the pairs (i, j) of a 2D expansion over j at point B: r[i], i = 0..M
-// (DER: with the derivative along j; r[i], i = 0..M-1)
-template <typename T, int K, int M, int B, bool DER>
-__device__ __forceinline__ void row_eval(const T* A, T* r)
+// The rows of points of a plane or face run as a rolled loop (unrolled, the
+// instructions of a tile pass outgrow the instruction cache): the row's basis
+// values come from the kernel arguments.
+// contraction of the pairs (i, j) of a 2D expansion over j with the row's values
+// c[j] (c[0] = 1): r[i], i = 0..M
+template <typename T, int M>
+__device__ __forceinline__ void row_eval(const T* A, const T* c, T* r)
 {
-    constexpr G1<K> G{};
-    constexpr int j0 = DER ? 1 : 0;
-    static_for<0, M + 1 - j0>([&](auto I) {
+    static_for<0, M + 1>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        T acc = T(0);
-        static_for<j0, M - i + 1>([&](auto J) {
-            constexpr int j = decltype(J)::value;
-            DG_SF_MAC(T, acc, DER ? G.D[j][B] : G.P[j][B], A[ip(M, i, j)], j == j0);
-        });
+        T acc = A[ip(M, i, 0)];
+        static_for<1, M - i + 1>([&](auto J) { acc += c[decltype(J)::value] * A[ip(M, i, decltype(J)::value)]; });
         r[i] = acc;
     });
 }
-// acc(i, j) (+)= (w_B/2) Pn_j(x_B) t[i], i + j <= M; the first row assigns
-template <typename T, int K, int M, int B>
-__device__ __forceinline__ void row_acc(const T* t, T* acc)
+// the same with the row's derivatives d[j] along j: r[i], i = 0..M-1
+template <typename T, int M>
+__device__ __forceinline__ void row_deriv(const T* A, const T* d, T* r)
 {
-    constexpr G1<K> G{};
+    static_for<0, M>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        T acc = d[1] * A[ip(M, i, 1)];
+        static_for<2, M - i + 1>([&](auto J) { acc += d[decltype(J)::value] * A[ip(M, i, decltype(J)::value)]; });
+        r[i] = acc;
+    });
+}
+// acc(i, j) += w[j] t[i], i + j <= M, w[j] = (w_B/2) Pn_j(x_B)
+template <typename T, int M>
+__device__ __forceinline__ void row_acc(const T* t, const T* w, T* acc)
+{
     static_for<0, M + 1>([&](auto I) {
         constexpr int i = decltype(I)::value;
-        static_for<0, M - i + 1>([&](auto J) {
-            constexpr int j = decltype(J)::value;
-            DG_SF_MAC(T, acc[ip(M, i, j)], 0.5 * G.w[B] * G.P[j][B], t[i], B == 0);
-        });
+        static_for<0, M - i + 1>(
+            [&](auto J) { acc[ip(M, i, decltype(J)::value)] += w[decltype(J)::value] * t[i]; });
     });
+}
+// the 1D tables by row: values, derivatives, weighted values
+template <typename T>
+struct Rows {
+    T P[4][4], D[4][4], W[4][4];
+};
+template <typename T, int K>
+inline void fill_rows(Rows<T>& r)
+{
+    constexpr G1<K> G{};
+    for (int a = 0; a <= K; ++a)
+        for (int m = 0; m <= K; ++m) {
+            r.P[a][m] = T(G.P[m][a]);
+            r.D[a][m] = T(G.D[m][a]);
+            r.W[a][m] = T(0.5 * G.w[a] * G.P[m][a]);
+        }
 }
 
 // contraction of the modes (i, j, l) over l with the plane's values pz[l]
@@ -338,6 +360,17 @@ __device__ __forceinline__ void cp_async_wait()
 
 constexpr int TCELL = 32;  // cells per block
 
+// row length in elements, padded to an odd number of 16-byte units (rows of
+// 8-byte vectors: to a multiple of 8 bytes that is no multiple of 16)
+template <typename T>
+constexpr int padded(int len)
+{
+    int bytes = len * (int)sizeof(T);
+    if (bytes % 16 == 8) return len;
+    while ((bytes / 16) % 2 == 0) bytes += 16;
+    return bytes / (int)sizeof(T);
+}
+
 // cell of a tile's lane: cells past the end repeat the last one (finite values,
 // not stored)
 __device__ __forceinline__ long clamp_cell(long c, long ncell) { return c < ncell ? c : ncell - 1; }
@@ -415,6 +448,7 @@ struct Args {
     int stage;         // 1: the step's dt, 0: dt_pimax
     int dtf;           // record the CFL bound
     int abar_in, abar_out;
+    Rows<T> rows;
     T two_h, inv_h, cs, cs2, eps, a2, b1;
     T rk_a, rk_b;
     double cs_d, hp, dt_pimax;
@@ -424,11 +458,11 @@ struct Args {
 // shared-memory layout of the volume kernel in elements of T
 template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
 struct VolCfg {
-    static constexpr int b = Dims<K>::b, n = K + 1, NT = 32 * n, PAD = 16 / (int)sizeof(T);
+    static constexpr int b = Dims<K>::b, n = K + 1, NT = 32 * n;
     static constexpr int NP = npair(K), NPD = npair(K - 1);
     static constexpr int NC = VOL ? 6 : 0, NV = PROJ ? (VABS ? 4 : 3) : 0;
-    static constexpr int LDU = 4 * b + PAD, LDA = 3 * b + PAD;
-    static constexpr int LDH = b + (b * (int)sizeof(T) % 32 == 0 ? PAD : 0);  // projected rows, per component
+    static constexpr int LDU = padded<T>(4 * b), LDA = padded<T>(3 * b);
+    static constexpr int LDH = padded<T>(b);  // projected rows, per component
     static constexpr int NX0 = NC * NPD + NV * NP;
     static constexpr int NX = (VOL && FORCE && 3 * NP > NX0) ? 3 * NP : NX0;  // exchanged entries
     static constexpr int oU = 0;                                // [2][32][LDU]
@@ -436,6 +470,10 @@ struct VolCfg {
     static constexpr int oR = oAh + (FORCE ? TCELL * LDA : 0);  // [32][LDU] result rows
     static constexpr int oX = oR + (VOL ? TCELL * LDU : 0);     // [NX][n][32]
     static constexpr int total = oX + NX * n * 32;
+    // the momentum components (and the projected velocity's) v = v0, v0 + n.. of warp w;
+    // at degree 3 warp 0 takes the density and |v| instead
+    __device__ static constexpr int v0(int w) { return K == 3 ? (w == 0 ? 4 : w) : w + 1; }
+    static constexpr int W_RHO = K == 1 ? 1 : 0, W_ABS = K == 3 ? 0 : 1;
     static_assert(NV == 0 || NP * n * 32 >= TCELL * LDH, "a projected row fits its entries");
     static_assert(total * (int)sizeof(T) >= NT * 8, "reduction buffer");
 };
@@ -452,8 +490,8 @@ struct VolCfg {
 // Bound: FP32 instruction issue (about 8.8 thousand instructions per cell at
 // degree 3 with PROJ, 880 bytes of HBM traffic); FP64 by the FP64 pipe.
 template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
-__global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K == 2 ? 4 : 8) : 1)
-    k_sf_vol(const Args<T> a)
+__global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL ? 3 : 4) : K == 2 ? 4 : 8) : 1)
+    k_sf_vol(const __grid_constant__ Args<T> a)
 {
     using C = VolCfg<T, K, VOL, FORCE, PROJ, VABS>;
     constexpr int b = C::b, n = C::n, NT = C::NT, NP = C::NP, NPD = C::NPD, LDU = C::LDU, LDA = C::LDA;
@@ -562,9 +600,11 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
             // per-cell forcing sums <rho a_h> = sum_l rho_l a_l (orthonormal basis), <rho>
             if constexpr (PROJ) {
                 auto dot = [&](int i) {
-                    T s = T(0);
+                    T s = T(0), x[b], y[b];
+                    ld_row<T, b>(sU, x);
+                    ld_row<T, b>(ah + i * b, y);
 #pragma unroll
-                    for (int l = 0; l < b; ++l) s += sU[l] * ah[i * b + l];
+                    for (int l = 0; l < b; ++l) s += x[l] * y[l];
                     return (double)s;
                 };
                 if (valid) {
@@ -581,43 +621,58 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
                     ld_row<T, b>(ah + f * b, uu);
                     plane_eval<T, K>(uu, pz, Aa[f]);
                 });
-                static_for<0, n>([&](auto B_) {
-                    constexpr int B = decltype(B_)::value;
+#pragma unroll
+                for (int f = 0; f < 3; ++f)
+#pragma unroll
+                    for (int e = 0; e < NP; ++e) S[f][e] = T(0);
+#pragma unroll 1
+                for (int B = 0; B < n; ++B) {
+                    const T *pj = a.rows.P[B], *wj = a.rows.W[B];
                     T r[n], rho[n];
-                    row_eval<T, K, K, B, false>(A[0], r);
+                    row_eval<T, K>(A[0], pj, r);
                     line_eval<T, K, K, false>(r, rho);
                     static_for<0, 3>([&](auto F) {
                         constexpr int f = decltype(F)::value;
                         T q[n], v[n], t[n];
-                        row_eval<T, K, K, B, false>(Aa[f], q);
+                        row_eval<T, K>(Aa[f], pj, q);
                         line_eval<T, K, K, false>(q, v);
 #pragma unroll
                         for (int i = 0; i < n; ++i) v[i] *= rho[i];
                         line_proj<T, K, K>(v, t);
-                        row_acc<T, K, K, B>(t, S[f]);
+                        row_acc<T, K>(t, wj, S[f]);
                     });
-                });
+                }
                 static_for<0, 3>([&](auto F) {
                     constexpr int f = decltype(F)::value;
 #pragma unroll
                     for (int e = 0; e < NP; ++e) sX[((f * NP + e) * n + w) * 32 + lane] = S[f][e];
                 });
                 __syncthreads();
-                // warp of the momentum component (the same thread adds the flux part below)
-                static_for<0, 3>([&](auto F) {
-                    constexpr int f = decltype(F)::value;
-                    if (w == (f + 1) % n) {
-                        T q[b];
-                        z_project<T, K, K>(sX + f * NP * n * 32, lane, q);
-                        st_row<T, b>(sR + lane * LDU + (1 + f) * b, q);
-                    }
-                });
+                // the thread of the momentum component adds the flux part to these rows below
+#pragma unroll 1
+                for (int v = C::v0(w); v < 4; v += n) {
+                    T q[b];
+                    z_project<T, K, K>(sX + (v - 1) * NP * n * 32, lane, q);
+                    st_row<T, b>(sR + lane * LDU + v * b, q);
+                }
                 __syncthreads();
             }
         }
         // ---- main pass: the plane's rows of points ----
         T Fx[VOL ? 6 : 1][VOL ? NPD : 1];  // sums of xx, yy, zz, xy, xz, yz (degree <= K-1)
         T Vx[PROJ ? C::NV : 1][PROJ ? NP : 1];  // sums of v (and |v|)
+        if constexpr (VOL) {
+#pragma unroll
+            for (int f = 0; f < 6; ++f)
+#pragma unroll
+                for (int e = 0; e < NPD; ++e) Fx[f][e] = T(0);
+        }
+        if constexpr (PROJ) {
+#pragma unroll
+            for (int f = 0; f < C::NV; ++f)
+#pragma unroll
+                for (int e = 0; e < NP; ++e) Vx[f][e] = T(0);
+        }
         auto rows = [&](auto DIV_) {
             constexpr bool DIV = decltype(DIV_)::value;
             T Az[DIV ? NPD : 1], Mz[DIV ? NPD : 1];  // d rho/dz, d m_z/dz
@@ -628,26 +683,27 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
                 ld_row<T, b>(sU + 3 * b, uu);
                 plane_deriv<T, K>(uu, dz, Mz);
             }
-            static_for<0, n>([&](auto B_) {
-                constexpr int B = decltype(B_)::value;
+#pragma unroll 1
+            for (int B = 0; B < n; ++B) {
+                const T *pj = a.rows.P[B], *dj = a.rows.D[B], *wj = a.rows.W[B];
                 T f[4][n];
                 T gx[n], gy[n], gz[n], dm[n];
                 static_for<0, 4>([&](auto F) {
                     constexpr int v = decltype(F)::value;
                     T r[n];
-                    row_eval<T, K, K, B, false>(A[v], r);
+                    row_eval<T, K>(A[v], pj, r);
                     line_eval<T, K, K, false>(r, f[v]);
                     if constexpr (DIV && v == 0) line_eval<T, K, K, true>(r, gx);
                     if constexpr (DIV && v == 1) line_eval<T, K, K, true>(r, dm);
                 });
                 if constexpr (DIV) {
                     T r[n], s[n], t[n];
-                    row_eval<T, K, K, B, true>(A[0], r);
+                    row_deriv<T, K>(A[0], dj, r);
                     line_eval<T, K, K - 1, false>(r, gy);
-                    row_eval<T, K, K - 1, B, false>(Az, r);
+                    row_eval<T, K - 1>(Az, pj, r);
                     line_eval<T, K, K - 1, false>(r, gz);
-                    row_eval<T, K, K, B, true>(A[2], r);
-                    row_eval<T, K, K - 1, B, false>(Mz, s);
+                    row_deriv<T, K>(A[2], dj, r);
+                    row_eval<T, K - 1>(Mz, pj, s);
 #pragma unroll
                     for (int i = 0; i < K; ++i) r[i] += s[i];
                     line_eval<T, K, K - 1, false>(r, t);
@@ -694,7 +750,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
 #pragma unroll
                         for (int i = 0; i < n; ++i) x[i] = diag ? p[i] * q[i] + P[i] : p[i] * q[i];
                         line_proj<T, K, K - 1>(x, t);
-                        row_acc<T, K, K - 1, B>(t, Fx[g]);
+                        row_acc<T, K - 1>(t, wj, Fx[g]);
                     };
                     comp(std::integral_constant<int, 0>{}, f[1], vx, true);
                     comp(std::integral_constant<int, 1>{}, f[2], vy, true);
@@ -710,16 +766,16 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
 #pragma unroll
                         for (int i = 0; i < n; ++i) x[i] = sqrt(vx[i] * vx[i] + vy[i] * vy[i] + vz[i] * vz[i]);
                         line_proj<T, K, K>(x, t);
-                        row_acc<T, K, K, B>(t, Vx[C::NV - 1]);
+                        row_acc<T, K>(t, wj, Vx[C::NV - 1]);
                     }
                     line_proj<T, K, K>(vx, t);
-                    row_acc<T, K, K, B>(t, Vx[0]);
+                    row_acc<T, K>(t, wj, Vx[0]);
                     line_proj<T, K, K>(vy, t);
-                    row_acc<T, K, K, B>(t, Vx[1]);
+                    row_acc<T, K>(t, wj, Vx[1]);
                     line_proj<T, K, K>(vz, t);
-                    row_acc<T, K, K, B>(t, Vx[2]);
+                    row_acc<T, K>(t, wj, Vx[2]);
                 }
-            });
+            }
         };
         if (VOL && need_div)
             rows(std::integral_constant<bool, VOL>{});
@@ -741,58 +797,58 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
             });
         }
         __syncthreads();
-        // ---- volume term (2/h) sum_d D_d^T Fhat_d of variable v (warp v mod n), and
-        // the projected components ----
+        // ---- volume term (2/h) sum_d D_d^T Fhat_d of a variable, and the projected
+        // components ----
         if constexpr (VOL) {
-            static_for<0, 4>([&](auto V_) {
-                constexpr int v = decltype(V_)::value;
-                if (w == v % n) {
-                    T r[b];
-                    if constexpr (v == 0) {
-                        T q[b];
+            if (w == C::W_RHO) {
+                T r[b], q[b];
 #pragma unroll
-                        for (int l = 0; l < b; ++l) r[l] = T(0);
-                        ld_row<T, b>(sU + b, q);
-                        modal_grad_T_acc<T, K, 0>(q, r, a.two_h);
-                        ld_row<T, b>(sU + 2 * b, q);
-                        modal_grad_T_acc<T, K, 1>(q, r, a.two_h);
-                        ld_row<T, b>(sU + 3 * b, q);
-                        modal_grad_T_acc<T, K, 2>(q, r, a.two_h);
-                    } else {
-                        constexpr int i = v - 1;
-                        constexpr int cx = i == 0 ? 0 : (i == 1 ? 3 : 4);
-                        constexpr int cy = i == 0 ? 3 : (i == 1 ? 1 : 5);
-                        constexpr int cz = i == 0 ? 4 : (i == 1 ? 5 : 2);
-                        T q[b];
-                        if constexpr (FORCE) {
-                            ld_row<T, b>(sR + lane * LDU + v * b, r);
-                        } else {
-#pragma unroll
-                            for (int l = 0; l < b; ++l) r[l] = T(0);
-                        }
-                        z_project<T, K, K - 1>(sX + cx * NPD * n * 32, lane, q);
-                        modal_grad_T_acc<T, K, 0>(q, r, a.two_h);
-                        z_project<T, K, K - 1>(sX + cy * NPD * n * 32, lane, q);
-                        modal_grad_T_acc<T, K, 1>(q, r, a.two_h);
-                        z_project<T, K, K - 1>(sX + cz * NPD * n * 32, lane, q);
-                        modal_grad_T_acc<T, K, 2>(q, r, a.two_h);
-                    }
-                    st_row<T, b>(sR + lane * LDU + v * b, r);
-                }
-            });
+                for (int l = 0; l < b; ++l) r[l] = T(0);
+                ld_row<T, b>(sU + b, q);
+                modal_grad_T_acc<T, K, 0>(q, r, a.two_h);
+                ld_row<T, b>(sU + 2 * b, q);
+                modal_grad_T_acc<T, K, 1>(q, r, a.two_h);
+                ld_row<T, b>(sU + 3 * b, q);
+                modal_grad_T_acc<T, K, 2>(q, r, a.two_h);
+                st_row<T, b>(sR + lane * LDU, r);
+            }
         }
-        if constexpr (PROJ) {
-            // the rows replace the component's entries, which only this warp reads
-            static_for<0, C::NV>([&](auto V_) {
-                constexpr int v = decltype(V_)::value;
-                if (w == (v + 1) % n) {
-                    T q[b];
-                    T* X = sX + (C::NC * NPD + v * NP) * n * 32;
-                    z_project<T, K, K>(X, lane, q);
-                    __syncwarp();
-                    st_row<T, b>(X + lane * C::LDH, q);
+#pragma unroll 1
+        for (int v = C::v0(w); v < 4; v += n) {
+            T q[b];
+            if constexpr (VOL) {
+                T r[b];
+                const int cx = v == 1 ? 0 : v + 1, cy = v == 1 ? 3 : (v == 2 ? 1 : 5), cz = v == 3 ? 2 : v + 3;
+                if constexpr (FORCE) {
+                    ld_row<T, b>(sR + lane * LDU + v * b, r);
+                } else {
+#pragma unroll
+                    for (int l = 0; l < b; ++l) r[l] = T(0);
                 }
-            });
+                z_project<T, K, K - 1>(sX + cx * NPD * n * 32, lane, q);
+                modal_grad_T_acc<T, K, 0>(q, r, a.two_h);
+                z_project<T, K, K - 1>(sX + cy * NPD * n * 32, lane, q);
+                modal_grad_T_acc<T, K, 1>(q, r, a.two_h);
+                z_project<T, K, K - 1>(sX + cz * NPD * n * 32, lane, q);
+                modal_grad_T_acc<T, K, 2>(q, r, a.two_h);
+                st_row<T, b>(sR + lane * LDU + v * b, r);
+            }
+            if constexpr (PROJ) {
+                // the rows replace the component's entries, which only this warp reads
+                T* X = sX + (C::NC * NPD + (v - 1) * NP) * n * 32;
+                z_project<T, K, K>(X, lane, q);
+                __syncwarp();
+                st_row<T, b>(X + lane * C::LDH, q);
+            }
+        }
+        if constexpr (VABS) {
+            if (w == C::W_ABS) {
+                T q[b];
+                T* X = sX + (C::NC * NPD + 3 * NP) * n * 32;
+                z_project<T, K, K>(X, lane, q);
+                __syncwarp();
+                st_row<T, b>(X + lane * C::LDH, q);
+            }
         }
         __syncthreads();
         // ---- coalesced stores ----
@@ -879,16 +935,22 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
 // ---------------------------------------------------------------------------
 // face kernel
 // ---------------------------------------------------------------------------
+// A block takes a brick of 4 x 4 x 2 cells (lane = cell, x fastest) with 4 warps:
+// warps 0-2 own the + faces of the 32 cells along x, y, z, warp 3 the 8 + 8 + 16
+// - faces of the brick's lower sides: 128 faces where 32 cells taken one by one
+// have 192, and 96 operand rows where those would read 224.  Bricks past the end of
+// the mesh hold the periodic images of its cells, which are the neighbours the
+// last cells need.
 template <typename T, int K>
 struct FaceCfg {
-    static constexpr int b = Dims<K>::b, NP = npair(K), NT = 192, PAD = 16 / (int)sizeof(T);
-    static constexpr int LD = 4 * b + PAD;      // rows rho, v (operands) and rho, m (states)
+    static constexpr int b = Dims<K>::b, NP = npair(K), NT = 128;
+    static constexpr int LD = padded<T>(4 * b);  // rows rho, v (operands) and rho, m (states)
     static constexpr int REG = TCELL * LD;
-    // regions 0-5: the neighbours across the faces, 6: the cells themselves; later 0:
-    // u^(s) (then the new state), 1: rvol, 2: u^n, 3-6: the lifted fluxes
-    static constexpr int oFlux = 3 * REG;
-    static constexpr int total = 7 * REG;
-    static_assert(6 * 4 * NP * 32 <= 4 * REG, "fluxes fit the free regions");
+    // rows 0-31: the brick's cells; 32-63: those across its -x, +x, -y, +y sides (8
+    // each); 64-95: across -z, +z (16 each).  Later 0-31: u^(s) (then the new state),
+    // 32-63: rvol, 64-95: u^n
+    static constexpr int oFlux = 3 * REG;  // [variable][pair][face]
+    static constexpr int total = oFlux + 4 * NP * 128;
 };
 
 // 2D coefficients of a field's trace on the + (SIDE 1) or - face along Dd
@@ -910,10 +972,10 @@ __device__ __forceinline__ void trace(const T* c, T* c2)
     });
 }
 
-// Bound: FP32 instruction issue (about 10 thousand instructions per cell at
-// degree 3); every face is computed by both its cells.
+// Bound: FP32 instruction issue (about 8 thousand instructions per cell at degree 3).
 template <typename T, int K, int RS, bool STAGE>
-__global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3 : 2) : 1) k_sf_faces(const Args<T> a)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? 4 : 3) : 1)
+    k_sf_faces(const __grid_constant__ Args<T> a)
 {
     using C = FaceCfg<T, K>;
     constexpr int b = C::b, n = K + 1, NP = C::NP, NT = C::NT, LD = C::LD, nq = n * n * n, nf = 6 * n * n;
@@ -921,15 +983,29 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
     T* sm = reinterpret_cast<T*>(smem_raw);
     __shared__ T s_th[TCELL];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const long c0 = (long)blockIdx.x * TCELL;
-    const int nvalid = (int)((a.ncell - c0) < TCELL ? (a.ncell - c0) : TCELL);
-    const int d = w >> 1, side = w & 1;
-    T* const self = sm + 6 * C::REG;
-    // ---- operand rows (rho, v): the neighbour across face w of every cell, and
-    // the cells themselves, by asynchronous copies of four lanes per cell ----
+    const int N = a.N, nbx = (N + 3) >> 2;
+    int x0, y0, z0;
+    {
+        const unsigned q = blockIdx.x / (unsigned)nbx;
+        x0 = 4 * (int)(blockIdx.x - q * nbx);
+        y0 = 4 * (int)(q % (unsigned)nbx);
+        z0 = 2 * (int)(q / (unsigned)nbx);
+    }
+    // cell of brick coordinates (-1..4, -1..4, -1..2), periodic
+    auto cell_of = [&](int i, int j, int k) -> long {
+        int x = x0 + i, y = y0 + j, z = z0 + k;
+        x = x < 0 ? N - 1 : (x < N ? x : x % N);
+        y = y < 0 ? N - 1 : (y < N ? y : y % N);
+        z = z < 0 ? N - 1 : (z < N ? z : z % N);
+        return ((long)z * N + y) * N + x;
+    };
+    // ---- operand rows (rho, v), four lanes per row ----
+    const int rs = tid >> 2, sub = tid & 3;  // row within a group of 32, lane of it
+    const int ri = rs & 3, rj = (rs >> 2) & 3, rk = rs >> 4;
+    const long rcell = cell_of(ri, rj, rk);
+    const bool rvalid = x0 + ri < N && y0 + rj < N && z0 + rk < N;
     {
         constexpr int CH = chunk<T, b>(), V = CH / (int)sizeof(T), NB = b / V;  // chunks of rho; 3 NB of v
-        const int sub = lane & 3;
         auto copy_row = [&](T* dst, long c) {
             const T* ru = a.u_in + c * 4 * b;
             const T* rv = a.vh_in + c * 3 * b - b;  // chunk ch >= NB: v
@@ -939,19 +1015,33 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
                 cp_async<CH>(dst + ch * V, (ch < NB ? ru : rv) + ch * V);
             }
         };
-        const long c = clamp_cell(c0 + lane, a.ncell);
-        int xyz[3];
-        cell_xyz(c, a.N, xyz[0], xyz[1], xyz[2]);
-        const int co = d == 0 ? xyz[0] : (d == 1 ? xyz[1] : xyz[2]);
-        const int stp = d == 0 ? 1 : (d == 1 ? a.N : a.N * a.N);
-        const int nb = (int)c + (side ? (co == a.N - 1 ? -(a.N - 1) * stp : stp) : (co == 0 ? (a.N - 1) * stp : -stp));
-#pragma unroll
-        for (int g = 0; g < 4; ++g) {
-            const int cl = 8 * g + (lane >> 2);
-            copy_row(sm + w * C::REG + cl * LD, (long)__shfl_sync(0xffffffffu, nb, cl));
-        }
-        if (w < 4) copy_row(self + (8 * w + (lane >> 2)) * LD, clamp_cell(c0 + 8 * w + (lane >> 2), a.ncell));
+        copy_row(sm + rs * LD, rcell);
+        // -x, +x: (j, k) = (rs & 3, (rs >> 2) & 1); -y, +y: (i, k) the same
+        const int hs = rs >> 3, h0 = rs & 3, h1 = (rs >> 2) & 1;
+        copy_row(sm + (32 + rs) * LD, hs < 2 ? cell_of(hs ? 4 : -1, h0, h1) : cell_of(h0, hs == 3 ? 4 : -1, h1));
+        copy_row(sm + (64 + rs) * LD, cell_of(ri, rj, rk ? 2 : -1));
         cp_async_commit();
+    }
+    // the thread's face: direction, rows of its lower (L) and upper (R) cell
+    int d, rowL, rowR;
+    {
+        const int i = lane & 3, j = (lane >> 2) & 3, k = lane >> 4;
+        if (w < 3) {
+            d = w;
+            rowL = lane;
+            rowR = w == 0 ? (i < 3 ? lane + 1 : 40 + 4 * k + j)
+                          : (w == 1 ? (j < 3 ? lane + 4 : 56 + 4 * k + i) : (k < 1 ? lane + 16 : 80 + 4 * j + i));
+        } else if (lane < 16) {
+            // lanes 0-7: -x faces of (j, k); 8-15: -y faces of (i, k)
+            d = lane >> 3;
+            const int e0 = lane & 3, e1 = (lane >> 2) & 1;
+            rowL = 32 + 16 * d + (lane & 7);
+            rowR = d == 0 ? 16 * e1 + 4 * e0 : 16 * e1 + e0;
+        } else {
+            d = 2;
+            rowL = 64 + lane - 16;
+            rowR = lane - 16;
+        }
     }
     const T dt = STAGE ? T(a.ctl->dt) : T(0);
     const bool fix = a.ahat != nullptr;
@@ -961,10 +1051,8 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
     // rho, v_n, v_t1, v_t2 ----
     T c2[8][NP];
     {
-        const T* own = self + lane * LD;
-        const T* nbr = sm + w * C::REG + lane * LD;
-        const T* Lp = side ? own : nbr;
-        const T* Rp = side ? nbr : own;
+        const T* Lp = sm + rowL * LD;
+        const T* Rp = sm + rowR * LD;
         auto traces = [&](auto D_) {
             constexpr int Dd = decltype(D_)::value;
             constexpr int t1 = Dd == 0 ? 1 : 0, t2 = Dd == 2 ? 1 : 2;
@@ -986,26 +1074,42 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
             traces(std::integral_constant<int, 2>{});
     }
     __syncthreads();
-    // the operand regions are free: the epilogue's inputs arrive during the fluxes
-    constexpr int CHU = chunk<T, 4 * b>();
-    tile_async<T, 4 * b, LD, NT, CHU>(sm, a.u_in, c0, a.ncell);
-    if ((reinterpret_cast<uintptr_t>(a.out) & (CHU - 1)) == 0) {
-        tile_async<T, 4 * b, LD, NT, CHU>(sm + C::REG, a.out, c0, a.ncell);
-    } else {
-        for (int e = tid; e < nvalid * 4 * b; e += NT) sm[C::REG + (e / (4 * b)) * LD + e % (4 * b)] = a.out[c0 * 4 * b + e];
+    // the operand rows are free: the epilogue's inputs arrive during the fluxes
+    constexpr int CHU = chunk<T, 4 * b>(), VU = CHU / (int)sizeof(T), NCU = 4 * b / VU;
+    static_assert(CHU == 16, "state rows in 16-byte chunks");
+    const bool out16 = (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0;
+    {
+        auto copy_state = [&](T* dst, const T* src) {
+            const T* s = src + rcell * 4 * b;
+            T* q = dst + rs * LD;
+#pragma unroll
+            for (int k = 0; k < (NCU + 3) / 4; ++k)
+                if (NCU % 4 == 0 || sub + 4 * k < NCU) cp_async<16>(q + (sub + 4 * k) * VU, s + (sub + 4 * k) * VU);
+        };
+        copy_state(sm, a.u_in);
+        if (out16) {
+            copy_state(sm + C::REG, a.out);
+        } else {
+            for (int e = sub; e < 4 * b; e += 4) sm[C::REG + rs * LD + e] = a.out[rcell * 4 * b + e];
+        }
+        if (STAGE && a.rk_a != T(0)) copy_state(sm + 2 * C::REG, a.u_n);
+        cp_async_commit();
     }
-    if (STAGE && a.rk_a != T(0)) tile_async<T, 4 * b, LD, NT, CHU>(sm + 2 * C::REG, a.u_n, c0, a.ncell);
-    cp_async_commit();
     // ---- Riemann fluxes at the face points, lifted row by row ----
     {
         T fx[4][NP];
-        static_for<0, n>([&](auto B_) {
-            constexpr int B = decltype(B_)::value;
+#pragma unroll
+        for (int f = 0; f < 4; ++f)
+#pragma unroll
+            for (int e = 0; e < NP; ++e) fx[f][e] = T(0);
+#pragma unroll 1
+        for (int B = 0; B < n; ++B) {
+            const T *pj = a.rows.P[B], *wj = a.rows.W[B];
             T W[8][n];
             static_for<0, 8>([&](auto F) {
                 constexpr int f = decltype(F)::value;
                 T r[n];
-                row_eval<T, K, K, B, false>(c2[f], r);
+                row_eval<T, K>(c2[f], pj, r);
                 line_eval<T, K, K, false>(r, W[f]);
             });
             T Fl[4][n];
@@ -1022,48 +1126,51 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
                 constexpr int f = decltype(F)::value;
                 T t[n];
                 line_proj<T, K, K>(Fl[f], t);
-                row_acc<T, K, K, B>(t, fx[f]);
+                row_acc<T, K>(t, wj, fx[f]);
             });
-        });
-        // entries [face][variable][pair][lane]
+        }
         const int v1 = 1 + d, v2 = d == 0 ? 2 : 1, v3 = d == 2 ? 2 : 3;
-        T* X = sm + C::oFlux + w * 4 * NP * 32 + lane;
+        T* X = sm + C::oFlux + tid;
 #pragma unroll
         for (int e = 0; e < NP; ++e) {
-            X[e * 32] = fx[0][e];
-            X[(v1 * NP + e) * 32] = fx[1][e];
-            X[(v2 * NP + e) * 32] = fx[2][e];
-            X[(v3 * NP + e) * 32] = fx[3][e];
+            X[e * 128] = fx[0][e];
+            X[(v1 * NP + e) * 128] = fx[1][e];
+            X[(v2 * NP + e) * 128] = fx[2][e];
+            X[(v3 * NP + e) * 128] = fx[3][e];
         }
     }
     cp_async_wait<0>();
     __syncthreads();
-    // ---- right-hand side of variable w (warps 0-3): surface term + rvol ----
+    // ---- right-hand side of variable w: surface term + rvol ----
     T r[b];
     unsigned int st = 0u;
-    const long cc = c0 + lane;
+    const int ci = lane & 3, cj = (lane >> 2) & 3, ck = lane >> 4;
+    const bool valid = x0 + ci < N && y0 + cj < N && z0 + ck < N;
     T* const row = sm + lane * LD + w * b;  // u^(s), later the result
-    if (w < 4) {
 #pragma unroll
-        for (int l = 0; l < b; ++l) r[l] = T(0);
-        static_for<0, 3>([&](auto D_) {
-            constexpr int Dd = decltype(D_)::value;
-            const T* Xm = sm + C::oFlux + ((2 * Dd) * 4 + w) * NP * 32 + lane;
-            const T* Xp = Xm + 4 * NP * 32;
-            static_for<0, K + 1>([&](auto I) {
-                constexpr int p = decltype(I)::value;
-                static_for<0, K - p + 1>([&](auto J) {
-                    constexpr int q = decltype(J)::value;
-                    const T xm = Xm[ip(K, p, q) * 32], xp = Xp[ip(K, p, q) * 32];
-                    const T ev = xm - xp, od = -(xm + xp);
-                    static_for<0, K - p - q + 1>([&](auto L) {
-                        constexpr int dn = decltype(L)::value;
-                        constexpr int m = Dd == 0 ? im<K>(dn, p, q) : (Dd == 1 ? im<K>(p, dn, q) : im<K>(p, q, dn));
-                        DG_SF_MAC(T, r[m], csqrt(2.0 * dn + 1.0), ((dn & 1) ? od : ev), false);
-                    });
+    for (int l = 0; l < b; ++l) r[l] = T(0);
+    static_for<0, 3>([&](auto D_) {
+        constexpr int Dd = decltype(D_)::value;
+        const T* X = sm + C::oFlux + w * NP * 128;
+        const T* Xp = X + 32 * Dd + lane;
+        const T* Xm = X + (Dd == 0 ? (ci > 0 ? lane - 1 : 96 + 4 * ck + cj)
+                                   : (Dd == 1 ? (cj > 0 ? 32 + lane - 4 : 104 + 4 * ck + ci)
+                                              : (ck > 0 ? 64 + lane - 16 : 112 + 4 * cj + ci)));
+        static_for<0, K + 1>([&](auto I) {
+            constexpr int p = decltype(I)::value;
+            static_for<0, K - p + 1>([&](auto J) {
+                constexpr int q = decltype(J)::value;
+                const T xm = Xm[ip(K, p, q) * 128], xp = Xp[ip(K, p, q) * 128];
+                const T ev = xm - xp, od = -(xm + xp);
+                static_for<0, K - p - q + 1>([&](auto L) {
+                    constexpr int dn = decltype(L)::value;
+                    constexpr int m = Dd == 0 ? im<K>(dn, p, q) : (Dd == 1 ? im<K>(p, dn, q) : im<K>(p, q, dn));
+                    DG_SF_MAC(T, r[m], csqrt(2.0 * dn + 1.0), ((dn & 1) ? od : ev), false);
                 });
             });
         });
+    });
+    {
         T x[b];
         ld_row<T, b>(row + C::REG, x);  // rvol
 #pragma unroll
@@ -1076,21 +1183,19 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
             for (int l = 0; l < b; ++l) r[l] -= ab * x[l];
         }
     }
+    // every warp has read rho before warp 0 replaces it
+    if (fix) __syncthreads();
     if constexpr (STAGE) {
-        // every warp has read rho before warp 0 replaces it
-        if (fix) __syncthreads();
-        if (w < 4) {
-            T x[b];
-            ld_row<T, b>(row, x);
-            if (a.rk_a != T(0)) {
-                T y[b];
-                ld_row<T, b>(row + 2 * C::REG, y);
+        T x[b];
+        ld_row<T, b>(row, x);
+        if (a.rk_a != T(0)) {
+            T y[b];
+            ld_row<T, b>(row + 2 * C::REG, y);
 #pragma unroll
-                for (int l = 0; l < b; ++l) r[l] = a.rk_a * y[l] + a.rk_b * (x[l] + dt * r[l]);
-            } else {
+            for (int l = 0; l < b; ++l) r[l] = a.rk_a * y[l] + a.rk_b * (x[l] + dt * r[l]);
+        } else {
 #pragma unroll
-                for (int l = 0; l < b; ++l) r[l] = a.rk_b * (x[l] + dt * r[l]);
-            }
+            for (int l = 0; l < b; ++l) r[l] = a.rk_b * (x[l] + dt * r[l]);
         }
         if (w == 0) {
             // positivity (Sec. 3.1): a cell passes when rho_0 - sum_l |rho_l| sup|phi_l| >= eps;
@@ -1102,7 +1207,7 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
                 part += T(sup_phi<K>(m)) * fabs(r[m]);
             });
             T th = T(1);
-            unsigned low = __ballot_sync(0xffffffffu, lane < nvalid && r[0] - part < a.eps);
+            unsigned low = __ballot_sync(0xffffffffu, valid && r[0] - part < a.eps);
             if (low) {
                 st_row<T, b>(row, r);
                 __syncwarp();
@@ -1126,7 +1231,7 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
                         mn = other < mn ? other : mn;
                     }
                     if (a.trouble && mn < T(0)) {
-                        if (lane == 0) a.trouble[c0 + c] |= DG_MARK_NEGATIVE;
+                        if (lane == c) a.trouble[cell_of(ci, cj, ck)] |= DG_MARK_NEGATIVE;
                         st |= DG_ST_TROUBLED_;
                     }
                     if (mn < a.eps) {
@@ -1143,24 +1248,32 @@ __global__ void __launch_bounds__(192, sizeof(T) == 4 ? (K == 1 ? 4 : K == 2 ? 3
             s_th[lane] = th;
         }
         __syncthreads();
-        if (w < 4) {
-            const T th = s_th[lane];
-            bool bad = !isfinite(r[0]);
+        const T th = s_th[lane];
+        bool bad = !isfinite(r[0]);
 #pragma unroll
-            for (int l = 1; l < b; ++l) {
-                r[l] *= th;
-                bad |= !isfinite(r[l]);
-            }
-            if (bad && cc < a.ncell) st |= DG_ST_NONFINITE_;
-            st = __reduce_or_sync(0xffffffffu, st);
-            if (lane == 0 && st) atomicOr(&a.ctl->status, st);
+        for (int l = 1; l < b; ++l) {
+            r[l] *= th;
+            bad |= !isfinite(r[l]);
         }
-    } else {
-        if (fix) __syncthreads();
+        if (bad && valid) st |= DG_ST_NONFINITE_;
+        st = __reduce_or_sync(0xffffffffu, st);
+        if (lane == 0 && st) atomicOr(&a.ctl->status, st);
     }
-    if (w < 4) st_row<T, b>(row, r);
+    st_row<T, b>(row, r);
     __syncthreads();
-    tile_store<T, 4 * b, LD, NT>(a.out, sm, c0, nvalid);
+    if (rvalid) {
+        T* g = a.out + rcell * 4 * b;
+        const T* q = sm + rs * LD;
+        if (out16) {
+#pragma unroll
+            for (int k = 0; k < (NCU + 3) / 4; ++k)
+                if (NCU % 4 == 0 || sub + 4 * k < NCU)
+                    *reinterpret_cast<uint4*>(g + (sub + 4 * k) * VU) =
+                        *reinterpret_cast<const uint4*>(q + (sub + 4 * k) * VU);
+        } else {
+            for (int e = sub; e < 4 * b; e += 4) g[e] = q[e];
+        }
+    }
 }
 
 }  // namespace sf

@@ -44,12 +44,12 @@ cudaError_t setup()
     if ((e = prepare_vol<T, K, false, false, true, true>(o + 6))) return e;
     if ((e = prepare_vol<T, K, false, true, true, true>(o + 7))) return e;
     const size_t sm = sizeof(T) * FaceCfg<T, K>::total;
-    if ((e = prepare(k_sf_faces<T, K, 0, true>, sm, 192, nullptr))) return e;
-    if ((e = prepare(k_sf_faces<T, K, 1, true>, sm, 192, nullptr))) return e;
-    if ((e = prepare(k_sf_faces<T, K, 2, true>, sm, 192, nullptr))) return e;
-    if ((e = prepare(k_sf_faces<T, K, 0, false>, sm, 192, nullptr))) return e;
-    if ((e = prepare(k_sf_faces<T, K, 1, false>, sm, 192, nullptr))) return e;
-    return prepare(k_sf_faces<T, K, 2, false>, sm, 192, nullptr);
+    if ((e = prepare(k_sf_faces<T, K, 0, true>, sm, 128, nullptr))) return e;
+    if ((e = prepare(k_sf_faces<T, K, 1, true>, sm, 128, nullptr))) return e;
+    if ((e = prepare(k_sf_faces<T, K, 2, true>, sm, 128, nullptr))) return e;
+    if ((e = prepare(k_sf_faces<T, K, 0, false>, sm, 128, nullptr))) return e;
+    if ((e = prepare(k_sf_faces<T, K, 1, false>, sm, 128, nullptr))) return e;
+    return prepare(k_sf_faces<T, K, 2, false>, sm, 128, nullptr);
 }
 
 template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
@@ -68,13 +68,13 @@ template <typename T, int K, bool STAGE>
 static cudaError_t go_faces(const Launch& L, const Args<T>& a)
 {
     const size_t sm = sizeof(T) * FaceCfg<T, K>::total;
-    const int g = (int)((L.ncell + TCELL - 1) / TCELL);
+    const int nb = (L.N + 3) / 4, g = nb * nb * ((L.N + 1) / 2);  // bricks of 4 x 4 x 2 cells
     if (L.ph.riemann == 2)
-        k_sf_faces<T, K, 2, STAGE><<<g, 192, sm, L.st>>>(a);
+        k_sf_faces<T, K, 2, STAGE><<<g, 128, sm, L.st>>>(a);
     else if (L.ph.riemann == 1)
-        k_sf_faces<T, K, 1, STAGE><<<g, 192, sm, L.st>>>(a);
+        k_sf_faces<T, K, 1, STAGE><<<g, 128, sm, L.st>>>(a);
     else
-        k_sf_faces<T, K, 0, STAGE><<<g, 192, sm, L.st>>>(a);
+        k_sf_faces<T, K, 0, STAGE><<<g, 128, sm, L.st>>>(a);
     return cudaGetLastError();
 }
 
@@ -101,6 +101,7 @@ cudaError_t launch(const Launch& L, const TileLaunch& t)
     a.N = L.N;
     a.av_mode = L.ph.av_mode;
     a.tcount = TileCfg<K, BK_FMA>::TC;
+    fill_rows<T, K>(a.rows);
     a.two_h = T(2.0 / L.ph.h);
     a.inv_h = T(1.0 / L.ph.h);
     a.cs = T(L.ph.cs);
