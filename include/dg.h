@@ -47,9 +47,11 @@ extern "C" {
 /* ---- precision modes ----------------------------------------------------- */
 #define DG_PREC_F64 0      /* everything in FP64 (parity mode)                   */
 #define DG_PREC_F32 1      /* FP32 state and arithmetic; FP64 global sums        */
-#define DG_PREC_X3 2       /* FP32 state; basis<->quadrature transforms on the
-                              tensor cores as split-BF16 x3 products with FP32
-                              accumulation; FP64 global sums                      */
+#define DG_PREC_X3 2       /* FP32 state; basis<->quadrature transforms in FP32
+                              (the kernels of DG_PREC_F32) or, by x3_backend or
+                              with the diffusion operator, on the tensor cores as
+                              split-BF16 x3 products with FP32 accumulation; FP64
+                              global sums                                        */
 
 /* ---- artificial viscosity modes ------------------------------------------ */
 #define DG_AV_OFF 0
@@ -68,8 +70,8 @@ extern "C" {
 #define DG_ST_LIMITED 1u   /* positivity rescaling happened in some cell         */
 #define DG_ST_FAIL 2u      /* a cell mean reached the density floor              */
 #define DG_ST_NONFINITE 4u /* a NaN/Inf was produced                              */
-#define DG_ST_TIMEOUT 8u   /* a tensor-core completion wait gave up (the launch
-                              stopped early; reported as DG_ECUDA)              */
+#define DG_ST_TIMEOUT 8u   /* a completion wait gave up (reserved: no kernel of
+                              this library waits on a flag)                       */
 #define DG_ST_REPEATED 16u /* positivity by repetition: a step was computed
                               again with troubled cells flattened               */
 
@@ -108,9 +110,11 @@ typedef struct {
     double nu_gate;        /* default 0 (no gating)                                */
     double diffusion;      /* eps of an added div(eps grad u) on all four variables
                               (Sec. 2, diffusion across cell boundaries); 0: off   */
-    int32_t fused_infer;   /* DG_AV_LEARNED steps: 1 = the last stage's kernel
-                              evaluates the next step's coefficient; 0 (default) =
-                              a separate inference launch per step.  Same values. */
+    int32_t fused_infer;   /* DG_AV_LEARNED steps: 1 = the next step's coefficient
+                              is evaluated at the end of a step (inside the last
+                              stage's kernel with the fused stage kernel, by a
+                              launch after the last projection otherwise); 0
+                              (default) = at the start of the step.  Same values. */
 } dg_nu_params;
 
 typedef struct {
@@ -133,16 +137,12 @@ typedef struct {
     void* scratch;         /* >= dg_scratch_bytes(), 256-byte aligned              */
     size_t scratch_bytes;
     int32_t riemann;       /* DG_RIEMANN_*; 0 (Rusanov) when zero-initialised     */
-    int32_t x3_backend;    /* DG_PREC_X3 at order 3 without diffusion: 0 (default)
-                              = 5th-generation tensor-core kernels (tcgen05 with
-                              TMEM accumulators: volume and face kernels per
-                              stage, the projection kernel after the last stage
-                              and, in driven steps, after every stage; the volume
-                              term through a caller-scratch buffer; fused_infer
-                              evaluates the sensor in that last projection);
-                              1 = the single fused stage kernel on warp-level
-                              mma.sync.  Other precisions, orders and the
-                              diffusion operator use the fused kernel either way */
+    int32_t x3_backend;    /* DG_PREC_X3 without diffusion: 0 (default) = the
+                              sum-factorised FP32 kernels of DG_PREC_F32 (faster
+                              and more accurate than the split products);
+                              1 = the single fused stage kernel with split-BF16 x3
+                              products on warp-level mma.sync, which the diffusion
+                              operator uses either way                            */
     int32_t positivity;    /* DG_POS_*; DG_POS_SCALE when zero-initialised        */
 } dg_opts;
 
@@ -290,7 +290,7 @@ int dg_l1_density(dg_ctx* ctx, const void* uA, const void* uB, double* out);
  * rho (h/p)^2 |div v| / (2 dt) as in Sec. 3.1; nu is evaluated once per step
  * (BF16 tensor-core inference, FP32 accumulation) and kept for its stages:
  * by a separate inference kernel at the start of the step, or (fused_infer)
- * by the last stage of the previous step, in the same kernel, for the state
+ * at the end of the previous step (see dg_nu_params), for the state
  * it writes.  Both give the same values bit for bit; on GB300 the separate
  * launch is the faster of the two.
  * Parameters: FP32 array of dg_av_param_count() floats in the order

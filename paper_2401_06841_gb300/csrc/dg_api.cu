@@ -402,15 +402,10 @@ struct dg_ctx {
     unsigned char* trouble = nullptr;
     unsigned char* level = nullptr;
     bool marks_dirty = false;  // marks or levels may be non-zero
-    // x3 at order 3: tcgen05 kernels (volume, faces, projection)
-    bool tc5 = false;
     // the sum-factorised kernels: a stage is a volume and a face launch (the volume
     // kernel of the stages after the first projects its own input), and one
     // projection launch ends the step
     bool sf = false;
-    void* t5tab = nullptr;
-    T5Maps t5maps{};  // tiled TMA descriptors of the state registers, rvol and a_h (tcgen05 kernels)
-    void* rvol = nullptr;
     int mlp_D = 0, mlp_P = 0;
     long adam_t = 0;
     bool weights_set = false;
@@ -441,7 +436,6 @@ struct ScratchLayout {
     size_t mw, mm, mv, mg, mpack, mloss, mwork;  // learned sensor: weights, Adam moments, grad, packed, loss, work
     size_t nu, nu2, vabs;                        // per-cell coefficients (this and the next step) and |v| projection (learned mode)
     size_t ana;                                  // turbulence statistics: 4 x DG_MAX_BINS doubles + 1
-    size_t t5tab, rvol;                          // order 3: tensor-core table block, FP32 volume term [c][4][b]
     size_t trouble, level;                       // positivity by repetition: per-cell marks and levels (bytes)
     size_t total;
 };
@@ -494,12 +488,6 @@ ScratchLayout scratch_layout(int K, int N, bool learned = false)
     s.vabs = off;
     const size_t b = (size_t)(K + 1) * (K + 2) * (K + 3) / 6;
     if (learned) off = align256(off + sizeof(double) * (size_t)ncell * b);
-    // order 3: the tables and the volume-term buffer of the tcgen05 x3 kernels
-    // (reserved for every precision: the size query does not take one)
-    s.t5tab = off;
-    if (K == 3) off = align256(off + tc5_table_bytes());
-    s.rvol = off;
-    if (K == 3) off = align256(off + sizeof(float) * (size_t)ncell * 4 * b);
     s.trouble = off;
     off = align256(off + (size_t)ncell);
     s.level = off;
@@ -520,6 +508,9 @@ int fail(dg_ctx* c, int code, const std::string& msg)
         if (e_ != cudaSuccess)                                                                     \
             return fail(ctx, DG_ECUDA, std::string(#call) + ": " + cudaGetErrorString(e_));        \
     } while (0)
+
+// split-BF16 products on the tensor cores (the fused mma.sync kernel)
+bool x3_products(const dg_ctx* c) { return c->prec == DG_PREC_X3 && !c->sf; }
 
 Launch make_launch(const dg_ctx* c)
 {
@@ -546,7 +537,7 @@ Launch make_launch(const dg_ctx* c)
     L.ctl = c->ctl;
     L.partials = c->partials;
     L.nsm = c->nsm;
-    L.bk = (c->prec == DG_PREC_X3) ? 1 : 0;
+    L.bk = x3_products(c) ? BK_X3 : BK_FMA;
     L.r1 = c->r1;
     L.gtab = c->gtab;
     return L;
@@ -606,67 +597,11 @@ void drop_carry(dg_ctx* c)
     if (c) c->carry = false;
 }
 
-// the x3 stage of order 3 on the tcgen05 kernels: a projection launch, or the
-// volume + face launches of a right-hand side / stage followed by the
-// projection of the stage's output (F_NEXTPROJ)
-cudaError_t tile_tc5(dg_ctx* c, const TileLaunch& t)
-{
-    Launch L = make_launch(c);
-    using TT = TileTab<3, BK_X3>;
-    T5Launch p{};
-    p.tab5 = c->t5tab;
-    p.maps = &c->t5maps;
-    p.rvol = c->rvol;
-    p.phiv = static_cast<const float*>(c->ttab) + TT::phiv;
-    p.phif = static_cast<const float*>(c->ttab) + TT::phif;
-    p.nu = t.nu;
-    p.ahat = t.ahat;
-    p.rk_a = t.rk_a;
-    p.rk_b = t.rk_b;
-    p.dt_pimax = t.dt_pimax;
-    p.trouble = t.mode == TM_RHS ? nullptr : t.trouble;
-    if (t.mode == TM_PROJECT) {
-        Timed tm(c, KIND_PROJECT);
-        p.kind = T5_PROJECT;
-        p.u_in = t.u_in;
-        p.vh_out = t.vh_out;
-        p.vabs_out = t.vabs_out;
-        p.flags = t.flags;
-        p.abar_out = t.abar_out;
-        return launch_tc5(L, p);
-    }
-    {
-        Timed tm(c, KIND_RHS);
-        p.kind = (t.mode == TM_RHS) ? T5_RHS : T5_STAGE;
-        p.u_in = t.u_in;
-        p.u_n = t.u_n;
-        p.out = t.out;
-        p.vh_in = t.vh_in;
-        p.vh_self = (t.flags & F_SELFPROJ) ? const_cast<void*>(t.vh_in) : nullptr;
-        p.flags = t.flags & F_FORCE;
-        p.abar_in = t.abar_in;
-        cudaError_t e = launch_tc5(L, p);
-        if (e != cudaSuccess) return e;
-    }
-    if (t.mode != TM_RHS && (t.flags & F_NEXTPROJ)) {
-        Timed tm(c, KIND_PROJECT);
-        T5Launch q = p;
-        q.kind = T5_PROJECT;
-        q.u_in = t.out;
-        q.vh_out = t.vh_out;
-        q.vabs_out = t.vabs_out;
-        q.nu_next = t.nu_next;
-        q.mlp = t.mlp;
-        q.flags = t.flags & (F_FORCE | F_DT);
-        q.abar_out = t.abar_out;
-        return launch_tc5(L, q);
-    }
-    return cudaSuccess;
-}
-
+// the launches of a projection, a right-hand side or a stage (with F_NEXTPROJ the
+// projection of its output: a launch of its own on the sum-factorised kernels, in
+// the fused kernel's epilogue otherwise)
 cudaError_t tile(dg_ctx* c, const TileLaunch& t)
 {
-    if (c->tc5) return tile_tc5(c, t);
     const Launch L = make_launch(c);
     auto go = [&](const TileLaunch& x) {
         Timed tm(c, x.mode == TM_PROJECT ? KIND_PROJECT : KIND_RHS);
@@ -895,16 +830,16 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
     ctx->nu_cell = (float*)(ctx->scratch + sl.nu);
     ctx->nu_next = (float*)(ctx->scratch + sl.nu2);
     ctx->vabs = ctx->scratch + sl.vabs;
-    ctx->t5tab = ctx->scratch + sl.t5tab;
-    ctx->rvol = ctx->scratch + sl.rvol;
     ctx->repeat = opts->positivity == DG_POS_REPEAT;
     ctx->trouble = reinterpret_cast<unsigned char*>(ctx->scratch + sl.trouble);
     ctx->level = reinterpret_cast<unsigned char*>(ctx->scratch + sl.level);
     ctx->marks_dirty = true;
-    // order-3 x3 on the tcgen05 kernels (the learned sensor's in-step evaluation,
-    // fused_infer, runs in their last projection)
-    ctx->tc5 = ctx->prec == DG_PREC_X3 && order == 3 && nu->diffusion == 0.0 && opts->x3_backend == 0;
-    ctx->sf = ctx->prec != DG_PREC_X3 && nu->diffusion == 0.0;
+    // x3 by default runs on the same kernels as FP32: axis by axis in FP32 registers
+    // the transforms take less time than as split-BF16 products on the tensor cores
+    // (64^3 P3, one driven step: 1.1 ms against 2.9 ms on tcgen05 products and 3.4 ms in
+    // the fused mma.sync kernel; the tensor pipe was 22-24 % busy, the rest of the time
+    // went into splitting operands, staging them and waiting for products)
+    ctx->sf = nu->diffusion == 0.0 && (ctx->prec != DG_PREC_X3 || opts->x3_backend == 0);
     ctx->mlp_D = 2 * ctx->b;
     ctx->mlp_P = mlp_params(ctx->mlp_D);
 
@@ -912,13 +847,6 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->nsm, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess) e = (ctx->prec == DG_PREC_F64) ? setup_kernels<double>(order) : setup_kernels<float>(order);
-    if (e == cudaSuccess && ctx->tc5) e = tc5_setup();
-    if (e == cudaSuccess && ctx->tc5) {
-        // whole tiles by tiled TMA loads (1D bulk copies where no descriptor could be made)
-        const void* bases[5] = {ctx->reg[0], ctx->reg[1], ctx->reg[2], ctx->rvol, ctx->ahat};
-        const int per[5] = {80, 80, 80, 80, 60};
-        if (tc5_make_maps(&ctx->t5maps, bases, per, 5, ctx->ncell) != cudaSuccess) ctx->t5maps.n = 0;
-    }
     if (e != cudaSuccess) {
         fprintf(stderr, "dg_init: %s\n", cudaGetErrorString(e));
         delete ctx;
@@ -926,7 +854,9 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
     }
     // tables in the element type of the precision mode
     std::vector<double> t = tables_for(order);
-    std::vector<char> tt = tile_tables_for(order, ctx->prec);
+    // x3 on the FP32 kernels takes their tables
+    std::vector<char> tt =
+        tile_tables_for(order, ctx->prec == DG_PREC_X3 && !x3_products(ctx) ? DG_PREC_F32 : ctx->prec);
     Ctl c0{};
     c0.dt_scale = 1.0;
     c0.dt_num = ctx->cfl * ctx->h / (order + 1);
@@ -943,12 +873,6 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
             e = cudaMemcpyAsync(ctx->tab, tf.data(), sizeof(float) * tf.size(), cudaMemcpyHostToDevice, ctx->st);
         }
         if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->ttab, tt.data(), tt.size(), cudaMemcpyHostToDevice, ctx->st);
-        std::vector<unsigned char> t5;
-        if (e == cudaSuccess && ctx->tc5) {
-            t5.resize(tc5_table_bytes());
-            if (tc5_build_tables(ctx->r1.x, ctx->r1.w, t5.data(), t5.size()) != 0) e = cudaErrorInvalidValue;
-            if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->t5tab, t5.data(), t5.size(), cudaMemcpyHostToDevice, ctx->st);
-        }
         if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->st);
     }
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->ahat, 0, vec_bytes(ctx), ctx->st);
@@ -1023,10 +947,7 @@ int dg_rhs(dg_ctx* ctx, const void* u_in, const void* ahat, void* dudt, double d
     t.flags = ahat ? F_FORCE : 0;
     t.abar_in = 0;
     CK(tile(ctx, t));
-    unsigned int st = 0u;
-    CK(cudaMemcpyAsync(&st, &ctx->ctl->status, sizeof(st), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
-    if (st & DG_ST_TIMEOUT) return fail(ctx, DG_ECUDA, "dg_rhs: a tensor-core completion wait timed out");
     return DG_OK;
 }
 
@@ -1188,11 +1109,11 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
                 t.ahat = force ? ctx->ahat : nullptr;
                 rk_weights(ctx->rk, s, ctx->prec != DG_PREC_F64, t.rk_a, t.rk_b);
                 // every stage projects its output; the last one for the next step,
-                // with the CFL bound (and |v| in learned mode).  On the tcgen05 kernels
-                // the stages after the first project their own input in the volume
-                // kernel instead (driven: with the forcing sums), so only the last
-                // stage's output gets a projection launch
-                const bool fold = ctx->tc5 || ctx->sf;
+                // with the CFL bound (and |v| in learned mode).  On the sum-factorised
+                // kernels the stages after the first project their own input in the
+                // volume kernel instead (driven: with the forcing sums), so only the
+                // last stage's output gets a projection launch
+                const bool fold = ctx->sf;
                 t.flags = (force ? F_FORCE : 0) | ((fold && !last) ? 0 : F_NEXTPROJ) | (last ? F_DT : 0) |
                           ((fold && s > 0) ? F_SELFPROJ : 0);
                 t.abar_in = (pb + s) & 1;
@@ -1254,7 +1175,6 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
         ctx->t += dt;
         ctx->dt_last = dt;
         ctx->steps += 1;
-        if (status & DG_ST_TIMEOUT) return fail(ctx, DG_ECUDA, "dg_step: a tensor-core completion wait timed out");
         if (status & DG_ST_NONFINITE) return fail(ctx, DG_ENONFINITE, "dg_step: non-finite coefficient");
     }
     if (t_out) *t_out = ctx->t;
@@ -1439,7 +1359,7 @@ int dg_generate_pairs(dg_ctx* ctx, double dt_for_pimax, float* x, float* y, int6
                                                                     : TileTab<3, BK_FMA>::phiv);
             CK(launch_features<double>(L, (const double*)u, (const double*)ctx->vabs, phiv, dt_for_pimax, x, y));
         } else {
-            const bool x3 = ctx->prec == DG_PREC_X3;
+            const bool x3 = x3_products(ctx);
             const int off = ctx->K == 1 ? (x3 ? TileTab<1, BK_X3>::phiv : TileTab<1, BK_FMA>::phiv)
                             : ctx->K == 2 ? (x3 ? TileTab<2, BK_X3>::phiv : TileTab<2, BK_FMA>::phiv)
                                           : (x3 ? TileTab<3, BK_X3>::phiv : TileTab<3, BK_FMA>::phiv);

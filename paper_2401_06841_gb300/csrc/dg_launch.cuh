@@ -64,54 +64,6 @@ cudaError_t launch_l1(const Launch& L, const T* uA, const T* uB);
 template <typename T>
 cudaError_t launch_flatten(const Launch& L, T* u, unsigned char* trouble, unsigned char* level);
 
-// x3 stage of degree 3 on the tcgen05 tensor cores (dg_tc5.cu): the
-// projection kernel, or the volume and face kernels of a right-hand side /
-// an SSP-RK stage
-enum { T5_PROJECT = 0, T5_RHS = 1, T5_STAGE = 2 };
-// tiled TMA descriptors (CUtensorMap, 128 bytes each) of the buffers whose whole
-// tiles the tcgen05 kernels stage: a context's state registers, the volume term
-// and the driving; a launch finds them by base address
-struct T5Map {
-    const void* base;
-    alignas(64) unsigned char map[128];
-};
-struct T5Maps {
-    int n;
-    T5Map m[8];
-};
-// one map per buffer [ncell][per] FP32 (boxes of 16 cells); DG_EINVAL-like
-// cudaErrorInvalidValue when the driver's encoder is missing or refuses
-cudaError_t tc5_make_maps(T5Maps* out, const void* const* bases, const int* per, int n, long ncell);
-
-struct T5Launch {
-    int kind;
-    const void* u_in;
-    const void* u_n;
-    void* out;
-    const void* vh_in;
-    void* vh_out;
-    void* vabs_out;
-    const void* ahat;
-    const float* nu;
-    void* rvol;          // volume term [c][4][b] FP32 (caller's scratch)
-    void* vh_self;       // undriven stages: the volume kernel projects v of u_in here (or nullptr)
-    float* nu_next;      // projection: the learned sensor's coefficient of u_in (or nullptr)
-    const uint32_t* mlp; // its packed network
-    const T5Maps* maps;  // tiled TMA descriptors of the context's buffers (or nullptr)
-    unsigned char* trouble;  // positivity by repetition: per-cell marks (or nullptr)
-    const void* tab5;    // table block (tc5_build_tables)
-    const void* phiv;    // [b][nq] FP32 phi at the volume points
-    const void* phif;    // [b][nf] FP32 phi at the face points
-    double rk_a, rk_b;
-    double dt_pimax;
-    int flags;
-    int abar_in, abar_out;
-};
-size_t tc5_table_bytes();
-int tc5_build_tables(const double* x, const double* w, unsigned char* out, size_t cap);
-cudaError_t tc5_setup();
-cudaError_t launch_tc5(const Launch& L, const T5Launch& t);
-
 // adiabatic system (dg_adi.cu): mode 0 projection of v and p (+ CFL bound
 // with F_DT, forcing sums with F_FORCE), 1 right-hand side, 2 stage
 // (right-hand side, SSP-RK combine, positivity of density and pressure),
