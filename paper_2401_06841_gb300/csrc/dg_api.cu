@@ -22,6 +22,7 @@
 
 #include <cufft.h>
 #include <dlfcn.h>
+#include "dg_force.cuh"
 #include "dg_launch.cuh"
 #include "dg_mlp.cuh"
 #include "dg_tables.cuh"
@@ -211,7 +212,7 @@ int tab_total(int K)
 // ---------------------------------------------------------------------------
 // Ornstein-Uhlenbeck driving (Sec. 4.2)
 // ---------------------------------------------------------------------------
-constexpr int kMaxModes = 512;
+constexpr int kMaxModes = kForceModes;
 
 struct Driver {
     bool on = false, dirty = false;
@@ -312,6 +313,41 @@ struct Driver {
     }
 };
 
+// the modes in the order and packing of the forcing projection (dg_force.cuh):
+// packed, pair starts and group starts into ints [3 kMaxModes], the amplitudes
+// (conjugated where kx is flipped) into amp_out [nm][3][2]
+ForceModes pack_modes(int nm, const int* kvec, const double* amp, std::vector<int>& ints, std::vector<double>& amp_out)
+{
+    std::vector<int> order(nm), sgn(nm);
+    for (int m = 0; m < nm; ++m) {
+        order[m] = m;
+        sgn[m] = kvec[3 * m] < 0 ? -1 : 1;
+    }
+    auto key = [&](int m, int d) { return sgn[m] * kvec[3 * m + d]; };
+    std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
+        for (int d = 0; d < 3; ++d)
+            if (key(p, d) != key(q, d)) return key(p, d) < key(q, d);
+        return false;
+    });
+    ints.assign(3 * kMaxModes, 0);
+    amp_out.assign(6 * (size_t)nm, 0.0);
+    ForceModes fm{nm, 0, 0};
+    for (int i = 0; i < nm; ++i) {
+        const int m = order[i], kx = key(m, 0), ky = key(m, 1), kz = key(m, 2);
+        ints[i] = kx | (ky + kForceKM) << 8 | (kz + kForceKM) << 16;
+        for (int v = 0; v < 3; ++v) {
+            amp_out[(i * 3 + v) * 2] = amp[(m * 3 + v) * 2];
+            amp_out[(i * 3 + v) * 2 + 1] = sgn[m] * amp[(m * 3 + v) * 2 + 1];
+        }
+        const bool newpair = i == 0 || (ints[i] ^ ints[i - 1]) & 0xffff;
+        if (newpair) {
+            if (i == 0 || (ints[i] ^ ints[i - 1]) & 0xff) ints[kForceGroups + fm.ngroup++] = fm.npair;
+            ints[kForcePairs + fm.npair++] = i;
+        }
+    }
+    return fm;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
@@ -371,7 +407,8 @@ struct dg_ctx {
     void* ttab = nullptr;
     int* d_kvec = nullptr;
     double* d_amp = nullptr;
-    void* gtab = nullptr;  // forcing: 1D factors
+    void* gtab = nullptr;  // forcing: 1D factors (of the mesh and the rule: built by the first projection)
+    bool gtab_ready = false;
     double* ana = nullptr; // turbulence statistics accumulators
     cufftHandle fft = 0;   // power-spectrum plan (created on first use)
     int fft_ng = 0;
@@ -703,23 +740,34 @@ cudaError_t learned_nu(dg_ctx* c, const void* u)
     return learned_infer(c, u, c->nu_cell);
 }
 
+// the packed modes and amplitudes to the device, then their projection into ahat
+// (the host buffers must outlive the copies)
+cudaError_t force_project(dg_ctx* c, const ForceModes& fm, const std::vector<int>& ints, const std::vector<double>& amp)
+{
+    cudaError_t e;
+    if ((e = cudaMemcpyAsync(c->d_kvec, ints.data(), sizeof(int) * ints.size(), cudaMemcpyHostToDevice, c->st))) return e;
+    if ((e = cudaMemcpyAsync(c->d_amp, amp.data(), sizeof(double) * amp.size(), cudaMemcpyHostToDevice, c->st))) return e;
+    const Launch L = make_launch(c);
+    if (!c->gtab_ready) {
+        Timed tm(c, KIND_FORCE);
+        if ((e = c->prec == DG_PREC_F64 ? launch_force_axis<double>(L) : launch_force_axis<float>(L))) return e;
+        c->gtab_ready = true;
+    }
+    Timed tm(c, KIND_FORCE);
+    return c->prec == DG_PREC_F64 ? launch_force<double>(L, fm, c->d_kvec, c->d_amp, (double*)c->ahat)
+                                  : launch_force<float>(L, fm, c->d_kvec, c->d_amp, (float*)c->ahat);
+}
+
 int upload_forcing(dg_ctx* ctx)
 {
     std::vector<double> amp;
     std::vector<int> kv;
     ctx->drv.amplitudes(amp, kv);
     if (ctx->drv.nm == 0) return DG_OK;
-    CK(cudaMemcpyAsync(ctx->d_kvec, kv.data(), sizeof(int) * kv.size(), cudaMemcpyHostToDevice, ctx->st));
-    CK(cudaMemcpyAsync(ctx->d_amp, amp.data(), sizeof(double) * amp.size(), cudaMemcpyHostToDevice, ctx->st));
-    Launch L = make_launch(ctx);
-    cudaError_t e;
-    {
-        Timed tm(ctx, KIND_FORCE);
-        e = (ctx->prec == DG_PREC_F64)
-                ? launch_force<double>(L, ctx->drv.nm, ctx->d_kvec, ctx->d_amp, ctx->drv.kmaxc, (double*)ctx->ahat)
-                : launch_force<float>(L, ctx->drv.nm, ctx->d_kvec, ctx->d_amp, ctx->drv.kmaxc, (float*)ctx->ahat);
-    }
-    CK(e);
+    std::vector<int> ints;
+    std::vector<double> pamp;
+    const ForceModes fm = pack_modes(ctx->drv.nm, kv.data(), amp.data(), ints, pamp);
+    CK(force_project(ctx, fm, ints, pamp));
     // the host buffers must stay valid until the copies ran
     CK(cudaStreamSynchronize(ctx->st));
     ctx->forcing_active = true;
@@ -996,17 +1044,10 @@ int dg_forcing_from_modes(dg_ctx* ctx, int nmodes, const int32_t* kvec, const do
     int kmaxc = 0;
     for (int i = 0; i < 3 * nmodes; ++i) kmaxc = std::max(kmaxc, std::abs((int)kvec[i]));
     if (kmaxc > 8) return fail(ctx, DG_EINVAL, "dg_forcing_from_modes: |k_d| > 8");
-    CK(cudaMemcpyAsync(ctx->d_kvec, kvec, sizeof(int) * 3 * nmodes, cudaMemcpyHostToDevice, ctx->st));
-    CK(cudaMemcpyAsync(ctx->d_amp, amp, sizeof(double) * 6 * nmodes, cudaMemcpyHostToDevice, ctx->st));
-    Launch L = make_launch(ctx);
-    cudaError_t e;
-    {
-        Timed tm(ctx, KIND_FORCE);
-        e = (ctx->prec == DG_PREC_F64)
-                ? launch_force<double>(L, nmodes, ctx->d_kvec, ctx->d_amp, kmaxc, (double*)ctx->ahat)
-                : launch_force<float>(L, nmodes, ctx->d_kvec, ctx->d_amp, kmaxc, (float*)ctx->ahat);
-    }
-    CK(e);
+    std::vector<int> ints;
+    std::vector<double> pamp;
+    const ForceModes fm = pack_modes(nmodes, kvec, amp, ints, pamp);
+    CK(force_project(ctx, fm, ints, pamp));
     CK(cudaStreamSynchronize(ctx->st));
     ctx->drv.on = false;
     ctx->forcing_active = true;
@@ -1614,7 +1655,8 @@ struct dg_adi_ctx {
     void* ahat = nullptr;   // driving a_h [c][3][b] (scratch)
     int* d_kvec = nullptr;
     double* d_amp = nullptr;
-    void* gtab = nullptr;
+    void* gtab = nullptr;  // forcing: 1D factors, built by the first projection
+    bool gtab_ready = false;
     Rule1 r1{};
     Driver drv;
     bool forcing_active = false;
@@ -1915,14 +1957,21 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
                 std::vector<double> amp;
                 std::vector<int> kv;
                 ctx->drv.amplitudes(amp, kv);
-                ACK(cudaMemcpyAsync(ctx->d_kvec, kv.data(), sizeof(int) * kv.size(), cudaMemcpyHostToDevice, ctx->st));
-                ACK(cudaMemcpyAsync(ctx->d_amp, amp.data(), sizeof(double) * amp.size(), cudaMemcpyHostToDevice,
+                std::vector<int> ints;
+                std::vector<double> pamp;
+                const ForceModes fm = pack_modes(ctx->drv.nm, kv.data(), amp.data(), ints, pamp);
+                ACK(cudaMemcpyAsync(ctx->d_kvec, ints.data(), sizeof(int) * ints.size(), cudaMemcpyHostToDevice,
+                                    ctx->st));
+                ACK(cudaMemcpyAsync(ctx->d_amp, pamp.data(), sizeof(double) * pamp.size(), cudaMemcpyHostToDevice,
                                     ctx->st));
                 const Launch L = adi_make_launch(ctx);
-                ACK(ctx->prec == DG_PREC_F64 ? launch_force<double>(L, ctx->drv.nm, ctx->d_kvec, ctx->d_amp,
-                                                                    ctx->drv.kmaxc, (double*)ctx->ahat)
-                                             : launch_force<float>(L, ctx->drv.nm, ctx->d_kvec, ctx->d_amp,
-                                                                   ctx->drv.kmaxc, (float*)ctx->ahat));
+                if (!ctx->gtab_ready) {
+                    ACK(ctx->prec == DG_PREC_F64 ? launch_force_axis<double>(L) : launch_force_axis<float>(L));
+                    ctx->gtab_ready = true;
+                }
+                ACK(ctx->prec == DG_PREC_F64
+                        ? launch_force<double>(L, fm, ctx->d_kvec, ctx->d_amp, (double*)ctx->ahat)
+                        : launch_force<float>(L, fm, ctx->d_kvec, ctx->d_amp, (float*)ctx->ahat));
                 ACK(cudaStreamSynchronize(ctx->st));  // the host amplitude buffers are reused
                 ctx->drv.dirty = false;
                 ctx->forcing_active = true;

@@ -52,8 +52,13 @@ struct TileLaunch {
 };
 template <typename T>
 cudaError_t launch_tile(const Launch& L, const TileLaunch& t);
+// forcing projection (dg_force.cuh): the 1D factors L.gtab of a mesh, once per
+// context, and the projection of a list of modes
+struct ForceModes;
 template <typename T>
-cudaError_t launch_force(const Launch& L, int nm, const int* kvec, const double* amp, int kmaxc, T* ahat);
+cudaError_t launch_force_axis(const Launch& L);
+template <typename T>
+cudaError_t launch_force(const Launch& L, const ForceModes& fm, const int* modes, const double* amp, T* ahat);
 template <typename T>
 cudaError_t launch_diag(const Launch& L, const T* u, const T* ahat, double dt_pimax, int flags);
 template <typename T>

@@ -4,6 +4,7 @@
 
 #include "dg_kernels.cuh"
 #include "dg_tile.cuh"
+#include "dg_force.cuh"
 #include "dg_launch.cuh"
 
 namespace dg {
@@ -18,12 +19,10 @@ cudaError_t launch(const Launch& L, const TileLaunch& t);
 
 template <typename T, int K>
 struct Occ {
-    static int tile[2][2][4], force, diag;  // [diffusion][back end][mode]
+    static int tile[2][2][4], diag;  // [diffusion][back end][mode]
 };
 template <typename T, int K>
 int Occ<T, K>::tile[2][2][4] = {};
-template <typename T, int K>
-int Occ<T, K>::force = 0;
 template <typename T, int K>
 int Occ<T, K>::diag = 0;
 
@@ -73,7 +72,8 @@ static cudaError_t setup_k()
     constexpr int NT = Tile<K>::NT;
     cudaError_t e;
     if ((e = setup_tiles<T, K>()) != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&Occ<T, K>::force, k_force<T, K>, 256, 0);
+    e = cudaFuncSetAttribute(k_force<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(T) * ForceCfg<T, K>::total));
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&Occ<T, K>::diag, k_diag<T, K>, NT, 0);
     return e;
@@ -177,14 +177,25 @@ cudaError_t tile_k(const Launch& L, const TileLaunch& t)
 }
 
 template <typename T, int K>
-static cudaError_t force_k(const Launch& L, int nm, const int* kvec, const double* amp, int kmaxc, T* ahat)
+static cudaError_t force_axis_k(const Launch& L, T* G)
 {
-    if (nm > 512 || kmaxc > kForceKM) return cudaErrorInvalidValue;
-    T* G = static_cast<T*>(L.gtab);
     const int ng = L.N * kForceNK * (K + 1);
-    k_force_axis<T, K><<<(ng + 255) / 256, 256, 0, L.st>>>(L.r1, L.N, kmaxc, G);
-    const long nb = (L.ncell + 255) / 256;
-    k_force<T, K><<<grid_for(nb, Occ<T, K>::force, L.nsm), 256, 0, L.st>>>(G, L.N, L.ncell, nm, kvec, amp, ahat);
+    k_force_axis<T, K><<<(ng + 255) / 256, 256, 0, L.st>>>(L.r1, L.N, G);
+    return cudaGetLastError();
+}
+
+template <typename T, int K>
+static cudaError_t force_k(const Launch& L, const ForceModes& fm, const int* modes, const double* amp, T* ahat)
+{
+    using C = ForceCfg<T, K>;
+    if (fm.nm > kForceModes || fm.npair > C::NPAIR || fm.ngroup > kForceKM + 1) return cudaErrorInvalidValue;
+    // rows of a plane per block: enough to share the plane's sums, few enough for
+    // about four blocks per multiprocessor
+    long rpb = (long)L.N * L.N / (4L * L.nsm);
+    rpb = rpb < 1 ? 1 : (rpb > L.N ? L.N : rpb);
+    const dim3 g((unsigned)((L.N + rpb - 1) / rpb), (unsigned)L.N);
+    k_force<T, K><<<g, C::NT, sizeof(T) * C::total, L.st>>>(static_cast<const T*>(L.gtab), L.N, (int)rpb, fm, modes,
+                                                          amp, ahat);
     return cudaGetLastError();
 }
 
@@ -236,9 +247,14 @@ cudaError_t launch_tile(const Launch& L, const TileLaunch& t)
     DG_DISPATCH(tile_k, t);
 }
 template <typename T>
-cudaError_t launch_force(const Launch& L, int nm, const int* kvec, const double* amp, int kmaxc, T* ahat)
+cudaError_t launch_force_axis(const Launch& L)
 {
-    DG_DISPATCH(force_k, nm, kvec, amp, kmaxc, ahat);
+    DG_DISPATCH(force_axis_k, static_cast<T*>(L.gtab));
+}
+template <typename T>
+cudaError_t launch_force(const Launch& L, const ForceModes& fm, const int* modes, const double* amp, T* ahat)
+{
+    DG_DISPATCH(force_k, fm, modes, amp, ahat);
 }
 template <typename T>
 cudaError_t launch_diag(const Launch& L, const T* u, const T* ahat, double dt_pimax, int flags)
@@ -266,7 +282,8 @@ cudaError_t launch_flatten(const Launch& L, T* u, unsigned char* trouble, unsign
 #define DG_INSTANTIATE(T)                                                                                         \
     template cudaError_t setup_kernels<T>(int);                                                                  \
     template cudaError_t launch_tile<T>(const Launch&, const TileLaunch&);                                       \
-    template cudaError_t launch_force<T>(const Launch&, int, const int*, const double*, int, T*);               \
+    template cudaError_t launch_force_axis<T>(const Launch&);                                                    \
+    template cudaError_t launch_force<T>(const Launch&, const ForceModes&, const int*, const double*, T*);      \
     template cudaError_t launch_diag<T>(const Launch&, const T*, const T*, double, int);                        \
     template cudaError_t launch_l1<T>(const Launch&, const T*, const T*);                                       \
     template cudaError_t launch_flatten<T>(const Launch&, T*, unsigned char*, unsigned char*);
