@@ -117,7 +117,8 @@ cudaError_t launch_shell(const Launch& L, const void* F, int Ng, int nbins, doub
 constexpr int kMlpHidden = 64;
 constexpr int kMlpBatchMax = 4096;
 inline int mlp_params(int D) { return kMlpHidden * D + kMlpHidden + kMlpHidden * kMlpHidden + 2 * kMlpHidden + 1; }
-inline size_t mlp_work_floats_host() { return (size_t)6 * kMlpHidden * kMlpBatchMax + kMlpBatchMax; }
+// partial gradient sums: pairs of floats per block of 32 samples (the largest network: D = 40)
+inline size_t mlp_work_floats_host() { return (size_t)(kMlpBatchMax / 32) * 2 * (mlp_params(40) + 1); }
 cudaError_t mlp_train_pass(cudaStream_t st, int D, const float* W, const float* X, const float* Y, int n, float* work,
                            float* G, double* loss);
 cudaError_t mlp_adam(cudaStream_t st, int P, float* W, const float* G, float* m, float* v, float lr, float b1, float b2,

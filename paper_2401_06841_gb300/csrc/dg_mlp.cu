@@ -10,12 +10,15 @@ template <int D>
 static cudaError_t train_pass_d(cudaStream_t st, const float* W, const float* X, const float* Y, int n, float* work,
                                 float* G, double* loss)
 {
-    const MlpLayout L = MlpLayout::make(D);
-    const size_t sm = sizeof(float) * L.P;
-    const int g = (n + 127) / 128;
-    k_mlp_fwd<D><<<g, 128, sm, st>>>(W, X, Y, n, work);
-    k_mlp_bwd<D><<<g, 128, sm, st>>>(W, n, work);
-    k_mlp_grad<D><<<(L.P + 1 + 255) / 256, 256, 0, st>>>(X, n, work, G, loss);
+    constexpr MlpLayout L = MlpLayout::make(D);
+    constexpr size_t sm = sizeof(float) * MlpPass<D>::total;
+    static_assert(mlp_work_floats() >= (size_t)(MLP_BMAX / MLP_SB) * 2 * (L.P + 1), "partial sums fit the work buffer");
+    cudaError_t e = cudaFuncSetAttribute(k_mlp_pass<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e != cudaSuccess) return e;
+    const int nb = (n + MLP_SB - 1) / MLP_SB;
+    float2* part = reinterpret_cast<float2*>(work);
+    k_mlp_pass<D><<<nb, 256, sm, st>>>(W, X, Y, n, part);
+    k_mlp_reduce<D><<<(L.P + 1 + 63) / 64, 256, 0, st>>>(part, nb, n, G, loss);
     return cudaGetLastError();
 }
 

@@ -2,8 +2,8 @@
 //   y = W3 . gelu(W2 gelu(W1 x + b1) + b2) + b3,   gelu(z) = z/2 (1 + erf(z/sqrt 2))
 // predicting y = log(nu / (cs h/p)) from x = (rho_l/rho_0, |v|hat_l/cs), the
 // normalised modal coefficients of the cell (D = 2b inputs, 64 hidden units).
-// Training runs in FP32 on the CUDA cores (forward with stored activations,
-// backward, per-parameter gradient sums in a fixed order, Adam); inference is
+// Training runs in FP32 on the CUDA cores (forward, backward and the gradient sums
+// of a block of samples in one kernel, a reduction in a fixed order, Adam); inference is
 // one fused kernel with BF16 tensor-core products and FP32 accumulation, the
 // accumulator fragments of a layer feeding the next layer's operand fragments
 // directly in registers.
@@ -21,7 +21,7 @@ constexpr int MLP_BMAX = 4096;  // largest training batch
 
 struct MlpLayout {
     int D, P, oW1, ob1, oW2, ob2, oW3, ob3;
-    __host__ __device__ static MlpLayout make(int D)
+    __host__ __device__ static constexpr MlpLayout make(int D)
     {
         MlpLayout L{};
         L.D = D;
@@ -36,122 +36,238 @@ struct MlpLayout {
     }
 };
 
-// training work arrays, each [64][MLP_BMAX] (sample index fastest) plus r [MLP_BMAX]
-enum { MW_Z1 = 0, MW_A1 = 1, MW_Z2 = 2, MW_A2 = 3, MW_DZ1 = 4, MW_DZ2 = 5, MW_R = 6 };
-constexpr size_t mlp_work_floats() { return (size_t)6 * MLP_H * MLP_BMAX + MLP_BMAX; }
+// training work: the gradient sums of every block of MLP_SB samples, [block][P + 1]
+// pairs of floats (the last one: the sum of squared errors)
+constexpr int MLP_SB = 32;
+constexpr size_t mlp_work_floats() { return (size_t)(MLP_BMAX / MLP_SB) * 2 * (MlpLayout::make(40).P + 1); }
 
 __device__ __forceinline__ float gelu_prime_f(float z)
 {
     return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * expf(-0.5f * z * z);
 }
 
-// forward pass of a batch, one thread per sample; stores z1, a1, z2, a2, r = y^ - y
+// a sum carried as an unevaluated pair of floats: the rounding error of every
+// product (FMA) and of every addition (Knuth's two-sum) goes into the second
+// float, so the sum is good to about 2^-46 of its terms.  FP64 sums would be no
+// better once rounded to the FP32 gradient, and run at a sixty-fourth of the rate.
+struct Pair {
+    float s = 0.f, c = 0.f;
+    __device__ __forceinline__ void add(float p, float e)
+    {
+        const float t = __fadd_rn(s, p), z = __fadd_rn(t, -s);
+        const float err = __fadd_rn(__fadd_rn(s, -__fadd_rn(t, -z)), __fadd_rn(p, -z));
+        s = t;
+        c = __fadd_rn(c, __fadd_rn(err, e));
+    }
+    __device__ __forceinline__ void add_prod(float a, float b)
+    {
+        const float p = __fmul_rn(a, b);
+        add(p, __fmaf_rn(a, b, -p));
+    }
+};
+
+// One training pass over MLP_SB samples per block, lane = sample, warp w = hidden
+// units 8w .. 8w+7: forward (activations in shared memory, pre-activations in
+// registers), backward, and the block's sums of the parameter gradients
+//   dz2 = (2 r / n) W3 gelu'(z2),  dz1 = (W2^T dz2) gelu'(z1),
+//   dW1 = dz1 x^T, dW2 = dz2 a1^T, dW3 = (2/n) sum r a2.
+// The products of a gradient entry are summed as pairs over the block's samples
+// and over the blocks (k_mlp_reduce) in a fixed order.
+// Bound: instruction issue of the 10-instruction pair products (6.8 thousand per
+// sample).  4096 samples at D = 40: forward, backward and gradients took 27 + 44 +
+// 2088 us as separate passes with one thread per sample and one per parameter in
+// FP64 over 27 blocks.
 template <int D>
-__global__ void __launch_bounds__(128) k_mlp_fwd(const float* __restrict__ W, const float* __restrict__ X,
-                                                 const float* __restrict__ Y, int n, float* __restrict__ work)
+struct MlpPass {
+    static constexpr MlpLayout L = MlpLayout::make(D);
+    static constexpr int SP = MLP_SB + 4;  // row stride of the transposed arrays (conflict-free 16-byte loads)
+    static constexpr int oX = (L.P + 3) / 4 * 4, oA1 = oX + D * SP, oA2 = oA1 + MLP_H * SP, oD1 = oA2 + MLP_H * SP;
+    static constexpr int oD2 = oD1 + MLP_H * SP, oR = oD2 + MLP_H * SP, total = oR + MLP_SB;
+    // thread tiles of dW1 [64][D]: TR x TC entries
+    static constexpr int TC = D % 5 == 0 ? 5 : 2, CG = D / TC, TR = MLP_H * CG / 256;
+    static_assert(D % 4 == 0 && TR * 256 == MLP_H * CG, "tiles cover dW1");
+};
+
+template <int D>
+__global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, const float* __restrict__ X,
+                                                  const float* __restrict__ Y, int n, float2* __restrict__ part)
 {
-    const MlpLayout L = MlpLayout::make(D);
-    extern __shared__ float sW[];
-    for (int e = threadIdx.x; e < L.P; e += blockDim.x) sW[e] = W[e];
+    using M = MlpPass<D>;
+    constexpr MlpLayout L = M::L;
+    constexpr int SP = M::SP;
+    extern __shared__ __align__(16) float sm[];
+    float* sX = sm + M::oX;
+    float* sA1 = sm + M::oA1;
+    float* sA2 = sm + M::oA2;
+    float* sD1 = sm + M::oD1;
+    float* sD2 = sm + M::oD2;
+    float* sR = sm + M::oR;
+    const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
+    const int i0 = blockIdx.x * MLP_SB, ns = min(MLP_SB, n - i0);
+    for (int e = tid; e < L.P; e += 256) sm[e] = W[e];
+    for (int e = tid; e < MLP_SB * D; e += 256) {
+        const int s = e / D, d = e - s * D;
+        sX[d * SP + s] = s < ns ? X[(size_t)i0 * D + e] : 0.f;
+    }
     __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float x[D];
+    float z1[8], z2[8];
 #pragma unroll
-    for (int d = 0; d < D; ++d) x[d] = X[(size_t)i * D + d];
-    float a1[MLP_H];
-#pragma unroll 4
-    for (int j = 0; j < MLP_H; ++j) {
-        float z = sW[L.ob1 + j];
+    for (int j = 0; j < 8; ++j) z1[j] = sm[L.ob1 + 8 * w + j];
+#pragma unroll 2
+    for (int d = 0; d < D; d += 4) {
+        const float x[4] = {sX[d * SP + lane], sX[(d + 1) * SP + lane], sX[(d + 2) * SP + lane], sX[(d + 3) * SP + lane]};
 #pragma unroll
-        for (int d = 0; d < D; ++d) z += sW[L.oW1 + j * D + d] * x[d];
-        a1[j] = gelu_f(z);
-        work[(size_t)MW_Z1 * MLP_H * MLP_BMAX + (size_t)j * MLP_BMAX + i] = z;
-        work[(size_t)MW_A1 * MLP_H * MLP_BMAX + (size_t)j * MLP_BMAX + i] = a1[j];
+        for (int j = 0; j < 8; ++j) {
+            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW1 + (8 * w + j) * D + d);
+            z1[j] += q.x * x[0];
+            z1[j] += q.y * x[1];
+            z1[j] += q.z * x[2];
+            z1[j] += q.w * x[3];
+        }
     }
-    float y = sW[L.ob3];
-#pragma unroll 4
-    for (int j = 0; j < MLP_H; ++j) {
-        float z = sW[L.ob2 + j];
 #pragma unroll
-        for (int k = 0; k < MLP_H; ++k) z += sW[L.oW2 + j * MLP_H + k] * a1[k];
-        const float a = gelu_f(z);
-        work[(size_t)MW_Z2 * MLP_H * MLP_BMAX + (size_t)j * MLP_BMAX + i] = z;
-        work[(size_t)MW_A2 * MLP_H * MLP_BMAX + (size_t)j * MLP_BMAX + i] = a;
-        y += sW[L.oW3 + j] * a;
+    for (int j = 0; j < 8; ++j) sA1[(8 * w + j) * SP + lane] = gelu_f(z1[j]);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < 8; ++j) z2[j] = sm[L.ob2 + 8 * w + j];
+#pragma unroll 2
+    for (int k = 0; k < MLP_H; k += 4) {
+        const float x[4] = {sA1[k * SP + lane], sA1[(k + 1) * SP + lane], sA1[(k + 2) * SP + lane],
+                            sA1[(k + 3) * SP + lane]};
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW2 + (8 * w + j) * MLP_H + k);
+            z2[j] += q.x * x[0];
+            z2[j] += q.y * x[1];
+            z2[j] += q.z * x[2];
+            z2[j] += q.w * x[3];
+        }
     }
-    work[(size_t)6 * MLP_H * MLP_BMAX + i] = y - Y[i];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) sA2[(8 * w + j) * SP + lane] = gelu_f(z2[j]);
+    __syncthreads();
+    if (w == 0) {
+        float y = sm[L.ob3];
+#pragma unroll 8
+        for (int j = 0; j < MLP_H; ++j) y += sm[L.oW3 + j] * sA2[j * SP + lane];
+        sR[lane] = lane < ns ? y - Y[i0 + lane] : 0.f;
+    }
+    __syncthreads();
+    const float d3 = 2.0f * sR[lane] / (float)n;
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+        sD2[(8 * w + j) * SP + lane] = d3 * sm[L.oW3 + 8 * w + j] * gelu_prime_f(z2[j]);
+    __syncthreads();
+    {
+        float s[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) s[k] = 0.f;
+#pragma unroll 4
+        for (int j = 0; j < MLP_H; ++j) {
+            const float dz = sD2[j * SP + lane];
+            const float4 q0 = *reinterpret_cast<const float4*>(sm + L.oW2 + j * MLP_H + 8 * w);
+            const float4 q1 = *reinterpret_cast<const float4*>(sm + L.oW2 + j * MLP_H + 8 * w + 4);
+            s[0] += q0.x * dz;
+            s[1] += q0.y * dz;
+            s[2] += q0.z * dz;
+            s[3] += q0.w * dz;
+            s[4] += q1.x * dz;
+            s[5] += q1.y * dz;
+            s[6] += q1.z * dz;
+            s[7] += q1.w * dz;
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) sD1[(8 * w + k) * SP + lane] = s[k] * gelu_prime_f(z1[k]);
+    }
+    __syncthreads();
+    float2* out = part + (size_t)blockIdx.x * (L.P + 1);
+    auto row4 = [](const float* p, float* o) {
+        const float4 v = *reinterpret_cast<const float4*>(p);
+        o[0] = v.x;
+        o[1] = v.y;
+        o[2] = v.z;
+        o[3] = v.w;
+    };
+    // sums over the samples of the products of rows i0 + i IS of A and j0 + j JS of B
+    // (interleaved rows: consecutive threads read consecutive rows)
+    auto tile = [&](auto R_, auto C_, auto IS_, auto JS_, const float* A, const float* B, float2* o, int ldo) {
+        constexpr int R = decltype(R_)::value, C = decltype(C_)::value, IS = decltype(IS_)::value,
+                      JS = decltype(JS_)::value;
+        Pair acc[R][C];
+#pragma unroll 1
+        for (int s = 0; s < MLP_SB; s += 4) {
+            float a[R][4], b[C][4];
+#pragma unroll
+            for (int i = 0; i < R; ++i) row4(A + i * IS * SP + s, a[i]);
+#pragma unroll
+            for (int j = 0; j < C; ++j) row4(B + j * JS * SP + s, b[j]);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int j = 0; j < C; ++j) acc[i][j].add_prod(a[i][q], b[j][q]);
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) o[i * IS * ldo + j * JS] = make_float2(acc[i][j].s, acc[i][j].c);
+    };
+    using std::integral_constant;
+    {
+        const int j = tid >> 4, k = tid & 15;
+        tile(integral_constant<int, 4>{}, integral_constant<int, 4>{}, integral_constant<int, 16>{},
+             integral_constant<int, 16>{}, sD2 + j * SP, sA1 + k * SP, out + L.oW2 + j * MLP_H + k, MLP_H);
+    }
+    {
+        const int j = tid / M::CG, d = tid % M::CG;
+        tile(integral_constant<int, M::TR>{}, integral_constant<int, M::TC>{}, integral_constant<int, 256 / M::CG>{},
+             integral_constant<int, M::CG>{}, sD1 + j * SP, sX + d * SP, out + L.oW1 + j * D + d, D);
+    }
+    // biases, the last layer and the loss: one entry per thread
+    if (tid < 3 * MLP_H + 2) {
+        const int j = tid & (MLP_H - 1), g = tid / MLP_H;
+        const float* a = g == 0 ? sD1 + j * SP : g == 1 ? sD2 + j * SP : g == 2 ? sA2 + j * SP : sR;
+        Pair acc;
+        for (int s = 0; s < MLP_SB; ++s) {
+            if (g < 2 || tid == 3 * MLP_H)
+                acc.add(a[s], 0.f);
+            else
+                acc.add_prod(a[s], sR[s]);
+        }
+        const int p = g == 0 ? L.ob1 + j : g == 1 ? L.ob2 + j : g == 2 ? L.oW3 + j : tid == 3 * MLP_H ? L.ob3 : L.P;
+        out[p] = make_float2(acc.s, acc.c);
+    }
 }
 
-// backward pass, one thread per sample: dz2 = (2 r / n) W3 gelu'(z2),
-// dz1 = (W2^T dz2) gelu'(z1)
+// gradient and loss from the blocks' sums: four threads per entry take the blocks
+// in quarters, added in order
 template <int D>
-__global__ void __launch_bounds__(128) k_mlp_bwd(const float* __restrict__ W, int n, float* __restrict__ work)
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float2* __restrict__ part, int nb, int n,
+                                                    float* __restrict__ G, double* __restrict__ loss)
 {
-    const MlpLayout L = MlpLayout::make(D);
-    extern __shared__ float sW[];
-    for (int e = threadIdx.x; e < L.P; e += blockDim.x) sW[e] = W[e];
+    constexpr MlpLayout L = MlpLayout::make(D);
+    __shared__ float2 s[4][64];
+    const int e = threadIdx.x & 63, q = threadIdx.x >> 6, p = blockIdx.x * 64 + e;
+    const int len = (nb + 3) / 4, b0 = q * len, b1 = min(nb, b0 + len);
+    Pair acc;
+    if (p <= L.P) {
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) {
+            const float2 v = part[(size_t)b * (L.P + 1) + p];
+            acc.add(v.x, v.y);
+        }
+    }
+    s[q][e] = make_float2(acc.s, acc.c);
     __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float d3 = 2.0f * work[(size_t)6 * MLP_H * MLP_BMAX + i] / (float)n;
-    float dz2[MLP_H];
-#pragma unroll
-    for (int j = 0; j < MLP_H; ++j) {
-        const float z = work[(size_t)MW_Z2 * MLP_H * MLP_BMAX + (size_t)j * MLP_BMAX + i];
-        dz2[j] = d3 * sW[L.oW3 + j] * gelu_prime_f(z);
-        work[(size_t)MW_DZ2 * MLP_H * MLP_BMAX + (size_t)j * MLP_BMAX + i] = dz2[j];
+    if (q == 0 && p <= L.P) {
+        for (int r = 1; r < 4; ++r) acc.add(s[r][e].x, s[r][e].y);
+        const double v = (double)acc.s + (double)acc.c;
+        if (p == L.P)
+            *loss = v / n;
+        else
+            G[p] = (float)(p >= L.oW3 ? 2.0 * v / n : v);
     }
-#pragma unroll 4
-    for (int k = 0; k < MLP_H; ++k) {
-        float s = 0.0f;
-#pragma unroll
-        for (int j = 0; j < MLP_H; ++j) s += sW[L.oW2 + j * MLP_H + k] * dz2[j];
-        const float z = work[(size_t)MW_Z1 * MLP_H * MLP_BMAX + (size_t)k * MLP_BMAX + i];
-        work[(size_t)MW_DZ1 * MLP_H * MLP_BMAX + (size_t)k * MLP_BMAX + i] = s * gelu_prime_f(z);
-    }
-}
-
-// gradient of the batch loss, one thread per parameter (fixed summation
-// order over the samples, FP64 accumulation); the extra thread P writes the
-// mean squared error
-template <int D>
-__global__ void __launch_bounds__(256) k_mlp_grad(const float* __restrict__ X, int n, const float* __restrict__ work,
-                                                  float* __restrict__ G, double* __restrict__ loss)
-{
-    const MlpLayout L = MlpLayout::make(D);
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > L.P) return;
-    const float* R = work + (size_t)6 * MLP_H * MLP_BMAX;
-    double acc = 0.0;
-    if (p == L.P) {
-        for (int i = 0; i < n; ++i) acc += (double)R[i] * (double)R[i];
-        *loss = acc / n;
-        return;
-    }
-    auto row = [&](int which, int j) { return work + ((size_t)which * MLP_H + j) * MLP_BMAX; };
-    if (p < L.ob1) {
-        const int j = p / D, d = p % D;
-        const float* dz = row(MW_DZ1, j);
-        for (int i = 0; i < n; ++i) acc += (double)dz[i] * (double)X[(size_t)i * D + d];
-    } else if (p < L.oW2) {
-        const float* dz = row(MW_DZ1, p - L.ob1);
-        for (int i = 0; i < n; ++i) acc += (double)dz[i];
-    } else if (p < L.ob2) {
-        const int j = (p - L.oW2) / MLP_H, k = (p - L.oW2) % MLP_H;
-        const float* dz = row(MW_DZ2, j);
-        const float* a = row(MW_A1, k);
-        for (int i = 0; i < n; ++i) acc += (double)dz[i] * (double)a[i];
-    } else if (p < L.oW3) {
-        const float* dz = row(MW_DZ2, p - L.ob2);
-        for (int i = 0; i < n; ++i) acc += (double)dz[i];
-    } else if (p < L.ob3) {
-        const float* a = row(MW_A2, p - L.oW3);
-        for (int i = 0; i < n; ++i) acc += 2.0 * (double)R[i] / n * (double)a[i];
-    } else {
-        for (int i = 0; i < n; ++i) acc += 2.0 * (double)R[i] / n;
-    }
-    G[p] = (float)acc;
 }
 
 // Adam (Kingma & Ba 2015) with bias corrections c1 = 1/(1-b1^t), c2 = 1/(1-b2^t)
