@@ -4,54 +4,70 @@
 
 #include "dg_adi.cuh"
 #include "dg_launch.cuh"
+#include "dg_sf_adi.cuh"
 
 namespace dg {
 
-namespace {
+namespace sf {
 
-template <typename T, int K, int MODE, bool DRIVEN>
-int adi_blocks_per_sm()
+template <typename T, int K, int MODE, bool FORCE, bool PROJ>
+cudaError_t adi_vol(const Launch& L, const AArgs<T>& a)
 {
-    static int occ = -1;
-    if (occ < 0) {
-        const int sm = (int)(sizeof(T) * AdiCfg<K, DRIVEN>::total);
-        cudaFuncSetAttribute(k_adi<T, K, MODE, DRIVEN>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm);
+    using C = AVolCfg<T, K, MODE, FORCE, PROJ>;
+    constexpr size_t sm = sizeof(T) * C::total;
+    static const int occ = [] {
         int o = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_adi<T, K, MODE, DRIVEN>, AdiCfg<K, DRIVEN>::NT, sm) !=
+        cudaFuncSetAttribute(k_sfa_vol<T, K, MODE, FORCE, PROJ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k_sfa_vol<T, K, MODE, FORCE, PROJ>, C::NT, sm) !=
             cudaSuccess)
             o = 1;
-        occ = o < 1 ? 1 : o;
-    }
-    return occ;
+        return o < 1 ? 1 : o;
+    }();
+    const long ntile = (L.ncell + TCELL - 1) / TCELL;
+    long g = (long)occ * L.nsm;
+    if (g > ntile) g = ntile;
+    if (g > kMaxGrid) g = kMaxGrid;
+    k_sfa_vol<T, K, MODE, FORCE, PROJ><<<(int)g, C::NT, sm, L.st>>>(a);
+    return cudaGetLastError();
 }
 
-template <typename T, int K, int MODE, bool DRIVEN = false>
-cudaError_t adi_launch(const Launch& L, const AdiArgs<T>& a)
+template <typename T, int K, int RS, bool STAGE>
+cudaError_t adi_faces(const Launch& L, const AArgs<T>& a)
 {
-    using A = AdiCfg<K, DRIVEN>;
-    const long ntile = (L.ncell + A::TC - 1) / A::TC;
-    long g = (long)adi_blocks_per_sm<T, K, MODE, DRIVEN>() * L.nsm;
-    if (g > ntile) g = ntile;
-    if (g < 1) g = 1;
-    k_adi<T, K, MODE, DRIVEN><<<(int)g, A::NT, sizeof(T) * A::total, L.st>>>(a);
+    constexpr size_t sm = sizeof(T) * AFaceCfg<T, K>::total;
+    static const cudaError_t ready = cudaFuncSetAttribute(k_sfa_faces<T, K, RS, STAGE>,
+                                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (ready != cudaSuccess) return ready;
+    const int nb = (L.N + 3) / 4, g = nb * nb * ((L.N + 1) / 2);  // bricks of 4 x 4 x 2 cells
+    k_sfa_faces<T, K, RS, STAGE><<<g, 128, sm, L.st>>>(a);
     return cudaGetLastError();
 }
 
 template <typename T, int K>
 cudaError_t adi_k(const Launch& L, double gamma, const AdiLaunch& t)
 {
-    AdiArgs<T> a{};
+    using TT = TileTab<K, BK_FMA>;
+    AArgs<T> a{};
+    const bool driven = (t.flags & F_FORCE) != 0;
+    if (driven && !t.ahat) return cudaErrorInvalidValue;
     a.u_in = static_cast<const T*>(t.u_in);
     a.u_n = static_cast<const T*>(t.u_n);
     a.out = static_cast<T*>(t.out);
     a.pr_in = static_cast<const T*>(t.pr_in);
     a.pr_out = static_cast<T*>(t.pr_out);
-    a.tab = static_cast<const T*>(L.ttab);
+    a.ahat = driven ? static_cast<const T*>(t.ahat) : nullptr;
+    a.phiv = static_cast<const T*>(L.ttab) + TT::phiv;
+    a.phif = static_cast<const T*>(L.ttab) + TT::phif;
     a.ctl = L.ctl;
+    a.partials = L.partials;
     a.ncell = L.ncell;
     a.N = L.N;
-    a.ph = L.ph;
-    a.gamma = gamma;
+    a.av_mode = L.ph.av_mode;
+    a.stage = t.mode == ADI_STAGE;
+    a.dtf = (t.flags & F_DT) ? 1 : 0;
+    a.abar_in = t.abar_in;
+    a.abar_out = t.abar_out;
+    fill_rows<T, K>(a.rows);
     a.gas.gamma = T(gamma);
     a.gas.g1 = T(gamma - 1.0);
     a.gas.ig1 = T(1.0 / (gamma - 1.0));
@@ -59,26 +75,45 @@ cudaError_t adi_k(const Launch& L, double gamma, const AdiLaunch& t)
     a.gas.kap = T(t.kap);
     a.gas.c0 = T((gamma - 1.0) * t.kap);
     a.gas.cres = T(t.cs_reset * t.cs_reset / (gamma - 1.0) - t.kap);
-    a.gas.fill_e = T((1.0 - (gamma - 1.0) * t.kap) / (gamma - 1.0));
+    a.two_h = T(2.0 / L.ph.h);
+    a.inv_h = T(1.0 / L.ph.h);
+    a.eps = T(L.ph.floor_);
+    a.a2 = T(L.ph.alpha * L.ph.hp * L.ph.hp);
+    a.bh = T(L.ph.beta * L.ph.hp);
     a.rk_a = T(t.rk_a);
     a.rk_b = T(t.rk_b);
+    a.hp = L.ph.hp;
+    a.h3 = L.ph.h * L.ph.h * L.ph.h;
     a.dt_pimax = t.dt_pimax;
-    a.flags = t.flags;
-    a.ahat = static_cast<const T*>(t.ahat);
-    a.partials = L.partials;
-    a.abar_in = t.abar_in;
-    a.abar_out = t.abar_out;
     a.beta = t.beta;
-    a.cs_reset = t.cs_reset;
     for (int i = 0; i < 3; ++i) a.bc[i] = t.bc[i];
-    for (int i = 0; i < 5; ++i) a.inflow[i] = t.inflow[i];
-    if ((t.flags & F_FORCE) && !t.ahat) return cudaErrorInvalidValue;
-    const bool driven = (t.flags & F_FORCE) != 0;
-    if (t.mode == ADI_PROJECT) return adi_launch<T, K, ADI_PROJECT>(L, a);
-    if (t.mode == ADI_RESET) return adi_launch<T, K, ADI_RESET>(L, a);
-    if (t.mode == ADI_RHS) return driven ? adi_launch<T, K, ADI_RHS, true>(L, a) : adi_launch<T, K, ADI_RHS>(L, a);
-    return driven ? adi_launch<T, K, ADI_STAGE, true>(L, a) : adi_launch<T, K, ADI_STAGE>(L, a);
+    for (int i = 0; i < 4; ++i) a.inflow[i] = T(t.inflow[i]);
+    a.inflow[4] = T(t.inflow[4] - (double)a.gas.c0 * t.inflow[0]);
+    if (t.mode == ADI_PROJECT)
+        return driven ? adi_vol<T, K, SFA_PROJECT, true, true>(L, a) : adi_vol<T, K, SFA_PROJECT, false, true>(L, a);
+    if (t.mode == ADI_RESET) return adi_vol<T, K, SFA_RESET, false, false>(L, a);
+    cudaError_t e;
+    if (t.flags & F_SELFPROJ) {
+        a.pr_out = const_cast<T*>(a.pr_in);
+        a.abar_out = t.abar_in;
+        e = driven ? adi_vol<T, K, SFA_VOLUME, true, true>(L, a) : adi_vol<T, K, SFA_VOLUME, false, true>(L, a);
+    } else {
+        e = driven ? adi_vol<T, K, SFA_VOLUME, true, false>(L, a) : adi_vol<T, K, SFA_VOLUME, false, false>(L, a);
+    }
+    if (e != cudaSuccess) return e;
+    if (a.stage)
+        return L.ph.riemann == 2 ? adi_faces<T, K, 2, true>(L, a) : adi_faces<T, K, 0, true>(L, a);
+    return L.ph.riemann == 2 ? adi_faces<T, K, 2, false>(L, a) : adi_faces<T, K, 0, false>(L, a);
 }
+
+}  // namespace sf
+
+// the degree-3 launcher compiles in a translation unit of its own
+#define DG_ADI_K3_EXTERN(T) \
+    extern template cudaError_t sf::adi_k<T, 3>(const Launch&, double, const AdiLaunch&);
+#define DG_ADI_K3_INSTANTIATE(T) template cudaError_t sf::adi_k<T, 3>(const Launch&, double, const AdiLaunch&);
+
+namespace {
 
 template <typename T, int K>
 cudaError_t adi_totals_k(const Launch& L, double gamma, double kap, const void* u, double* partials, int* nblocks)
@@ -98,9 +133,9 @@ cudaError_t adi_totals_k(const Launch& L, double gamma, double kap, const void* 
 template <typename T>
 cudaError_t launch_adi(const Launch& L, double gamma, const AdiLaunch& t)
 {
-    if (L.K == 1) return adi_k<T, 1>(L, gamma, t);
-    if (L.K == 2) return adi_k<T, 2>(L, gamma, t);
-    return adi_k<T, 3>(L, gamma, t);
+    if (L.K == 1) return sf::adi_k<T, 1>(L, gamma, t);
+    if (L.K == 2) return sf::adi_k<T, 2>(L, gamma, t);
+    return sf::adi_k<T, 3>(L, gamma, t);
 }
 
 template <typename T>

@@ -1994,8 +1994,8 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
             ACK(cudaMemsetAsync(&ctx->ctl->status, 0, sizeof(unsigned int), ctx->st));
             ACK(cudaMemsetAsync(&ctx->ctl->smax, 0, sizeof(unsigned long long), ctx->st));
             ACK(cudaMemsetAsync(&ctx->ctl->diag[1], 0, sizeof(double), ctx->st));
-            // projections of v and p of u^n (with its CFL bound); every stage but the
-            // last projects its output for the next one (alternating buffers)
+            // projections of v and p of u^n (with its CFL bound); the later stages project
+            // their inputs (alternating buffers)
             void* pr[2] = {ctx->prim, ctx->prim2};
             AdiLaunch p{};
             p.mode = ADI_PROJECT;
@@ -2013,7 +2013,8 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
                 t.out = ctx->reg[out[s]];
                 t.pr_in = pr[s & 1];
                 t.pr_out = pr[(s + 1) & 1];
-                t.flags = (s + 1 < ctx->rk ? F_NEXTPROJ : 0) | (force ? F_FORCE : 0);
+                // the stages after the first project their own input in their volume kernel
+                t.flags = (s > 0 ? F_SELFPROJ : 0) | (force ? F_FORCE : 0);
                 t.ahat = ctx->ahat;
                 t.abar_in = s & 1;
                 t.abar_out = (s + 1) & 1;

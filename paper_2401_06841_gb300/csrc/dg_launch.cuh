@@ -69,10 +69,11 @@ cudaError_t launch_l1(const Launch& L, const T* uA, const T* uB);
 template <typename T>
 cudaError_t launch_flatten(const Launch& L, T* u, unsigned char* trouble, unsigned char* level);
 
-// adiabatic system (dg_adi.cu): mode 0 projection of v and p (+ CFL bound
+// adiabatic system (dg_sf_adi.cuh): mode 0 projection of v and p (+ CFL bound
 // with F_DT, forcing sums with F_FORCE), 1 right-hand side, 2 stage
-// (right-hand side, SSP-RK combine, positivity of density and pressure),
-// 3 isothermal reset of the thermal energy (in place)
+// (right-hand side, SSP-RK combine, positivity of density and pressure; with
+// F_SELFPROJ the projections of its input are written to pr_in first), 3 isothermal
+// reset of the thermal energy (in place)
 enum { ADI_PROJECT = 0, ADI_RHS = 1, ADI_STAGE = 2, ADI_RESET = 3 };
 struct AdiLaunch {
     int mode;

@@ -918,7 +918,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL 
             reduce(sum3, x4);
             if (tid == 0) mine[3] = x4[0];
         }
-        if (last_block_reduce<NT>(a.partials, mine, FORCE ? 4 : 0, &a.ctl->cnt_proj, s_tot, s_buf)) {
+        if (last_block_reduce<NT>(a.partials, mine, FORCE ? 4 : 0, &a.ctl->cnt_proj, s_tot)) {
             if (tid == 0) {
                 const int o = a.abar_out;
                 for (int i = 0; i < 3; ++i) a.ctl->abar2[o][i] = FORCE ? s_tot[i] / s_tot[3] : 0.0;

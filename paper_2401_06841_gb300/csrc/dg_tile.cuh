@@ -1375,7 +1375,7 @@ __global__ void __launch_bounds__(256) k_tile(TArgs<T> a)
             }
             __syncthreads();
         }
-        if (last_block_reduce<NT>(a.partials, mine, 4, &a.ctl->cnt_proj, s_tot, s_buf)) {
+        if (last_block_reduce<NT>(a.partials, mine, 4, &a.ctl->cnt_proj, s_tot)) {
             if (tid == 0) {
                 const int o = a.abar_out;
                 if (a.flags & F_FORCE) {
