@@ -3,40 +3,114 @@
 // velocity structure function, and the velocity sampled on the (k+1)N Fourier
 // grid with the shell sums of its power spectrum.  All evaluation in FP64
 // from the state's coefficients (FP64 or FP32), accumulation in FP64.
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+
 #include "dg_launch.cuh"
 #include "dg_launch_impl.cuh"
+#include "dg_sf.cuh"
 
 namespace dg {
 
-// sqrt(2m+1) P_m(x), m = 0..K, by the three-term recurrence
+// All of these kernels are bound by the FP64 pipe (2 lanes per clock and SM, a
+// sixty-fourth of FP32's): they evaluate the expansions axis by axis, and keep
+// divisions, roots and logarithms out of FP64 where single precision decides.
+
+// sqrt(2m+1) P_m(x), m = 0..K (K <= 3)
 template <int K>
 __device__ __forceinline__ void pnorm_all(double x, double* p)
 {
+    constexpr double r3 = csqrt(3.0), r5 = csqrt(5.0), r7 = csqrt(7.0);
     p[0] = 1.0;
-    if constexpr (K >= 1) p[1] = x;
-#pragma unroll
-    for (int m = 2; m <= K; ++m) p[m] = ((2.0 * m - 1.0) * x * p[m - 1] - (m - 1.0) * p[m - 2]) / m;
-#pragma unroll
-    for (int m = 1; m <= K; ++m) p[m] *= sqrt(2.0 * m + 1.0);
+    if constexpr (K >= 1) p[1] = r3 * x;
+    if constexpr (K >= 2) p[2] = (1.5 * r5) * x * x - 0.5 * r5;
+    if constexpr (K >= 3) p[3] = x * ((2.5 * r7) * x * x - 1.5 * r7);
 }
 
-// the fields (rho, m_x, m_y, m_z) of one cell at reference point xi
+// b coefficients: 16-byte loads where the row starts on a 16-byte boundary
+template <typename T, int b>
+__device__ __forceinline__ void load_row(const T* __restrict__ p, T* o)
+{
+    constexpr int V = 16 / (int)sizeof(T);
+    if (b % V == 0 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0) {
+#pragma unroll
+        for (int l = 0; l + V <= b; l += V) {
+            const uint4 q = __ldg(reinterpret_cast<const uint4*>(p + l));
+            memcpy(o + l, &q, 16);
+        }
+    } else {
+#pragma unroll
+        for (int l = 0; l < b; ++l) o[l] = __ldg(p + l);
+    }
+}
+
+// the fields (rho, m_x, m_y, m_z) of one cell at reference point xi, summed along
+// x, y, z in turn
 template <typename T, int K>
 __device__ __forceinline__ void eval_point(const T* __restrict__ uc, const double xi[3], double f[4])
 {
     constexpr int b = Dims<K>::b;
-    constexpr Modes<K> M{};
     double px[K + 1], py[K + 1], pz[K + 1];
     pnorm_all<K>(xi[0], px);
     pnorm_all<K>(xi[1], py);
     pnorm_all<K>(xi[2], pz);
-    f[0] = f[1] = f[2] = f[3] = 0.0;
-    static_for<0, b>([&](auto L) {
-        constexpr int l = decltype(L)::value;
-        const double ph = px[M.i[l]] * py[M.j[l]] * pz[M.l[l]];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) f[v] += (double)uc[v * b + l] * ph;
-    });
+    for (int v = 0; v < 4; ++v) {
+        T u[b];
+        load_row<T, b>(uc + v * b, u);
+        double fz = 0.0;
+        static_for<0, K + 1>([&](auto L) {
+            constexpr int l = decltype(L)::value;
+            double fy = 0.0;
+            static_for<0, K - l + 1>([&](auto J) {
+                constexpr int j = decltype(J)::value;
+                double fx = (double)u[sf::im<K>(0, j, l)];
+                static_for<1, K - l - j + 1>([&](auto I) {
+                    constexpr int i = decltype(I)::value;
+                    fx += px[i] * (double)u[sf::im<K>(i, j, l)];
+                });
+                fy = j == 0 ? fx : fy + py[j] * fx;
+            });
+            fz = l == 0 ? fy : fz + pz[l] * fy;
+        });
+        f[v] = fz;
+    }
+}
+
+// values of the normalised Legendre polynomials at n points of an axis, symmetric
+// about 0: P[a][m]
+struct Line {
+    double P[4][4];
+};
+// the n values of a line from the coefficients r[0..K] (even and odd parts of the
+// mirrored points share their products)
+template <int K>
+__device__ __forceinline__ void line_values(const Line& t, const double* r, double* out)
+{
+    constexpr int n = K + 1;
+#pragma unroll
+    for (int q = 0; q < (n + 1) / 2; ++q) {
+        const int a = n - 1 - q;
+        double e = r[0], o = 0.0;
+#pragma unroll
+        for (int m = 2; m <= K; m += 2) e += t.P[a][m] * r[m];
+#pragma unroll
+        for (int m = 1; m <= K; m += 2) o = m == 1 ? t.P[a][m] * r[m] : o + t.P[a][m] * r[m];
+        out[a] = e + o;
+        if (a != q) out[q] = e - o;
+    }
+}
+
+// the coefficients of field v of a cell in FP64
+template <typename T, int K>
+__device__ __forceinline__ void load_field(const T* __restrict__ uc, int v, double* o)
+{
+    constexpr int b = Dims<K>::b;
+    T x[b];
+    load_row<T, b>(uc + v * b, x);
+#pragma unroll
+    for (int l = 0; l < b; ++l) o[l] = (double)x[l];
 }
 
 // velocity m/rho at a point x of the periodic unit box
@@ -58,8 +132,9 @@ __device__ __forceinline__ void velocity_at(const T* __restrict__ u, int N, cons
     const long c = ((long)ic[2] * N + ic[1]) * N + ic[0];
     double f[4];
     eval_point<T, K>(u + c * 4 * Dims<K>::b, xi, f);
+    const double ir = 1.0 / f[0];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) v[d] = f[1 + d] / f[0];
+    for (int d = 0; d < 3; ++d) v[d] = f[1 + d] * ir;
 }
 
 // SplitMix64: the n-th output of the sequence started from `seed`, as a
@@ -91,33 +166,63 @@ __global__ void __launch_bounds__(256) k_mean_rho(const T* __restrict__ u, long 
     if (threadIdx.x == 0) atomicAdd(mean, s[0] / (double)ncell);
 }
 
-// volume-weighted histogram of log10(rho / mean) over the Gauss points of
-// every cell; each sample carries w_q / 8 / ncell of the volume
-template <typename T, int K>
-__global__ void __launch_bounds__(256) k_density_pdf(const T* __restrict__ u, long ncell, Rule1 r, const double* mean,
-                                                     double lo, double ds, int nbins, double* __restrict__ hist)
+// volume-weighted histogram of log10(rho / mean) over the Gauss points of every
+// cell.  The weights w_a w_b w_c take four values (the number of inner points among
+// a, b, c: two distinct 1D weights), so the samples are counted per bin and weight
+// class in integers, cnt[bin][class], and weighted once at the end.  The bin
+// floor((log10(rho/mean) - lo)/ds) comes from single precision, and from FP64 where
+// that lands within tol of a bin edge (tol above its error: same bins).
+// One thread per cell (64 points of degree 3: 16 M points in 6.2 ms with a thread
+// and a full evaluation per point).
+template <int K>
+__host__ __device__ constexpr int inner(int a)
 {
-    constexpr int n = K + 1, nq = n * n * n, b = Dims<K>::b;
-    extern __shared__ double s_hist[];
-    for (int i = threadIdx.x; i < nbins; i += blockDim.x) s_hist[i] = 0.0;
+    return K == 3 ? (a == 1 || a == 2) : (K == 2 ? a == 1 : 0);
+}
+template <typename T, int K>
+__global__ void __launch_bounds__(128) k_density_pdf(const T* __restrict__ u, long ncell,
+                                                     const __grid_constant__ Line t, const double* mean, double lo,
+                                                     double ds, float tol, int nbins,
+                                                     unsigned long long* __restrict__ cnt)
+{
+    constexpr int n = K + 1, b = Dims<K>::b, NP = sf::npair(K);
+    extern __shared__ unsigned int s_cnt[];
+    for (int i = threadIdx.x; i < 4 * nbins; i += blockDim.x) s_cnt[i] = 0u;
     __syncthreads();
     const double rm = *mean;
-    const long items = ncell * nq;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < items; e += (long)gridDim.x * blockDim.x) {
-        const long c = e / nq;
-        const int q = (int)(e % nq), a0 = q % n, a1 = (q / n) % n, a2 = q / (n * n);
-        const double xi[3] = {r.x[a0], r.x[a1], r.x[a2]};
-        double f[4];
-        eval_point<T, K>(u + c * 4 * b, xi, f);
-        if (!(f[0] > 0.0)) continue;
-        const double sv = log10(f[0] / rm);
-        const double bin = floor((sv - lo) / ds);
-        if (bin >= 0.0 && bin < (double)nbins)
-            atomicAdd(&s_hist[(int)bin], r.w[a0] * r.w[a1] * r.w[a2] / 8.0 / (double)ncell);
+    const float irm = (float)(1.0 / rm), lof = (float)lo, ids = (float)(1.0 / ds);
+    for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell; c += (long)gridDim.x * blockDim.x) {
+        double r[b], A[NP];
+        load_field<T, K>(u + c * 4 * b, 0, r);
+#pragma unroll 1
+        for (int z = 0; z < n; ++z) {
+            sf::plane_eval<double, K>(r, t.P[z], A);
+#pragma unroll 1
+            for (int y = 0; y < n; ++y) {
+                double q[n], f[n];
+                sf::row_eval<double, K>(A, t.P[y], q);
+                line_values<K>(t, q, f);
+                const int c2 = inner<K>(z) + inner<K>(y);
+#pragma unroll
+                for (int x = 0; x < n; ++x) {
+                    if (!(f[x] > 0.0)) continue;
+                    const float g = (float)f[x] * irm;
+                    const float s = (log10f(g) - lof) * ids, fl = floorf(s), fr = s - fl;
+                    int bin = -1;
+                    if (!(g > 1e-30f && g < 1e30f) || !(fr > tol && fr < 1.0f - tol)) {
+                        const double e = floor((log10(f[x] / rm) - lo) / ds);
+                        if (e >= 0.0 && e < (double)nbins) bin = (int)e;
+                    } else if (fl >= 0.0f && fl < (float)nbins) {
+                        bin = (int)fl;
+                    }
+                    if (bin >= 0) atomicAdd(&s_cnt[4 * bin + c2 + inner<K>(x)], 1u);
+                }
+            }
+        }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < nbins; i += blockDim.x)
-        if (s_hist[i] != 0.0) atomicAdd(&hist[i], s_hist[i]);
+    for (int i = threadIdx.x; i < 4 * nbins; i += blockDim.x)
+        if (s_cnt[i]) atomicAdd(&cnt[i], (unsigned long long)s_cnt[i]);
 }
 
 // structure-function pairs: item = j * npairs + p, five uniforms per item
@@ -127,12 +232,16 @@ __global__ void __launch_bounds__(256) k_structure(const T* __restrict__ u, int 
                                                    double* __restrict__ acc)
 {
     extern __shared__ double s_acc[];
-    for (int i = threadIdx.x; i < nbins; i += blockDim.x) s_acc[i] = 0.0;
+    double* s_l = s_acc + nbins;  // the bins' separations
+    for (int i = threadIdx.x; i < nbins; i += blockDim.x) {
+        s_acc[i] = 0.0;
+        s_l[i] = lmin * pow(lmax / lmin, (i + 0.5) / nbins);
+    }
     __syncthreads();
     const long items = (long)nbins * npairs;
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < items; e += (long)gridDim.x * blockDim.x) {
         const int j = (int)(e / npairs);
-        const double l = lmin * pow(lmax / lmin, (j + 0.5) / nbins);
+        const double l = s_l[j];
         const unsigned long long n0 = (unsigned long long)e * 5ull;
         double x[3], y[3], va[3], vb[3];
 #pragma unroll
@@ -158,27 +267,51 @@ __global__ void __launch_bounds__(256) k_structure(const T* __restrict__ u, int 
 
 // velocity component d on the Ng = (K+1) N grid, x_g = (g + 1/2)/Ng:
 // out[(gz Ng + gy) Ng + gx]
+// one thread per cell: rho and m_d axis by axis at the cell's (K+1)^3 grid points
 template <typename T, int K>
-__global__ void __launch_bounds__(256) k_sample(const T* __restrict__ u, int N, int d, double* __restrict__ out)
+__global__ void __launch_bounds__(128) k_sample(const T* __restrict__ u, int N, int d, const __grid_constant__ Line t,
+                                                double* __restrict__ out)
 {
-    constexpr int p = K + 1, b = Dims<K>::b;
-    const int Ng = p * N;
-    const long n3 = (long)Ng * Ng * Ng;
-    for (long g = blockIdx.x * 256L + threadIdx.x; g < n3; g += (long)gridDim.x * 256) {
-        const int gx = (int)(g % Ng), gy = (int)((g / Ng) % Ng), gz = (int)(g / ((long)Ng * Ng));
-        const double xi[3] = {(2.0 * (gx % p) + 1.0) / p - 1.0, (2.0 * (gy % p) + 1.0) / p - 1.0,
-                              (2.0 * (gz % p) + 1.0) / p - 1.0};
-        const long c = ((long)(gz / p) * N + gy / p) * N + gx / p;
-        double f[4];
-        eval_point<T, K>(u + c * 4 * b, xi, f);
-        out[g] = f[1 + d] / f[0];
+    constexpr int p = K + 1, b = Dims<K>::b, NP = sf::npair(K);
+    const long Ng = (long)p * N, ncell = (long)N * N * N;
+    for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell; c += (long)gridDim.x * blockDim.x) {
+        int ix, iy, iz;
+        cell_xyz(c, N, ix, iy, iz);
+        double r[b], m[b], A[NP], M[NP];
+        load_field<T, K>(u + c * 4 * b, 0, r);
+        load_field<T, K>(u + c * 4 * b, 1 + d, m);
+        double* o = out + ((long)iz * p * Ng + (long)iy * p) * Ng + (long)ix * p;
+#pragma unroll 1
+        for (int z = 0; z < p; ++z) {
+            sf::plane_eval<double, K>(r, t.P[z], A);
+            sf::plane_eval<double, K>(m, t.P[z], M);
+#pragma unroll 1
+            for (int y = 0; y < p; ++y) {
+                double q[p], f[p], g[p];
+                sf::row_eval<double, K>(A, t.P[y], q);
+                line_values<K>(t, q, f);
+                sf::row_eval<double, K>(M, t.P[y], q);
+                line_values<K>(t, q, g);
+                double* w = o + (z * Ng + y) * Ng;
+                if constexpr (p % 2 == 0) {
+#pragma unroll
+                    for (int x = 0; x < p; x += 2)
+                        *reinterpret_cast<double2*>(w + x) = make_double2(g[x] / f[x], g[x + 1] / f[x + 1]);
+                } else {
+#pragma unroll
+                    for (int x = 0; x < p; ++x) w[x] = g[x] / f[x];
+                }
+            }
+        }
     }
 }
 
 // shell sums of |F|^2 scale^2 over the half spectrum of a real-to-complex
 // transform F[gz][gy][kx] (kx = 0..Ng/2); a mode with 0 < kx < Ng/2 stands
 // for itself and its conjugate partner.  Bins logarithmic in |kappa|:
-// i = floor(log|kappa| / log kmax * nbins), capped at nbins - 1
+// i = floor(log|kappa| / log kmax * nbins), capped at nbins - 1; from single
+// precision, and from FP64 where that lands within tol of a bin edge (tol above its
+// error: same bins)
 __global__ void __launch_bounds__(256) k_shell(const double2* __restrict__ F, int Ng, int nbins, double scale2,
                                                int first, double* __restrict__ power, double* __restrict__ ksum,
                                                unsigned long long* __restrict__ count)
@@ -196,19 +329,22 @@ __global__ void __launch_bounds__(256) k_shell(const double2* __restrict__ F, in
     const int nh = Ng / 2 + 1;
     const long total = (long)Ng * Ng * nh;
     const double lkmax = log(sqrt(3.0) * Ng / 2.0);
+    const float hb = (float)(0.5 * nbins / lkmax), tol = 1e-6f * nbins;
     for (long e = blockIdx.x * 256L + threadIdx.x; e < total; e += (long)gridDim.x * 256) {
         const int kx = (int)(e % nh), gy = (int)((e / nh) % Ng), gz = (int)(e / ((long)nh * Ng));
         const int ky = (2 * gy <= Ng) ? gy : gy - Ng, kz = (2 * gz <= Ng) ? gz : gz - Ng;
-        const double kk = sqrt((double)kx * kx + (double)ky * ky + (double)kz * kz);
-        if (kk == 0.0) continue;
+        const long k2 = (long)kx * kx + (long)ky * ky + (long)kz * kz;
+        if (k2 == 0) continue;
         const double wgt = (kx == 0 || 2 * kx == Ng) ? 1.0 : 2.0;
-        int bin = (int)floor(log(kk) / lkmax * nbins);
+        const float s = logf((float)k2) * hb, fl = floorf(s), fr = s - fl;
+        int bin = (int)fl;
+        if (!(fr > tol && fr < 1.0f - tol)) bin = (int)floor(log(sqrt((double)k2)) / lkmax * nbins);
         if (bin > nbins - 1) bin = nbins - 1;
         if (bin < 0) bin = 0;
         const double2 z = F[e];
         atomicAdd(&s_pow[bin], wgt * (z.x * z.x + z.y * z.y) * scale2);
         if (first) {
-            atomicAdd(&s_k[bin], wgt * kk);
+            atomicAdd(&s_k[bin], wgt * sqrt((double)k2));
             atomicAdd(&s_cnt[bin], (unsigned long long)wgt);
         }
     }
@@ -229,13 +365,37 @@ static int grid_of(long items, int nsm)
     return g < 1 ? 1 : (int)g;
 }
 
+// values of the normalised Legendre polynomials at the points x[0..n)
+static Line line_of(const double* x, int n)
+{
+    Line t{};
+    for (int a = 0; a < n; ++a) {
+        const double y = x[a];
+        const double p[4] = {1.0, y, 1.5 * y * y - 0.5, y * (2.5 * y * y - 1.5)};
+        for (int m = 0; m < n; ++m) t.P[a][m] = std::sqrt(2.0 * m + 1.0) * p[m];
+    }
+    return t;
+}
+
+// cnt [nbins][4]: samples per bin and weight class; the weights of the classes in
+// weight[4] (products of three 1D weights / 8, over the cells)
 template <typename T, int K>
-static cudaError_t pdf_k(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean, double* hist)
+static cudaError_t pdf_k(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean,
+                         unsigned long long* cnt, double* weight)
 {
     k_mean_rho<T, K><<<grid_of(L.ncell, L.nsm), 256, 0, L.st>>>(u, L.ncell, mean);
-    const long items = L.ncell * Dims<K>::nq;
-    k_density_pdf<T, K><<<grid_of(items, L.nsm), 256, sizeof(double) * nbins, L.st>>>(
-        u, L.ncell, L.r1, mean, lo, (hi - lo) / nbins, nbins, hist);
+    const double ds = (hi - lo) / nbins;
+    // error of the single-precision bin coordinate: the logarithm's (below 1e-6 of
+    // its size) over ds and the rounding of the coordinate
+    const double tol = 1e-6 * (2.0 + std::fabs(lo) + std::fabs(hi)) / ds + 1e-6 * nbins;
+    long g = (L.ncell + 127) / 128;
+    if (g > 16L * L.nsm) g = 16L * L.nsm;
+    const size_t sm = sizeof(unsigned int) * 4 * nbins;
+    k_density_pdf<T, K><<<(int)g, 128, sm, L.st>>>(u, L.ncell, line_of(L.r1.x, K + 1), mean, lo, ds,
+                                                   (float)std::min(tol, 1.0), nbins, cnt);
+    const double wo = L.r1.w[0], wi = K >= 2 ? L.r1.w[1] : wo;
+    for (int c = 0; c < 4; ++c)
+        weight[c] = std::pow(wi, c) * std::pow(wo, 3 - c) / 8.0 / (double)L.ncell;
     return cudaGetLastError();
 }
 
@@ -243,7 +403,7 @@ template <typename T, int K>
 static cudaError_t sfunc_k(const Launch& L, const T* u, int nbins, long npairs, unsigned long long seed, double* acc)
 {
     const double lmin = 1.0 / ((K + 1) * (double)L.N), lmax = 0.5;
-    k_structure<T, K><<<grid_of((long)nbins * npairs, L.nsm), 256, sizeof(double) * nbins, L.st>>>(
+    k_structure<T, K><<<grid_of((long)nbins * npairs, L.nsm), 256, 2 * sizeof(double) * nbins, L.st>>>(
         u, L.N, nbins, npairs, seed, lmin, lmax, acc);
     return cudaGetLastError();
 }
@@ -251,16 +411,19 @@ static cudaError_t sfunc_k(const Launch& L, const T* u, int nbins, long npairs, 
 template <typename T, int K>
 static cudaError_t sample_k(const Launch& L, const T* u, int d, double* out)
 {
-    const long Ng = (long)(K + 1) * L.N;
-    k_sample<T, K><<<grid_of(Ng * Ng * Ng, L.nsm), 256, 0, L.st>>>(u, L.N, d, out);
+    double x[4];
+    for (int a = 0; a <= K; ++a) x[a] = (2.0 * a + 1.0) / (K + 1) - 1.0;
+    long g = (L.ncell + 127) / 128;
+    if (g > 16L * L.nsm) g = 16L * L.nsm;
+    k_sample<T, K><<<(int)g, 128, 0, L.st>>>(u, L.N, d, line_of(x, K + 1), out);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_density_pdf(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean,
-                               double* hist)
+                               unsigned long long* cnt, double* weight)
 {
-    DG_DISPATCH(pdf_k, u, lo, hi, nbins, mean, hist);
+    DG_DISPATCH(pdf_k, u, lo, hi, nbins, mean, cnt, weight);
 }
 
 template <typename T>
@@ -286,7 +449,8 @@ cudaError_t launch_shell(const Launch& L, const void* F, int Ng, int nbins, doub
 }
 
 #define DG_ANALYSIS_INSTANTIATE(T)                                                                               \
-    template cudaError_t launch_density_pdf<T>(const Launch&, const T*, double, double, int, double*, double*); \
+    template cudaError_t launch_density_pdf<T>(const Launch&, const T*, double, double, int, double*,           \
+                                               unsigned long long*, double*);                                   \
     template cudaError_t launch_structure<T>(const Launch&, const T*, int, long, unsigned long long, double*);   \
     template cudaError_t launch_sample<T>(const Launch&, const T*, int, double*);
 DG_ANALYSIS_INSTANTIATE(float)
