@@ -70,15 +70,25 @@ __global__ void __launch_bounds__(256) k_force_axis(Rule1 r, int N, T* G)
 template <typename T, int K>
 struct ForceCfg {
     static constexpr int b = Dims<K>::b, n = K + 1, NP = sf::npair(K), CELLS = 64, NT = 3 * CELLS;
-    static constexpr int NPAIR = (kForceKM + 1) * kForceNK;  // largest number of (kx, ky) pairs
+    static constexpr int NG = kForceKM + 1, NPAIR = NG * kForceNK;  // largest numbers of kx and of (kx, ky)
+    static constexpr int RB = 4;                                    // rows whose sums are formed together
     static constexpr int LD = sf::padded<T>(3 * b);
-    static constexpr int oHz = 0;                                    // [pair][l][v] complex
-    static constexpr int oHy = oHz + NPAIR * n * 3 * 2;              // [group][pair (j, l)][v] complex
-    static constexpr int oOut = (oHy + (kForceKM + 1) * NP * 3 * 2 + 3) / 4 * 4;  // [64][3][b]
-    static constexpr int total = oOut + CELLS * LD;
+    // shared memory in elements of T, sized by the modes at hand (few of the possible
+    // ones in use: several blocks per SM)
+    int hz, hy, gx, out, total;
+    __host__ __device__ explicit ForceCfg(const ForceModes& fm)
+    {
+        hz = 0;                                  // [pair][l][v] complex
+        hy = hz + fm.npair * n * 3 * 2;          // [row][group][pair (j, l)][v] complex
+        gx = hy + RB * fm.ngroup * NP * 3 * 2;   // [group][i][re, im][cell]
+        out = (gx + fm.ngroup * n * 2 * CELLS + 3) / 4 * 4;  // [64][3][b]
+        total = out + CELLS * LD;
+    }
 };
 
-// block: rows iy0 .. iy0 + rpb - 1 of the plane iz = blockIdx.y
+// block: rows iy0 .. iy0 + rpb - 1 of the plane iz = blockIdx.y, RB of them at a time
+// (their sums over ky are short chains of dependent loads: several rows in flight
+// cover the latency), 64 cells at a time
 template <typename T, int K>
 __global__ void __launch_bounds__(192) k_force(const T* __restrict__ G, int N, int rpb, ForceModes fm,
                                                const int* __restrict__ modes, const double* __restrict__ amp,
@@ -88,19 +98,24 @@ __global__ void __launch_bounds__(192) k_force(const T* __restrict__ G, int N, i
     constexpr int b = C::b, n = C::n, NP = C::NP, NT = C::NT, LD = C::LD;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* sm = reinterpret_cast<T*>(smem_raw);
-    T* hz = sm + C::oHz;
-    T* hy = sm + C::oHy;
-    T* so = sm + C::oOut;
+    const C lay(fm);
+    T* hz = sm + lay.hz;
+    T* hy = sm + lay.hy;
+    T* gx = sm + lay.gx;
+    T* so = sm + lay.out;
+    const int HY = 2 * fm.ngroup * NP * 3;
+    __shared__ int s_mode[kForceModes], s_pair[C::NPAIR + 1], s_group[C::NG + 1];
     const int tid = threadIdx.x, iz = blockIdx.y;
-    const int* pairs = modes + kForcePairs;
-    const int* groups = modes + kForceGroups;
+    for (int e = tid; e < fm.nm; e += NT) s_mode[e] = modes[e];
+    for (int e = tid; e <= fm.npair; e += NT) s_pair[e] = e < fm.npair ? modes[kForcePairs + e] : fm.nm;
+    for (int e = tid; e <= fm.ngroup; e += NT) s_group[e] = e < fm.ngroup ? modes[kForceGroups + e] : fm.npair;
+    __syncthreads();
     const T* gz = G + (long)iz * kForceNK * n * 2;
     for (int e = tid; e < fm.npair * n * 3; e += NT) {
         const int p = e / (n * 3), l = (e / 3) % n, v = e % 3;
-        const int m0 = pairs[p], m1 = p + 1 < fm.npair ? pairs[p + 1] : fm.nm;
         T re = T(0), im = T(0);
-        for (int m = m0; m < m1; ++m) {
-            const T* g = gz + ((modes[m] >> 16) * n + l) * 2;
+        for (int m = s_pair[p]; m < s_pair[p + 1]; ++m) {
+            const T* g = gz + ((s_mode[m] >> 16) * n + l) * 2;
             const T ar = T(2.0 * amp[(m * 3 + v) * 2]), ai = T(2.0 * amp[(m * 3 + v) * 2 + 1]);
             re += ar * g[0] - ai * g[1];
             im += ar * g[1] + ai * g[0];
@@ -109,61 +124,73 @@ __global__ void __launch_bounds__(192) k_force(const T* __restrict__ G, int N, i
         hz[2 * e + 1] = im;
     }
     const int iy1 = min(N, (int)(blockIdx.x + 1) * rpb);
-    for (int iy = blockIdx.x * rpb; iy < iy1; ++iy) {
+    const int v = tid / C::CELLS, cl = tid % C::CELLS;
+    for (int y0 = blockIdx.x * rpb; y0 < iy1; y0 += C::RB) {
+        const int nr = min(C::RB, iy1 - y0);
         __syncthreads();
-        const T* gy = G + (long)iy * kForceNK * n * 2;
-        for (int e = tid; e < fm.ngroup * NP * 3; e += NT) {
-            const int g = e / (NP * 3), pr = (e / 3) % NP, v = e % 3;
+        const int per = fm.ngroup * NP * 3;
+        for (int e = tid; e < nr * per; e += NT) {
+            const int r = e / per, q = e - r * per, g = q / (NP * 3), pr = (q / 3) % NP, c = q % 3;
             // the pair (j, l) of index pr
             int j = 0, l = pr;
             while (l > K - j) l -= K - j + 1, ++j;
-            const int p0 = groups[g], p1 = g + 1 < fm.ngroup ? groups[g + 1] : fm.npair;
+            const T* gy = G + ((long)(y0 + r) * kForceNK * n + j) * 2;
             T re = T(0), im = T(0);
-            for (int p = p0; p < p1; ++p) {
-                const T* y = gy + (((modes[pairs[p]] >> 8) & 255) * n + j) * 2;
-                const T hr = hz[2 * ((p * n + l) * 3 + v)], hi = hz[2 * ((p * n + l) * 3 + v) + 1];
+            for (int p = s_group[g]; p < s_group[g + 1]; ++p) {
+                const T* y = gy + ((s_mode[s_pair[p]] >> 8) & 255) * n * 2;
+                const T hr = hz[2 * ((p * n + l) * 3 + c)], hi = hz[2 * ((p * n + l) * 3 + c) + 1];
                 re += y[0] * hr - y[1] * hi;
                 im += y[0] * hi + y[1] * hr;
             }
-            hy[2 * e] = re;
-            hy[2 * e + 1] = im;
+            hy[r * HY + 2 * q] = re;
+            hy[r * HY + 2 * q + 1] = im;
         }
-        const int v = tid / C::CELLS, cl = tid % C::CELLS;
-        T* row = ahat + ((long)iz * N + iy) * N * 3 * b;
         for (int x0 = 0; x0 < N; x0 += C::CELLS) {
-            __syncthreads();
-            const int ix = x0 + cl;
-            if (ix < N) {
-                T acc[b];
+            const int nc = min(C::CELLS, N - x0);
+            if (N > C::CELLS || y0 == (int)blockIdx.x * rpb) {
+                // the chunk's factors along x
+                __syncthreads();
+                for (int e = tid; e < fm.ngroup * C::CELLS; e += NT) {
+                    const int g = e / C::CELLS, c = e % C::CELLS;
+                    const int kx = s_mode[s_pair[s_group[g]]] & 255;
+                    if (c < nc) {
+                        const T* x = G + ((long)((x0 + c) * kForceNK + kx + kForceKM) * n) * 2;
 #pragma unroll
-                for (int l = 0; l < b; ++l) acc[l] = T(0);
-                for (int g = 0; g < fm.ngroup; ++g) {
-                    const int kx = modes[pairs[groups[g]]] & 255;
-                    const T* x = G + ((long)(ix * kForceNK + kx + kForceKM) * n) * 2;
-                    T xr[n], xi[n];
-#pragma unroll
-                    for (int i = 0; i < n; ++i) {
-                        xr[i] = __ldg(x + 2 * i);
-                        xi[i] = __ldg(x + 2 * i + 1);
+                        for (int i = 0; i < 2 * n; ++i) gx[(g * 2 * n + i) * C::CELLS + c] = __ldg(x + i);
                     }
-                    const T* H = hy + 2 * (g * NP * 3 + v);
-                    static_for<0, K + 1>([&](auto J) {
-                        constexpr int j = decltype(J)::value;
-                        static_for<0, K - j + 1>([&](auto L) {
-                            constexpr int l = decltype(L)::value;
-                            const T hr = H[sf::ip(K, j, l) * 6], hi = H[sf::ip(K, j, l) * 6 + 1];
-                            static_for<0, K - j - l + 1>([&](auto I) {
-                                constexpr int i = decltype(I)::value;
-                                acc[sf::im<K>(i, j, l)] += xr[i] * hr - xi[i] * hi;
+                }
+            }
+            for (int r = 0; r < nr; ++r) {
+                __syncthreads();
+                if (cl < nc) {
+                    T acc[b];
+#pragma unroll
+                    for (int l = 0; l < b; ++l) acc[l] = T(0);
+                    for (int g = 0; g < fm.ngroup; ++g) {
+                        T xr[n], xi[n];
+#pragma unroll
+                        for (int i = 0; i < n; ++i) {
+                            xr[i] = gx[(g * 2 * n + 2 * i) * C::CELLS + cl];
+                            xi[i] = gx[(g * 2 * n + 2 * i + 1) * C::CELLS + cl];
+                        }
+                        const T* H = hy + r * HY + 2 * (g * NP * 3 + v);
+                        static_for<0, K + 1>([&](auto J) {
+                            constexpr int j = decltype(J)::value;
+                            static_for<0, K - j + 1>([&](auto L) {
+                                constexpr int l = decltype(L)::value;
+                                const T hr = H[sf::ip(K, j, l) * 6], hi = H[sf::ip(K, j, l) * 6 + 1];
+                                static_for<0, K - j - l + 1>([&](auto I) {
+                                    constexpr int i = decltype(I)::value;
+                                    acc[sf::im<K>(i, j, l)] += xr[i] * hr - xi[i] * hi;
+                                });
                             });
                         });
-                    });
+                    }
+                    sf::st_row<T, b>(so + cl * LD + v * b, acc);
                 }
-                sf::st_row<T, b>(so + cl * LD + v * b, acc);
+                __syncthreads();
+                sf::tile_store<T, 3 * b, LD, NT>(ahat + ((long)iz * N + y0 + r) * N * 3 * b, so, x0, nc);
             }
-            __syncthreads();
-            const int nc = min(C::CELLS, N - x0);
-            sf::tile_store<T, 3 * b, LD, NT>(row, so, x0, nc);
         }
     }
 }

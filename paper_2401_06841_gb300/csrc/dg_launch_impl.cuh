@@ -73,7 +73,9 @@ static cudaError_t setup_k()
     cudaError_t e;
     if ((e = setup_tiles<T, K>()) != cudaSuccess) return e;
     e = cudaFuncSetAttribute(k_force<T, K>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(T) * ForceCfg<T, K>::total));
+                             (int)(sizeof(T) * ForceCfg<T, K>(ForceModes{kForceModes, ForceCfg<T, K>::NPAIR,
+                                                                         ForceCfg<T, K>::NG})
+                                                   .total));
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&Occ<T, K>::diag, k_diag<T, K>, NT, 0);
     return e;
@@ -188,13 +190,13 @@ template <typename T, int K>
 static cudaError_t force_k(const Launch& L, const ForceModes& fm, const int* modes, const double* amp, T* ahat)
 {
     using C = ForceCfg<T, K>;
-    if (fm.nm > kForceModes || fm.npair > C::NPAIR || fm.ngroup > kForceKM + 1) return cudaErrorInvalidValue;
+    if (fm.nm > kForceModes || fm.npair > C::NPAIR || fm.ngroup > C::NG) return cudaErrorInvalidValue;
     // rows of a plane per block: enough to share the plane's sums, few enough for
-    // about four blocks per multiprocessor
-    long rpb = (long)L.N * L.N / (4L * L.nsm);
+    // about eight blocks per multiprocessor
+    long rpb = (long)L.N * L.N / (8L * L.nsm);
     rpb = rpb < 1 ? 1 : (rpb > L.N ? L.N : rpb);
     const dim3 g((unsigned)((L.N + rpb - 1) / rpb), (unsigned)L.N);
-    k_force<T, K><<<g, C::NT, sizeof(T) * C::total, L.st>>>(static_cast<const T*>(L.gtab), L.N, (int)rpb, fm, modes,
+    k_force<T, K><<<g, C::NT, sizeof(T) * C(fm).total, L.st>>>(static_cast<const T*>(L.gtab), L.N, (int)rpb, fm, modes,
                                                           amp, ahat);
     return cudaGetLastError();
 }
