@@ -35,102 +35,62 @@ struct AdiGas {
 
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
 
-// Rusanov flux along Dd from primitive face states W = (rho, v_x, v_y, v_z, p - c0 rho):
-// 1/2 (F(U_L) + F(U_R)) - 1/2 lambda (U_R - U_L), lambda = max(|v_n| + c)
-template <typename T, int Dd>
+// Face fluxes along the normal (component 1) from primitive face states W = (rho, v_n,
+// v_t1, v_t2, p - c0 rho).  Rusanov, (F_L + F_R)/2 - lambda (U_R - U_L)/2 with lambda =
+// max(|v_n| + c): the momentum carried by q_L = rho_L (v_n,L + lambda)/2 and q_R = rho_R
+// (v_n,R - lambda)/2, mass and energy from the differences of rho and e (slow flows would
+// lose them between terms of the size rho c)
+template <typename T>
 __device__ __forceinline__ void adi_rusanov(const AdiGas<T>& G, const T* WL, const T* WR, T* F)
 {
-    const T g1 = G.g1, gamma = G.gamma;
-    T UL[5], UR[5], FL[5], FR[5], ls[2];
-    const T* W[2] = {WL, WR};
-    T* U[2] = {UL, UR};
-    T* Fx[2] = {FL, FR};
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const T* w = W[s];
-        const T rho = w[0], vn = w[1 + Dd], p = w[4] + G.c0 * rho;  // w[4]: the pressure deviation
-        U[s][0] = rho;
-        U[s][1] = rho * w[1];
-        U[s][2] = rho * w[2];
-        U[s][3] = rho * w[3];
-        U[s][4] = w[4] / g1 + T(0.5) * rho * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-        Fx[s][0] = U[s][1 + Dd];
-        Fx[s][1] = U[s][1] * vn;
-        Fx[s][2] = U[s][2] * vn;
-        Fx[s][3] = U[s][3] * vn;
-        Fx[s][1 + Dd] += p;
-        Fx[s][4] = (U[s][4] + p) * vn;
-        ls[s] = fabs(vn) + sqrt(gamma * p / rho);
-    }
+    const T pL = WL[4] + G.c0 * WL[0], pR = WR[4] + G.c0 * WR[0];  // W[4]: the pressure deviation
+    const T aL = fabs(WL[1]) + fast_sqrt<T>(G.gamma * pL * rcp<T>(WL[0]));
+    const T aR = fabs(WR[1]) + fast_sqrt<T>(G.gamma * pR * rcp<T>(WR[0]));
     // the larger of the two (a NaN of the right state propagates, as in the oracle)
-    const T lam = ls[0] > ls[1] ? ls[0] : ls[1];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) F[v] = T(0.5) * (FL[v] + FR[v]) - T(0.5) * lam * (UR[v] - UL[v]);
+    const T hl = T(0.5) * (aL > aR ? aL : aR);
+    const T hL = T(0.5) * WL[1], hR = T(0.5) * WR[1];
+    const T mL = WL[0] * hL, mR = WR[0] * hR;
+    const T qL = mL + hl * WL[0], qR = mR - hl * WR[0];
+    const T eL = WL[4] * G.ig1 + T(0.5) * WL[0] * (WL[1] * WL[1] + WL[2] * WL[2] + WL[3] * WL[3]);
+    const T eR = WR[4] * G.ig1 + T(0.5) * WR[0] * (WR[1] * WR[1] + WR[2] * WR[2] + WR[3] * WR[3]);
+    F[0] = (mL + mR) - hl * (WR[0] - WL[0]);
+    F[1] = T(0.5) * (pL + pR) + (qL * WL[1] + qR * WR[1]);
+    F[2] = qL * WL[2] + qR * WR[2];
+    F[3] = qL * WL[3] + qR * WR[3];
+    F[4] = ((eL + pL) * hL + (eR + pR) * hR) - hl * (eR - eL);
 }
 
-// HLLC flux along Dd from primitive face states (the contact wave restored in
-// the two-wave model): Davis bounds S_L = min(u - c), S_R = max(u + c) over the
-// two states, the contact speed S* from the pressures and the mass fluxes
-// relative to the bounds, star states U*_K = rho_K (S_K - u_K)/(S_K - S*)
-// (1, S* along Dd, the tangential velocities, E_K/rho_K + (S* - u_K)(S* +
-// p_K/(rho_K (S_K - u_K)))), and the flux of the region x/t = 0 falls in
-template <typename T, int Dd>
+// HLLC (the contact wave restored in the two-wave model): Davis bounds S_L = min(u - c),
+// S_R = max(u + c) over the two states, the contact speed S* from the pressures and the
+// mass fluxes q_K = rho_K (S_K - u_K) relative to the bounds; behind the contact, on the
+// side K that x/t = 0 lies on, rho* = q_K/(S_K - S*), p* = p_K + q_K (S* - u_K), E* =
+// (E_K (S_K - u_K) - p_K u_K + p* S*)/(S_K - S*), and the flux is that of this state at
+// the normal velocity S* (outside the bounds: of the state K itself)
+template <typename T>
 __device__ __forceinline__ void adi_hllc(const AdiGas<T>& G, const T* WL, const T* WR, T* F)
 {
-    const T g1 = G.g1, gamma = G.gamma;
-    T U[2][5], Fx[2][5], c[2], un[2], pp[2];
-    const T* W[2] = {WL, WR};
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        const T* w = W[s];
-        const T rho = w[0], p = w[4] + G.c0 * rho;  // w[4]: the pressure deviation
-        pp[s] = p;
-        un[s] = w[1 + Dd];
-        U[s][0] = rho;
-        U[s][1] = rho * w[1];
-        U[s][2] = rho * w[2];
-        U[s][3] = rho * w[3];
-        U[s][4] = w[4] / g1 + T(0.5) * rho * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
-        Fx[s][0] = U[s][1 + Dd];
-        Fx[s][1] = U[s][1] * un[s];
-        Fx[s][2] = U[s][2] * un[s];
-        Fx[s][3] = U[s][3] * un[s];
-        Fx[s][1 + Dd] += p;
-        Fx[s][4] = (U[s][4] + p) * un[s];
-        c[s] = sqrt(gamma * p / rho);
-    }
-    const T a0 = un[0] - c[0], a1 = un[1] - c[1], b0 = un[0] + c[0], b1 = un[1] + c[1];
+    const T pL = WL[4] + G.c0 * WL[0], pR = WR[4] + G.c0 * WR[0];
+    const T cL = fast_sqrt<T>(G.gamma * pL * rcp<T>(WL[0])), cR = fast_sqrt<T>(G.gamma * pR * rcp<T>(WR[0]));
+    const T a0 = WL[1] - cL, a1 = WR[1] - cR, b0 = WL[1] + cL, b1 = WR[1] + cR;
     const T SL = a0 < a1 ? a0 : a1, SR = b0 > b1 ? b0 : b1;
-    if (SL >= T(0)) {
+    const T qL = WL[0] * (SL - WL[1]), qR = WR[0] * (SR - WR[1]);
+    const T Ss = (pR - pL + WL[1] * qL - WR[1] * qR) * rcp<T>(qL - qR);
+    // selects keep everything in registers
+    const bool outer = SL >= T(0) || SR <= T(0);
+    const bool lft = SL >= T(0) || (!(SR <= T(0)) && Ss >= T(0));
+    const T SK = lft ? SL : SR, qK = lft ? qL : qR, pK = lft ? pL : pR;
+    T w[5];
 #pragma unroll
-        for (int v = 0; v < 5; ++v) F[v] = Fx[0][v];
-        return;
-    }
-    if (SR <= T(0)) {
-#pragma unroll
-        for (int v = 0; v < 5; ++v) F[v] = Fx[1][v];
-        return;
-    }
-    const T qL = WL[0] * (SL - un[0]), qR = WR[0] * (SR - un[1]);
-    const T Ss = (pp[1] - pp[0] + un[0] * qL - un[1] * qR) / (qL - qR);
-    // the side of the contact x/t = 0 lies on (selects keep everything in registers)
-    const bool lft = Ss >= T(0);
-    const T SK = lft ? SL : SR, qK = lft ? qL : qR, uK = lft ? un[0] : un[1], pK = lft ? pp[0] : pp[1];
-    T wK[5], UK[5], FK[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-        wK[v] = lft ? WL[v] : WR[v];
-        UK[v] = lft ? U[0][v] : U[1][v];
-        FK[v] = lft ? Fx[0][v] : Fx[1][v];
-    }
-    const T f = qK / (SK - Ss);
-    T Us[5];
-    Us[0] = f;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) Us[1 + i] = f * (i == Dd ? Ss : wK[1 + i]);
-    Us[4] = f * (UK[4] / wK[0] + (Ss - uK) * (Ss + pK / qK));
-#pragma unroll
-    for (int v = 0; v < 5; ++v) F[v] = FK[v] + SK * (Us[v] - UK[v]);
+    for (int v = 0; v < 5; ++v) w[v] = lft ? WL[v] : WR[v];
+    const T e = w[4] * G.ig1 + T(0.5) * w[0] * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]);
+    const T r = rcp<T>(SK - Ss);
+    const T us = outer ? w[1] : Ss, ps = outer ? pK : pK + qK * (Ss - w[1]), rs = outer ? w[0] : qK * r;
+    const T es = outer ? e : (e * (SK - w[1]) - pK * w[1] + ps * Ss) * r;
+    F[0] = rs * us;
+    F[1] = F[0] * us + ps;
+    F[2] = F[0] * w[2];
+    F[3] = F[0] * w[3];
+    F[4] = (es + ps) * us;
 }
 
 // smallest t in [0, 1] with p(ub + t d) = eps (p(ub) > eps > p(ub + d)): the

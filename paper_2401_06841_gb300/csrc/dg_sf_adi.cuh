@@ -293,7 +293,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
                         // viscous pressure (Sec. 3.1) with the local sound speed, A = -div v
                         const T Ad = (vx[i] * gx[i] + vy[i] * gy[i] + vz[i] * gz[i] - dm[i]) * (ir * a.two_h);
                         const T ra = rho * Ad;
-                        T Pi = ra * (a.a2 * Ad + a.bh * sqrt(a.gas.gamma * p * ir));
+                        T Pi = ra * (a.a2 * Ad + a.bh * fast_sqrt<T>(a.gas.gamma * p * ir));
                         if (cap >= T(0)) {
                             const T Pm = ra * cap;
                             Pi = Pi > Pm ? Pm : Pi;
@@ -384,20 +384,22 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
 #pragma unroll
                     for (int i = 0; i < n; ++i)
                         x[i] = f[0][i] * a.gas.cres +
-                               T(0.5) * (f[1][i] * f[1][i] + f[2][i] * f[2][i] + f[3][i] * f[3][i]) / f[0][i];
+                               T(0.5) * (f[1][i] * f[1][i] + f[2][i] * f[2][i] + f[3][i] * f[3][i]) * rcp<T>(f[0][i]);
                     line_proj<T, K, K>(x, t);
                     row_acc<T, K>(t, wj, Vx);
                 } else {
 #pragma unroll
                     for (int i = 0; i < n; ++i) {
                         const T rho = f[0][i], ir = rcp<T>(rho);
-                        const T pd = adi_pdev<T>(a.gas, rho, f[1][i], f[2][i], f[3][i], f[NF - 1][i]);
-                        f[1][i] *= ir;
-                        f[2][i] *= ir;
-                        f[3][i] *= ir;
-                        f[NF - 1][i] = pd;  // projected: p - c0 rho
+                        const T vx = f[1][i] * ir, vy = f[2][i] * ir, vz = f[3][i] * ir;
+                        // projected: p - c0 rho
+                        const T pd = g1 * (f[NF - 1][i] - T(0.5) * (f[1][i] * vx + f[2][i] * vy + f[3][i] * vz));
+                        f[1][i] = vx;
+                        f[2][i] = vy;
+                        f[3][i] = vz;
+                        f[NF - 1][i] = pd;
                         if (MODE == SFA_PROJECT && a.dtf && valid) {
-                            const T cs = sqrt(a.gas.gamma * (pd + c0g * rho) * ir);
+                            const T cs = fast_sqrt<T>(a.gas.gamma * (pd + c0g * rho) * ir);
                             const T sp = fabs(f[1][i]) + fabs(f[2][i]) + fabs(f[3][i]) + T(3) * cs;
                             smax = sp > smax ? sp : smax;
                         }
@@ -679,9 +681,9 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 5 : K == 2 ? 3
                 const T WR[5] = {W[5][i], W[6][i], W[7][i], W[8][i], W[9][i]};
                 T F[5];
                 if constexpr (RS == 2)
-                    adi_hllc<T, 0>(a.gas, WL, WR, F);
+                    adi_hllc<T>(a.gas, WL, WR, F);
                 else
-                    adi_rusanov<T, 0>(a.gas, WL, WR, F);
+                    adi_rusanov<T>(a.gas, WL, WR, F);
 #pragma unroll
                 for (int v = 0; v < 5; ++v) Fl[v][i] = F[v];
             }
