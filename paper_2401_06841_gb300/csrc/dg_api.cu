@@ -12,6 +12,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 #include <memory>
 #include <new>
@@ -223,6 +224,22 @@ struct Driver {
     uint64_t rng = 0;
     bool have_spare = false;
     double spare = 0;
+    // the modes and amplitudes of the present x as the forcing projection takes them
+    struct Pack {
+        ForceModes fm{};
+        std::vector<int> ints;
+        std::vector<double> amp;
+    } pack;
+    bool packed = false;
+    // the next update, made while the device works on a step
+    struct Next {
+        bool ready = false;
+        double x[kMaxModes][3][2];
+        uint64_t rng;
+        bool have_spare;
+        double spare;
+        Pack pack;
+    } nx;
 
     // SplitMix64 (Steele, Lea & Flood 2014)
     uint64_t next()
@@ -281,6 +298,79 @@ struct Driver {
         t_off = F.t_off;
         on = F.on != 0;
         dirty = true;
+        packed = nx.ready = false;
+    }
+    void save(dg_meta& m) const
+    {
+        m.forcing_on = on ? 1 : 0;
+        m.forcing_dirty = dirty ? 1 : 0;
+        m.t_next = t_next;
+        m.rng = rng;
+        m.have_spare = have_spare ? 1 : 0;
+        m.spare = spare;
+        m.nmodes = nm;
+        std::memcpy(m.x, x, sizeof(double) * 6 * nm);
+    }
+    // (the amplitudes are projected again before the next step)
+    void restore(const dg_meta& m)
+    {
+        on = m.forcing_on != 0;
+        t_next = m.t_next;
+        rng = m.rng;
+        have_spare = m.have_spare != 0;
+        spare = m.spare;
+        std::memcpy(x, m.x, sizeof(double) * 6 * m.nmodes);
+        dirty = on;
+        packed = nx.ready = false;
+    }
+    // the OU updates due at time t
+    void update(double t)
+    {
+        while (t >= t_next) {
+            if (nx.ready) {
+                std::memcpy(x, nx.x, sizeof(double) * 6 * nm);
+                rng = nx.rng;
+                have_spare = nx.have_spare;
+                spare = nx.spare;
+                std::swap(pack, nx.pack);
+                packed = true;
+                nx.ready = false;
+            } else {
+                advance();
+                packed = false;
+            }
+            t_next += dtd;
+            dirty = true;
+        }
+    }
+    // the update after the present one into nx (a few hundred normal deviates and
+    // the packing of the modes: ~20 us that would otherwise lie between two steps)
+    void ahead()
+    {
+        if (!on || nx.ready) return;
+        double x0[kMaxModes][3][2];
+        std::memcpy(x0, x, sizeof(double) * 6 * nm);
+        const uint64_t rng0 = rng;
+        const bool have0 = have_spare;
+        const double spare0 = spare;
+        advance();
+        make_pack(nx.pack);
+        std::memcpy(nx.x, x, sizeof(double) * 6 * nm);
+        nx.rng = rng;
+        nx.have_spare = have_spare;
+        nx.spare = spare;
+        nx.ready = true;
+        std::memcpy(x, x0, sizeof(double) * 6 * nm);
+        rng = rng0;
+        have_spare = have0;
+        spare = spare0;
+    }
+    void make_pack(Pack& p) const;
+    const Pack& packs()
+    {
+        if (!packed) make_pack(pack);
+        packed = true;
+        return pack;
     }
     void advance()
     {
@@ -348,6 +438,66 @@ ForceModes pack_modes(int nm, const int* kvec, const double* amp, std::vector<in
     return fm;
 }
 
+void Driver::make_pack(Pack& p) const
+{
+    std::vector<double> a;
+    std::vector<int> k;
+    amplitudes(a, k);
+    p.fm = pack_modes(nm, k.data(), a.data(), p.ints, p.amp);
+}
+
+// Pinned host memory of a context, for what dg_step and dg_adi_step exchange with
+// the device between two steps: a copy from or to pageable memory blocks the host
+// for ~5-10 us each.  One step's transfers are complete before the next one's begin
+// (the host waits for the read-back).
+struct Mail {
+    Ctl in, back;
+    int kvec[3 * kMaxModes];
+    double amp[6 * kMaxModes];
+};
+// bytes of Ctl that the host sets before an attempt, and that it reads back
+constexpr size_t kCtlIn = offsetof(Ctl, dt), kCtlBack = kCtlIn + sizeof(double);
+
+struct MailBox {
+    Mail* m = nullptr;
+    cudaEvent_t done = nullptr;  // the read-back has arrived
+    cudaError_t open()
+    {
+        cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(&m), sizeof(Mail));
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done, cudaEventDisableTiming);
+        return e;
+    }
+    // what an attempt starts from: status, sums and bounds cleared
+    cudaError_t post(Ctl* ctl, double dt_scale, double fixed_dt, cudaStream_t st)
+    {
+        std::memset(static_cast<void*>(&m->in), 0, kCtlIn);
+        m->in.dt_scale = dt_scale;
+        m->in.fixed_dt = fixed_dt;
+        return cudaMemcpyAsync(ctl, &m->in, kCtlIn, cudaMemcpyHostToDevice, st);
+    }
+    cudaError_t request(const Ctl* ctl, cudaStream_t st)
+    {
+        const cudaError_t e = cudaMemcpyAsync(&m->back, ctl, kCtlBack, cudaMemcpyDeviceToHost, st);
+        return e != cudaSuccess ? e : cudaEventRecord(done, st);
+    }
+    cudaError_t wait() { return cudaEventSynchronize(done); }
+    cudaError_t modes(const Driver::Pack& p, int* d_kvec, double* d_amp, cudaStream_t st)
+    {
+        std::memcpy(m->kvec, p.ints.data(), sizeof(int) * p.ints.size());
+        std::memcpy(m->amp, p.amp.data(), sizeof(double) * p.amp.size());
+        const cudaError_t e =
+            cudaMemcpyAsync(d_kvec, m->kvec, sizeof(int) * p.ints.size(), cudaMemcpyHostToDevice, st);
+        return e != cudaSuccess
+                   ? e
+                   : cudaMemcpyAsync(d_amp, m->amp, sizeof(double) * p.amp.size(), cudaMemcpyHostToDevice, st);
+    }
+    ~MailBox()
+    {
+        if (done) cudaEventDestroy(done);
+        if (m) cudaFreeHost(m);
+    }
+};
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 }  // namespace
@@ -407,6 +557,7 @@ struct dg_ctx {
     void* ttab = nullptr;
     int* d_kvec = nullptr;
     double* d_amp = nullptr;
+    MailBox mail;
     void* gtab = nullptr;  // forcing: 1D factors (of the mesh and the rule: built by the first projection)
     bool gtab_ready = false;
     double* ana = nullptr; // turbulence statistics accumulators
@@ -634,19 +785,20 @@ void drop_carry(dg_ctx* c)
     if (c) c->carry = false;
 }
 
-// the launches of a projection, a right-hand side or a stage (with F_NEXTPROJ the
-// projection of its output: a launch of its own on the sum-factorised kernels, in
-// the fused kernel's epilogue otherwise)
+cudaError_t learned_infer(dg_ctx* c, const void* u, float* nu);
+
+// the launches of a projection, a right-hand side or a stage
 cudaError_t tile(dg_ctx* c, const TileLaunch& t)
 {
     const Launch L = make_launch(c);
-    auto go = [&](const TileLaunch& x) {
-        Timed tm(c, x.mode == TM_PROJECT ? KIND_PROJECT : KIND_RHS);
-        return (c->prec == DG_PREC_F64) ? launch_tile<double>(L, x) : launch_tile<float>(L, x);
-    };
-    const cudaError_t e = go(t);
-    if (e != cudaSuccess || !c->sf || t.mode == TM_PROJECT || t.mode == TM_RHS || !(t.flags & F_NEXTPROJ)) return e;
-    // the projection of the stage's output, with the CFL bound
+    Timed tm(c, t.mode == TM_PROJECT ? KIND_PROJECT : KIND_RHS);
+    return (c->prec == DG_PREC_F64) ? launch_tile<double>(L, t) : launch_tile<float>(L, t);
+}
+
+// sum-factorised kernels: the projection of the last stage's output for the next
+// step, with the CFL bound (and, fused_infer, the next step's coefficient from it)
+cudaError_t next_projection(dg_ctx* c, const TileLaunch& t)
+{
     TileLaunch p{};
     p.mode = TM_PROJECT;
     p.u_in = t.out;
@@ -656,18 +808,21 @@ cudaError_t tile(dg_ctx* c, const TileLaunch& t)
     p.flags = t.flags & (F_FORCE | F_DT);
     p.abar_out = t.abar_out;
     p.trouble = t.trouble;
-    return go(p);
+    const cudaError_t e = tile(c, p);
+    return e != cudaSuccess || !t.nu_next ? e : learned_infer(c, t.out, t.nu_next);
 }
 
-// projection of u into vhat (+ forcing sums into abar slot, + CFL dt)
-cudaError_t project(dg_ctx* c, const void* u, void* vhat, const void* ahat, bool dt_flag, int abar_out)
+// projection of u into vhat (+ forcing sums into abar slot, + CFL dt, + |v|)
+cudaError_t project(dg_ctx* c, const void* u, void* vhat, const void* ahat, bool dt_flag, int abar_out,
+                    void* vabs = nullptr)
 {
     TileLaunch t{};
     t.mode = 0;
     t.u_in = u;
     t.vh_out = vhat;
     t.ahat = ahat;
-    t.flags = (ahat ? F_FORCE : 0) | (dt_flag ? F_DT : 0);
+    t.flags = (ahat ? F_FORCE : 0) | (dt_flag ? F_DT : 0) | (vabs ? F_VABS : 0);
+    t.vabs_out = vabs;
     t.abar_out = abar_out;
     return tile(c, t);
 }
@@ -740,13 +895,12 @@ cudaError_t learned_nu(dg_ctx* c, const void* u)
     return learned_infer(c, u, c->nu_cell);
 }
 
-// the packed modes and amplitudes to the device, then their projection into ahat
-// (the host buffers must outlive the copies)
-cudaError_t force_project(dg_ctx* c, const ForceModes& fm, const std::vector<int>& ints, const std::vector<double>& amp)
+// the packed modes and amplitudes to the device (through the mailbox, whose earlier
+// copies have run), then their projection into ahat
+cudaError_t force_project(dg_ctx* c, const Driver::Pack& p)
 {
-    cudaError_t e;
-    if ((e = cudaMemcpyAsync(c->d_kvec, ints.data(), sizeof(int) * ints.size(), cudaMemcpyHostToDevice, c->st))) return e;
-    if ((e = cudaMemcpyAsync(c->d_amp, amp.data(), sizeof(double) * amp.size(), cudaMemcpyHostToDevice, c->st))) return e;
+    cudaError_t e = c->mail.modes(p, c->d_kvec, c->d_amp, c->st);
+    if (e != cudaSuccess) return e;
     const Launch L = make_launch(c);
     if (!c->gtab_ready) {
         Timed tm(c, KIND_FORCE);
@@ -754,22 +908,14 @@ cudaError_t force_project(dg_ctx* c, const ForceModes& fm, const std::vector<int
         c->gtab_ready = true;
     }
     Timed tm(c, KIND_FORCE);
-    return c->prec == DG_PREC_F64 ? launch_force<double>(L, fm, c->d_kvec, c->d_amp, (double*)c->ahat)
-                                  : launch_force<float>(L, fm, c->d_kvec, c->d_amp, (float*)c->ahat);
+    return c->prec == DG_PREC_F64 ? launch_force<double>(L, p.fm, c->d_kvec, c->d_amp, (double*)c->ahat)
+                                  : launch_force<float>(L, p.fm, c->d_kvec, c->d_amp, (float*)c->ahat);
 }
 
 int upload_forcing(dg_ctx* ctx)
 {
-    std::vector<double> amp;
-    std::vector<int> kv;
-    ctx->drv.amplitudes(amp, kv);
     if (ctx->drv.nm == 0) return DG_OK;
-    std::vector<int> ints;
-    std::vector<double> pamp;
-    const ForceModes fm = pack_modes(ctx->drv.nm, kv.data(), amp.data(), ints, pamp);
-    CK(force_project(ctx, fm, ints, pamp));
-    // the host buffers must stay valid until the copies ran
-    CK(cudaStreamSynchronize(ctx->st));
+    CK(force_project(ctx, ctx->drv.packs()));
     ctx->forcing_active = true;
     return DG_OK;
 }
@@ -912,7 +1058,8 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
         const double hp = ctx->h / (order + 1);
         c0.dt_diff = nu->diffusion > 0.0 ? ctx->cfl * hp * hp / (2.0 * nu->diffusion) : 0.0;
     }
-    e = cudaMemcpyAsync(ctx->ctl, &c0, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->st);
+    e = ctx->mail.open();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->ctl, &c0, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->st);
     if (e == cudaSuccess) {
         if (ctx->prec == DG_PREC_F64) {
             e = cudaMemcpyAsync(ctx->tab, t.data(), sizeof(double) * t.size(), cudaMemcpyHostToDevice, ctx->st);
@@ -982,8 +1129,8 @@ int dg_rhs(dg_ctx* ctx, const void* u_in, const void* ahat, void* dudt, double d
     if (!u_in || !dudt) return fail(ctx, DG_EINVAL, "dg_rhs: null buffer");
     const bool learned = ctx->nu.mode == DG_AV_LEARNED;
     if (learned && !ctx->weights_set) return fail(ctx, DG_ESTATE, "dg_rhs: learned mode needs dg_set_av_weights");
-    if (learned) CK(learned_nu(ctx, u_in));
-    CK(project(ctx, u_in, vh_buf(ctx, 0), ahat, false, 0));
+    CK(project(ctx, u_in, vh_buf(ctx, 0), ahat, false, 0, learned ? ctx->vabs : nullptr));
+    if (learned) CK(learned_infer(ctx, u_in, ctx->nu_cell));
     TileLaunch t{};
     t.nu = learned ? ctx->nu_cell : nullptr;
     t.mode = 1;
@@ -1044,10 +1191,9 @@ int dg_forcing_from_modes(dg_ctx* ctx, int nmodes, const int32_t* kvec, const do
     int kmaxc = 0;
     for (int i = 0; i < 3 * nmodes; ++i) kmaxc = std::max(kmaxc, std::abs((int)kvec[i]));
     if (kmaxc > 8) return fail(ctx, DG_EINVAL, "dg_forcing_from_modes: |k_d| > 8");
-    std::vector<int> ints;
-    std::vector<double> pamp;
-    const ForceModes fm = pack_modes(nmodes, kvec, amp, ints, pamp);
-    CK(force_project(ctx, fm, ints, pamp));
+    Driver::Pack p;
+    p.fm = pack_modes(nmodes, kvec, amp, p.ints, p.amp);
+    CK(force_project(ctx, p));
     CK(cudaStreamSynchronize(ctx->st));
     ctx->drv.on = false;
     ctx->forcing_active = true;
@@ -1070,11 +1216,7 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
             CK(cudaMemsetAsync(ctx->ahat, 0, vec_bytes(ctx), ctx->st));
         }
         if (ctx->drv.on) {
-            while (ctx->t >= ctx->drv.t_next) {
-                ctx->drv.advance();
-                ctx->drv.t_next += ctx->drv.dtd;
-                ctx->drv.dirty = true;
-            }
+            ctx->drv.update(ctx->t);
             if (ctx->drv.dirty) {
                 ctx->carry = false;  // new a_h: the forcing sums change
                 int rc = upload_forcing(ctx);
@@ -1089,7 +1231,7 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
         const int in2[2] = {A, B}, out2[2] = {B, C};
         const int* in = ctx->rk == 2 ? in2 : in3;
         const int* out = ctx->rk == 2 ? out2 : out3;
-        bool ok = false;
+        bool ok = false, carried = false;
         double dt = 0.0;
         unsigned int status = 0u;
         const bool learned = ctx->nu.mode == DG_AV_LEARNED;
@@ -1112,16 +1254,11 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
         int halvings = 0, attempts = 0;
         for (int retry = 0; retry < max_attempts && halvings <= max_halvings && !ok; ++retry) {
             attempts = retry + 1;
-            struct {
-                double dt_scale, fixed_dt;
-            } hs = {1.0 / (double)(1 << halvings), fixed_dt};
-            CK(cudaMemcpyAsync(&ctx->ctl->dt_scale, &hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->st));
-            unsigned int zero = 0u;
-            CK(cudaMemcpyAsync(&ctx->ctl->status, &zero, sizeof(zero), cudaMemcpyHostToDevice, ctx->st));
+            CK(ctx->mail.post(ctx->ctl, 1.0 / (double)(1 << halvings), fixed_dt, ctx->st));
             // stage 1 needs the projection of u^n (+ its wave-speed bound): carried
-            // over from the last stage of the previous step, else a projection
-            // launch; later stages get theirs from the previous stage's epilogue
-            // (double-buffered vhat / abar slots, alternating from slot pb)
+            // over from the end of the previous step, else a projection launch; for
+            // the later stages see below (double-buffered vhat / abar slots,
+            // alternating from slot pb)
             const bool use_carry = retry == 0 && ctx->carry;
             ctx->carry = false;
             // learned mode: the coefficient once per step, cached for all stages; the
@@ -1130,13 +1267,18 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
             if (learned) {
                 if (use_carry && fused)
                     std::swap(ctx->nu_cell, ctx->nu_next);
-                else
-                    CK(use_carry ? learned_infer(ctx, ctx->reg[A], ctx->nu_cell) : learned_nu(ctx, ctx->reg[A]));
+                else if (use_carry)
+                    CK(learned_infer(ctx, ctx->reg[A], ctx->nu_cell));
             }
-            if (!use_carry) CK(project(ctx, ctx->reg[A], vh_buf(ctx, pb), force ? ctx->ahat : nullptr, true, pb));
+            if (!use_carry) {
+                CK(project(ctx, ctx->reg[A], vh_buf(ctx, pb), force ? ctx->ahat : nullptr, true, pb,
+                           learned ? ctx->vabs : nullptr));
+                if (learned) CK(learned_infer(ctx, ctx->reg[A], ctx->nu_cell));
+            }
+            TileLaunch t{};
             for (int s = 0; s < ctx->rk; ++s) {
                 const bool last = s + 1 == ctx->rk;
-                TileLaunch t{};
+                t = TileLaunch{};
                 t.nu = learned ? ctx->nu_cell : nullptr;
                 t.mode = (learned && last) ? 3 : 2;
                 t.nu_next = (learned && last && fused) ? ctx->nu_next : nullptr;
@@ -1149,31 +1291,39 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
                 t.vh_out = vh_buf(ctx, (pb + s + 1) & 1);
                 t.ahat = force ? ctx->ahat : nullptr;
                 rk_weights(ctx->rk, s, ctx->prec != DG_PREC_F64, t.rk_a, t.rk_b);
-                // every stage projects its output; the last one for the next step,
-                // with the CFL bound (and |v| in learned mode).  On the sum-factorised
-                // kernels the stages after the first project their own input in the
-                // volume kernel instead (driven: with the forcing sums), so only the
-                // last stage's output gets a projection launch
-                const bool fold = ctx->sf;
-                t.flags = (force ? F_FORCE : 0) | ((fold && !last) ? 0 : F_NEXTPROJ) | (last ? F_DT : 0) |
-                          ((fold && s > 0) ? F_SELFPROJ : 0);
+                // every stage of the fused kernel projects its output; the last one for
+                // the next step, with the CFL bound (and |v| in learned mode).  On the
+                // sum-factorised kernels the stages after the first project their own
+                // input in the volume kernel instead (driven: with the forcing sums), and
+                // the last stage's output gets a projection launch
+                t.flags = (force ? F_FORCE : 0) | (ctx->sf ? 0 : F_NEXTPROJ) | (last ? F_DT : 0) |
+                          ((ctx->sf && s > 0) ? F_SELFPROJ : 0);
                 t.abar_in = (pb + s) & 1;
                 t.abar_out = (pb + s + 1) & 1;
                 t.trouble = marks;
                 CK(tile(ctx, t));
-                // fused_infer on the sum-factorised kernels: the next step's coefficient
-                // from the |v| projection the stage has just left
-                if (ctx->sf && t.nu_next) CK(learned_infer(ctx, t.out, ctx->nu_next));
             }
-            struct {
-                unsigned int status;
-                double dt;
-            } back{};
-            CK(cudaMemcpyAsync(&back.status, &ctx->ctl->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->st));
-            CK(cudaMemcpyAsync(&back.dt, &ctx->ctl->dt, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-            CK(cudaStreamSynchronize(ctx->st));
-            status = back.status;
-            dt = back.dt;
+            // The read-back goes before the projection for the next step where that
+            // cannot change the status, so that the host's turn (~15 us from the end of
+            // the read-back to the next launch) passes while it runs.  The projection is
+            // left out where the next step of this call makes another because it starts
+            // with an update of the driving; if that was foreseen wrongly, it is made
+            // after the wait.
+            const bool next = ctx->sf;
+            const bool defer = next && !repeat && !learned && st + 1 < nsteps && ctx->drv.on &&
+                               ctx->t + ctx->dt_last >= ctx->drv.t_next;
+            if (next && repeat) CK(next_projection(ctx, t));
+            CK(ctx->mail.request(ctx->ctl, ctx->st));
+            if (next && !repeat && !defer) CK(next_projection(ctx, t));
+            ctx->drv.ahead();
+            CK(ctx->mail.wait());
+            status = ctx->mail.m->back.status;
+            dt = ctx->mail.m->back.dt;
+            carried = !defer;
+            if (defer && !(status & (DG_ST_FAIL | DG_ST_NONFINITE)) && ctx->t + dt < ctx->drv.t_next) {
+                CK(next_projection(ctx, t));
+                carried = true;
+            }
             ok = !(status & (DG_ST_FAIL | DG_ST_TROUBLED_));
             if (ok) break;
             if (!repeat) {
@@ -1182,7 +1332,7 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
             }
             // flatten the marked cells of u^n; a flat one (or a failed mean) halves dt
             ctx->marks_dirty = true;
-            CK(cudaMemcpyAsync(&ctx->ctl->status, &zero, sizeof(zero), cudaMemcpyHostToDevice, ctx->st));
+            CK(cudaMemsetAsync(&ctx->ctl->status, 0, sizeof(unsigned int), ctx->st));
             {
                 Timed tm(ctx, KIND_OTHER);
                 Launch L = make_launch(ctx);
@@ -1191,9 +1341,9 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
                                     : launch_flatten<float>(L, (float*)ctx->reg[A], ctx->trouble, ctx->level);
                 CK(e);
             }
-            unsigned int fst = 0u;
-            CK(cudaMemcpyAsync(&fst, &ctx->ctl->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->st));
-            CK(cudaStreamSynchronize(ctx->st));
+            CK(ctx->mail.request(ctx->ctl, ctx->st));
+            CK(ctx->mail.wait());
+            const unsigned int fst = ctx->mail.m->back.status;
             if ((fst & DG_ST_FLAT_) || (status & DG_ST_FAIL)) {
                 ++halvings;
             } else if (!(fst & DG_ST_SCALED_)) {
@@ -1206,16 +1356,19 @@ int dg_step(dg_ctx* ctx, int nsteps, double fixed_dt, double* t_out, double* dt_
         if (repeat && attempts > 1) status |= DG_ST_REPEATED;
         if (!ok) {
             ctx->status |= status;
+            CK(cudaStreamSynchronize(ctx->st));
             return fail(ctx, DG_EPOSITIVITY, repeat ? "dg_step: positivity repetitions exhausted"
                                                     : "dg_step: positivity retries exhausted");
         }
         ctx->status |= status;
         ctx->cur = out[ctx->rk - 1];
         ctx->pb = (pb + ctx->rk) & 1;
-        ctx->carry = !(status & DG_ST_NONFINITE);
+        ctx->carry = carried && !(status & DG_ST_NONFINITE);
         ctx->t += dt;
         ctx->dt_last = dt;
         ctx->steps += 1;
+        // the projection for the next step may still be running
+        if (st + 1 == nsteps || (status & DG_ST_NONFINITE)) CK(cudaStreamSynchronize(ctx->st));
         if (status & DG_ST_NONFINITE) return fail(ctx, DG_ENONFINITE, "dg_step: non-finite coefficient");
     }
     if (t_out) *t_out = ctx->t;
@@ -1486,14 +1639,7 @@ int dg_get_meta(dg_ctx* ctx, dg_meta* m)
     m->t = ctx->t;
     m->steps = ctx->steps;
     m->dt_last = ctx->dt_last;
-    m->forcing_on = ctx->drv.on ? 1 : 0;
-    m->forcing_dirty = ctx->drv.dirty ? 1 : 0;
-    m->t_next = ctx->drv.t_next;
-    m->rng = ctx->drv.rng;
-    m->have_spare = ctx->drv.have_spare ? 1 : 0;
-    m->spare = ctx->drv.spare;
-    m->nmodes = ctx->drv.nm;
-    std::memcpy(m->x, ctx->drv.x, sizeof(double) * 6 * ctx->drv.nm);
+    ctx->drv.save(*m);
     return DG_OK;
 }
 
@@ -1505,14 +1651,8 @@ int dg_set_meta(dg_ctx* ctx, const dg_meta* m)
     ctx->t = m->t;
     ctx->steps = m->steps;
     ctx->dt_last = m->dt_last;
-    ctx->drv.on = m->forcing_on != 0;
-    ctx->drv.t_next = m->t_next;
-    ctx->drv.rng = m->rng;
-    ctx->drv.have_spare = m->have_spare != 0;
-    ctx->drv.spare = m->spare;
-    std::memcpy(ctx->drv.x, m->x, sizeof(double) * 6 * m->nmodes);
     // re-project the current OU amplitudes before the next step
-    ctx->drv.dirty = ctx->drv.on;
+    ctx->drv.restore(*m);
     if (!ctx->drv.on) ctx->forcing_active = false;
     return DG_OK;
 }
@@ -1661,6 +1801,7 @@ struct dg_adi_ctx {
     void* ahat = nullptr;   // driving a_h [c][3][b] (scratch)
     int* d_kvec = nullptr;
     double* d_amp = nullptr;
+    MailBox mail;
     void* gtab = nullptr;  // forcing: 1D factors, built by the first projection
     bool gtab_ready = false;
     Rule1 r1{};
@@ -1858,6 +1999,7 @@ int dg_adi_init(dg_adi_ctx** out, const dg_mesh* mesh, int order, const dg_nu_pa
     Ctl c0{};
     c0.dt_scale = 1.0;
     c0.dt_num = ctx->cfl * ctx->h / (ctx->K + 1);
+    if (e == cudaSuccess) e = ctx->mail.open();
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->ttab, tt.data(), tt.size(), cudaMemcpyHostToDevice, ctx->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(ctx->ctl, &c0, sizeof(Ctl), cudaMemcpyHostToDevice, ctx->st);
     if (e == cudaSuccess)
@@ -1954,31 +2096,18 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
             ACK(cudaMemsetAsync(ctx->ahat, 0, ahat_bytes, ctx->st));
         }
         if (ctx->drv.on) {
-            while (ctx->t >= ctx->drv.t_next) {
-                ctx->drv.advance();
-                ctx->drv.t_next += ctx->drv.dtd;
-                ctx->drv.dirty = true;
-            }
+            ctx->drv.update(ctx->t);
             if (ctx->drv.dirty) {
-                std::vector<double> amp;
-                std::vector<int> kv;
-                ctx->drv.amplitudes(amp, kv);
-                std::vector<int> ints;
-                std::vector<double> pamp;
-                const ForceModes fm = pack_modes(ctx->drv.nm, kv.data(), amp.data(), ints, pamp);
-                ACK(cudaMemcpyAsync(ctx->d_kvec, ints.data(), sizeof(int) * ints.size(), cudaMemcpyHostToDevice,
-                                    ctx->st));
-                ACK(cudaMemcpyAsync(ctx->d_amp, pamp.data(), sizeof(double) * pamp.size(), cudaMemcpyHostToDevice,
-                                    ctx->st));
+                const Driver::Pack& pk = ctx->drv.packs();
+                ACK(ctx->mail.modes(pk, ctx->d_kvec, ctx->d_amp, ctx->st));
                 const Launch L = adi_make_launch(ctx);
                 if (!ctx->gtab_ready) {
                     ACK(ctx->prec == DG_PREC_F64 ? launch_force_axis<double>(L) : launch_force_axis<float>(L));
                     ctx->gtab_ready = true;
                 }
                 ACK(ctx->prec == DG_PREC_F64
-                        ? launch_force<double>(L, fm, ctx->d_kvec, ctx->d_amp, (double*)ctx->ahat)
-                        : launch_force<float>(L, fm, ctx->d_kvec, ctx->d_amp, (float*)ctx->ahat));
-                ACK(cudaStreamSynchronize(ctx->st));  // the host amplitude buffers are reused
+                        ? launch_force<double>(L, pk.fm, ctx->d_kvec, ctx->d_amp, (double*)ctx->ahat)
+                        : launch_force<float>(L, pk.fm, ctx->d_kvec, ctx->d_amp, (float*)ctx->ahat));
                 ctx->drv.dirty = false;
                 ctx->forcing_active = true;
             }
@@ -1991,15 +2120,9 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
         const int* out = ctx->rk == 2 ? out2 : out3;
         bool ok = false;
         unsigned int status = 0u;
-        double dt = 0.0, inj = 0.0;
+        double dt = 0.0, inj = 0.0, diss = 0.0;
         for (int retry = 0; retry <= 3 && !ok; ++retry) {
-            struct {
-                double dt_scale, fixed_dt;
-            } hs = {1.0 / (double)(1 << retry), fixed_dt};
-            ACK(cudaMemcpyAsync(&ctx->ctl->dt_scale, &hs, sizeof(hs), cudaMemcpyHostToDevice, ctx->st));
-            ACK(cudaMemsetAsync(&ctx->ctl->status, 0, sizeof(unsigned int), ctx->st));
-            ACK(cudaMemsetAsync(&ctx->ctl->smax, 0, sizeof(unsigned long long), ctx->st));
-            ACK(cudaMemsetAsync(&ctx->ctl->diag[1], 0, sizeof(double), ctx->st));
+            ACK(ctx->mail.post(ctx->ctl, 1.0 / (double)(1 << retry), fixed_dt, ctx->st));
             // projections of v and p of u^n (with its CFL bound); the later stages project
             // their inputs (alternating buffers)
             void* pr[2] = {ctx->prim, ctx->prim2};
@@ -2028,37 +2151,31 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
                 rk_weights(ctx->rk, s, ctx->prec != DG_PREC_F64, t.rk_a, t.rk_b);
                 ACK(adi_go(ctx, t));
             }
-            struct {
-                unsigned int status;
-                double dt, inj;
-            } back{};
-            ACK(cudaMemcpyAsync(&back.status, &ctx->ctl->status, sizeof(unsigned int), cudaMemcpyDeviceToHost, ctx->st));
-            ACK(cudaMemcpyAsync(&back.dt, &ctx->ctl->dt, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-            ACK(cudaMemcpyAsync(&back.inj, &ctx->ctl->diag[1], sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-            ACK(cudaStreamSynchronize(ctx->st));
-            status = back.status;
-            dt = back.dt;
-            inj = back.inj;
+            if (ctx->cs_reset > 0.0) {
+                // uniform temperature restored in the last stage's output; the thermal
+                // energy taken out is the dissipation.  (Enqueued before the status is
+                // known: a failed attempt starts again from u^n.)
+                AdiLaunch r{};
+                r.mode = ADI_RESET;
+                r.u_in = ctx->reg[out[ctx->rk - 1]];
+                r.out = ctx->reg[out[ctx->rk - 1]];
+                r.cs_reset = ctx->cs_reset;
+                ACK(adi_go(ctx, r));
+            }
+            ACK(ctx->mail.request(ctx->ctl, ctx->st));
+            ctx->drv.ahead();
+            ACK(ctx->mail.wait());
+            status = ctx->mail.m->back.status;
+            dt = ctx->mail.m->back.dt;
+            inj = ctx->mail.m->back.work[0];
+            diss = ctx->mail.m->back.work[1];
             ok = !(status & DG_ST_FAIL);
         }
         ctx->status |= status;
         if (!ok) return afail(ctx, DG_EPOSITIVITY, "dg_adi_step: positivity retries exhausted");
         ctx->cur = out[ctx->rk - 1];
         if (force) ctx->injected += inj;
-        if (ctx->cs_reset > 0.0) {
-            // uniform temperature restored; the thermal energy taken out is the dissipation
-            ACK(cudaMemsetAsync(&ctx->ctl->diag[2], 0, sizeof(double), ctx->st));
-            AdiLaunch r{};
-            r.mode = ADI_RESET;
-            r.u_in = ctx->reg[ctx->cur];
-            r.out = ctx->reg[ctx->cur];
-            r.cs_reset = ctx->cs_reset;
-            ACK(adi_go(ctx, r));
-            double d = 0.0;
-            ACK(cudaMemcpyAsync(&d, &ctx->ctl->diag[2], sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
-            ACK(cudaStreamSynchronize(ctx->st));
-            ctx->dissipated += d;
-        }
+        if (ctx->cs_reset > 0.0) ctx->dissipated += diss;
         ctx->t += dt;
         ctx->dt_last = dt;
         ctx->steps += 1;
@@ -2126,14 +2243,7 @@ int dg_adi_get_meta(dg_adi_ctx* ctx, dg_adi_meta* m)
     m->m.t = ctx->t;
     m->m.steps = ctx->steps;
     m->m.dt_last = ctx->dt_last;
-    m->m.forcing_on = ctx->drv.on ? 1 : 0;
-    m->m.forcing_dirty = ctx->drv.dirty ? 1 : 0;
-    m->m.t_next = ctx->drv.t_next;
-    m->m.rng = ctx->drv.rng;
-    m->m.have_spare = ctx->drv.have_spare ? 1 : 0;
-    m->m.spare = ctx->drv.spare;
-    m->m.nmodes = ctx->drv.nm;
-    std::memcpy(m->m.x, ctx->drv.x, sizeof(double) * 6 * ctx->drv.nm);
+    ctx->drv.save(m->m);
     m->injected = ctx->injected;
     m->dissipated = ctx->dissipated;
     return DG_OK;
@@ -2147,14 +2257,7 @@ int dg_adi_set_meta(dg_adi_ctx* ctx, const dg_adi_meta* m)
     ctx->t = m->m.t;
     ctx->steps = m->m.steps;
     ctx->dt_last = m->m.dt_last;
-    ctx->drv.on = m->m.forcing_on != 0;
-    ctx->drv.t_next = m->m.t_next;
-    ctx->drv.rng = m->m.rng;
-    ctx->drv.have_spare = m->m.have_spare != 0;
-    ctx->drv.spare = m->m.spare;
-    std::memcpy(ctx->drv.x, m->m.x, sizeof(double) * 6 * m->m.nmodes);
-    // the forcing is projected again from these OU amplitudes before the next step
-    ctx->drv.dirty = ctx->drv.on;
+    ctx->drv.restore(m->m);
     if (!ctx->drv.on) ctx->forcing_active = false;
     ctx->injected = m->injected;
     ctx->dissipated = m->dissipated;

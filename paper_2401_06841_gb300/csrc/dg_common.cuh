@@ -117,14 +117,17 @@ struct Rule1 {
 };
 
 struct Ctl {
+    // written by the host before every attempt of a step, in one copy (up to dt)
     unsigned int status;     // sticky DG_ST_* bits
     unsigned int cnt_proj;   // last-block counter of the projection kernel
     unsigned int cnt_diag;   // last-block counter of diagnostics / L1
     unsigned int pad0;
     unsigned long long smax; // bits of max sum_d(|v_d|+cs) (positive double)
-    double dt;               // dt of the current step (fixes Pi_max), written for the host
     double dt_scale;         // 1, 1/2, 1/4, 1/8 on retries
     double fixed_dt;         // > 0 replaces the CFL dt
+    double work[2];          // adiabatic: energy injected by the driving, energy taken out by the reset
+    // read back together with the fields above
+    double dt;               // dt of the current step (fixes Pi_max), written for the host
     double abar2[2][3];      // <rho a_h>/<rho>, one slot per projected-velocity buffer
     double dt_num;           // cfl h / (k+1)
     double diag[16];         // diagnostics result

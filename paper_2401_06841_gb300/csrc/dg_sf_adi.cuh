@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
             reduce(diss, d, n);
             if (tid == 0) mine[0] = d[0];  // component 0 is warp 0's
             if (last_block_reduce<NT>(a.partials + 8, mine, 1, &a.ctl->cnt_diag, s_tot) && tid == 0)
-                a.ctl->diag[2] += s_tot[0] * a.h3;
+                a.ctl->work[1] += s_tot[0] * a.h3;
         } else {
             // 0-2 <rho a_h>, 3 <rho>, 4 <m.a_h>, 5-7 <m>
             constexpr int nc = n < 3 ? n : 3;
@@ -504,7 +504,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
                 if (PROJ)
                     for (int i = 0; i < 3; ++i) a.ctl->abar2[a.abar_out][i] = ab[i];
                 if (VOL && a.stage)
-                    a.ctl->diag[1] += a.beta * dtd * a.h3 *
+                    a.ctl->work[0] += a.beta * dtd * a.h3 *
                                       (s_tot[4] - ab[0] * s_tot[5] - ab[1] * s_tot[6] - ab[2] * s_tot[7]);
             }
         }
