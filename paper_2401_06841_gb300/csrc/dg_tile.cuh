@@ -256,37 +256,6 @@ __device__ __forceinline__ void stage_async_state(T* dst, const T* src, int coun
     }
 }
 
-// reciprocal within about one ulp: the hardware approximation (PTX rcp.approx)
-// refined by Newton-Raphson steps r <- r + r (1 - x r), one in FP32, two in FP64 (four
-// instructions of the slow FP64 pipe instead of a division's dozen)
-template <typename T>
-__device__ __forceinline__ T rcp(T x)
-{
-    if constexpr (sizeof(T) == 4) {
-        float r0;
-        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(x));
-        const float e = fmaf(-x, r0, 1.0f);
-        return fmaf(r0, e, r0);
-    } else {
-        double r;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-        r = fma(r, fma(-x, r, 1.0), r);
-        return fma(r, fma(-x, r, 1.0), r);
-    }
-}
-// square root: in FP32 the hardware approximation (relative error below 2^-22)
-template <typename T>
-__device__ __forceinline__ T fast_sqrt(T x)
-{
-    if constexpr (sizeof(T) == 4) {
-        float r;
-        asm("sqrt.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
-        return r;
-    } else {
-        return sqrt(x);
-    }
-}
-
 // --------------------------------------------------------------------------
 // block GEMM on the CUDA cores: C[M][N] = A[M][K] B[K][N] (row-major, shared)
 // thread micro-tile TM x TN with interleaved rows (row = mt + i*M/TM)
