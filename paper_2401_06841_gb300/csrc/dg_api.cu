@@ -452,6 +452,7 @@ void Driver::make_pack(Pack& p) const
 // (the host waits for the read-back).
 struct Mail {
     Ctl in, back;
+    double loss;  // written by the training kernels
     int kvec[3 * kMaxModes];
     double amp[6 * kMaxModes];
 };
@@ -579,7 +580,6 @@ struct dg_ctx {
     float* mv = nullptr;       // Adam second moments
     float* mg = nullptr;       // gradient
     uint32_t* mpack = nullptr; // packed BF16 inference weights
-    double* mloss = nullptr;
     float* mwork = nullptr;
     float* nu_cell = nullptr;  // per-cell coefficient (learned mode)
     float* nu_next = nullptr;  // the next step's coefficient, written by the last stage (learned mode)
@@ -621,7 +621,7 @@ namespace {
 
 struct ScratchLayout {
     size_t ctl, partials, tab, ttab, kvec, amp, gtab;
-    size_t mw, mm, mv, mg, mpack, mloss, mwork;  // learned sensor: weights, Adam moments, grad, packed, loss, work
+    size_t mw, mm, mv, mg, mpack, mwork;  // learned sensor: weights, Adam moments, grad, packed, work
     size_t nu, nu2, vabs;                        // per-cell coefficients (this and the next step) and |v| projection (learned mode)
     size_t ana;                                  // turbulence statistics: 4 x DG_MAX_BINS doubles + 1
     size_t trouble, level;                       // positivity by repetition: per-cell marks and levels (bytes)
@@ -663,8 +663,6 @@ ScratchLayout scratch_layout(int K, int N, bool learned = false)
     off = align256(off + sizeof(float) * kMlpMaxParams);
     s.mpack = off;
     off = align256(off + sizeof(uint32_t) * kMlpPackWords);
-    s.mloss = off;
-    off = align256(off + sizeof(double) * 16);
     s.mwork = off;
     off = align256(off + sizeof(float) * mlp_work_floats_host());
     s.ana = off;
@@ -1019,7 +1017,6 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
     ctx->mv = (float*)(ctx->scratch + sl.mv);
     ctx->mg = (float*)(ctx->scratch + sl.mg);
     ctx->mpack = (uint32_t*)(ctx->scratch + sl.mpack);
-    ctx->mloss = (double*)(ctx->scratch + sl.mloss);
     ctx->mwork = (float*)(ctx->scratch + sl.mwork);
     ctx->nu_cell = (float*)(ctx->scratch + sl.nu);
     ctx->nu_next = (float*)(ctx->scratch + sl.nu2);
@@ -1478,11 +1475,11 @@ int dg_mlp_grad(dg_ctx* ctx, const float* x, const float* y, int64_t n, float* g
     if (!ctx->weights_set) return fail(ctx, DG_ESTATE, "dg_mlp_grad: no weights");
     {
         Timed tm(ctx, KIND_OTHER);
-        CK(mlp_train_pass(ctx->st, ctx->mlp_D, ctx->mw, x, y, (int)n, ctx->mwork, ctx->mg, ctx->mloss));
+        // the gradient straight to the caller, the loss to pinned host memory
+        CK(mlp_train_pass(ctx->st, ctx->mlp_D, ctx->mw, x, y, (int)n, ctx->mwork, grad, &ctx->mail.m->loss));
     }
-    CK(cudaMemcpyAsync(grad, ctx->mg, sizeof(float) * ctx->mlp_P, cudaMemcpyDeviceToDevice, ctx->st));
-    CK(cudaMemcpyAsync(loss, ctx->mloss, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
+    *loss = ctx->mail.m->loss;
     return DG_OK;
 }
 
@@ -1500,16 +1497,14 @@ int dg_mlp_train(dg_ctx* ctx, const float* x, const float* y, int64_t n, const d
         losses.clear();
         for (int64_t s0 = 0; s0 < n; s0 += o->batch) {
             const int nb = (int)std::min<int64_t>(o->batch, n - s0);
-            CK(mlp_train_pass(ctx->st, D, ctx->mw, x + s0 * D, y + s0, nb, ctx->mwork, ctx->mg, ctx->mloss));
+            CK(mlp_train_pass(ctx->st, D, ctx->mw, x + s0 * D, y + s0, nb, ctx->mwork, ctx->mg, &ctx->mail.m->loss));
             ctx->adam_t += 1;
             const float c1 = (float)(1.0 / (1.0 - std::pow(o->beta1, (double)ctx->adam_t)));
             const float c2 = (float)(1.0 / (1.0 - std::pow(o->beta2, (double)ctx->adam_t)));
             CK(mlp_adam(ctx->st, ctx->mlp_P, ctx->mw, ctx->mg, ctx->mm, ctx->mv, (float)o->lr, (float)o->beta1,
                         (float)o->beta2, (float)o->eps, c1, c2));
-            double l = 0.0;
-            CK(cudaMemcpyAsync(&l, ctx->mloss, sizeof(double), cudaMemcpyDeviceToHost, ctx->st));
             CK(cudaStreamSynchronize(ctx->st));
-            losses.push_back(l);
+            losses.push_back(ctx->mail.m->loss);
         }
         double sum = 0.0;
         for (double l : losses) sum += l;

@@ -67,16 +67,19 @@ struct Pair {
 };
 
 // One training pass over MLP_SB samples per block, lane = sample, warp w = hidden
-// units 8w .. 8w+7: forward (activations in shared memory, pre-activations in
+// units 4w .. 4w+3: forward (activations in shared memory, pre-activations in
 // registers), backward, and the block's sums of the parameter gradients
 //   dz2 = (2 r / n) W3 gelu'(z2),  dz1 = (W2^T dz2) gelu'(z1),
 //   dW1 = dz1 x^T, dW2 = dz2 a1^T, dW3 = (2/n) sum r a2.
 // The products of a gradient entry are summed as pairs over the block's samples
 // and over the blocks (k_mlp_reduce) in a fixed order.
 // Bound: instruction issue of the 10-instruction pair products (6.8 thousand per
-// sample).  4096 samples at D = 40: forward, backward and gradients took 27 + 44 +
-// 2088 us as separate passes with one thread per sample and one per parameter in
-// FP64 over 27 blocks.
+// sample), with four warps per scheduler in flight; half of the warps sum dW2, the
+// others dW1 and the rest.  4096 samples at D = 40: forward, backward and gradients
+// took 27 + 44 + 2088 us as separate passes with one thread per sample and one per
+// parameter in FP64 over 27 blocks, 29 us here with 8 warps that summed dW2 and dW1 in
+// turn, 25 us with 16.
+constexpr int MLP_NT = 512, MLP_HW = MLP_H / (MLP_NT / 32);  // threads, hidden units per warp
 template <int D>
 struct MlpPass {
     static constexpr MlpLayout L = MlpLayout::make(D);
@@ -86,15 +89,16 @@ struct MlpPass {
     // thread tiles of dW1 [64][D]: TR x TC entries
     static constexpr int TC = D % 5 == 0 ? 5 : 2, CG = D / TC, TR = MLP_H * CG / 256;
     static_assert(D % 4 == 0 && TR * 256 == MLP_H * CG, "tiles cover dW1");
+    static_assert(MLP_HW == 4 && L.oW2 % 4 == 0, "a warp's weights of a row are one 16-byte load");
 };
 
 template <int D>
-__global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, const float* __restrict__ X,
+__global__ void __launch_bounds__(MLP_NT) k_mlp_pass(const float* __restrict__ W, const float* __restrict__ X,
                                                   const float* __restrict__ Y, int n, float2* __restrict__ part)
 {
     using M = MlpPass<D>;
     constexpr MlpLayout L = M::L;
-    constexpr int SP = M::SP;
+    constexpr int SP = M::SP, HW = MLP_HW;
     extern __shared__ __align__(16) float sm[];
     float* sX = sm + M::oX;
     float* sA1 = sm + M::oA1;
@@ -104,21 +108,23 @@ __global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, c
     float* sR = sm + M::oR;
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
     const int i0 = blockIdx.x * MLP_SB, ns = min(MLP_SB, n - i0);
-    for (int e = tid; e < L.P; e += 256) sm[e] = W[e];
-    for (int e = tid; e < MLP_SB * D; e += 256) {
+    for (int e = tid; e < L.P / 4; e += MLP_NT)
+        reinterpret_cast<float4*>(sm)[e] = __ldg(reinterpret_cast<const float4*>(W) + e);
+    if (tid < L.P % 4) sm[L.P / 4 * 4 + tid] = W[L.P / 4 * 4 + tid];
+    for (int e = tid; e < MLP_SB * D; e += MLP_NT) {
         const int s = e / D, d = e - s * D;
         sX[d * SP + s] = s < ns ? X[(size_t)i0 * D + e] : 0.f;
     }
     __syncthreads();
-    float z1[8], z2[8];
+    float z1[HW], z2[HW];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) z1[j] = sm[L.ob1 + 8 * w + j];
+    for (int j = 0; j < HW; ++j) z1[j] = sm[L.ob1 + HW * w + j];
 #pragma unroll 2
     for (int d = 0; d < D; d += 4) {
         const float x[4] = {sX[d * SP + lane], sX[(d + 1) * SP + lane], sX[(d + 2) * SP + lane], sX[(d + 3) * SP + lane]};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW1 + (8 * w + j) * D + d);
+        for (int j = 0; j < HW; ++j) {
+            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW1 + (HW * w + j) * D + d);
             z1[j] += q.x * x[0];
             z1[j] += q.y * x[1];
             z1[j] += q.z * x[2];
@@ -126,17 +132,17 @@ __global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, c
         }
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sA1[(8 * w + j) * SP + lane] = gelu_f(z1[j]);
+    for (int j = 0; j < HW; ++j) sA1[(HW * w + j) * SP + lane] = gelu_f(z1[j]);
     __syncthreads();
 #pragma unroll
-    for (int j = 0; j < 8; ++j) z2[j] = sm[L.ob2 + 8 * w + j];
+    for (int j = 0; j < HW; ++j) z2[j] = sm[L.ob2 + HW * w + j];
 #pragma unroll 2
     for (int k = 0; k < MLP_H; k += 4) {
         const float x[4] = {sA1[k * SP + lane], sA1[(k + 1) * SP + lane], sA1[(k + 2) * SP + lane],
                             sA1[(k + 3) * SP + lane]};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW2 + (8 * w + j) * MLP_H + k);
+        for (int j = 0; j < HW; ++j) {
+            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW2 + (HW * w + j) * MLP_H + k);
             z2[j] += q.x * x[0];
             z2[j] += q.y * x[1];
             z2[j] += q.z * x[2];
@@ -144,7 +150,7 @@ __global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, c
         }
     }
 #pragma unroll
-    for (int j = 0; j < 8; ++j) sA2[(8 * w + j) * SP + lane] = gelu_f(z2[j]);
+    for (int j = 0; j < HW; ++j) sA2[(HW * w + j) * SP + lane] = gelu_f(z2[j]);
     __syncthreads();
     if (w == 0) {
         float y = sm[L.ob3];
@@ -155,29 +161,24 @@ __global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, c
     __syncthreads();
     const float d3 = 2.0f * sR[lane] / (float)n;
 #pragma unroll
-    for (int j = 0; j < 8; ++j)
-        sD2[(8 * w + j) * SP + lane] = d3 * sm[L.oW3 + 8 * w + j] * gelu_prime_f(z2[j]);
+    for (int j = 0; j < HW; ++j)
+        sD2[(HW * w + j) * SP + lane] = d3 * sm[L.oW3 + HW * w + j] * gelu_prime_f(z2[j]);
     __syncthreads();
     {
-        float s[8];
+        float s[HW];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) s[k] = 0.f;
+        for (int k = 0; k < HW; ++k) s[k] = 0.f;
 #pragma unroll 4
         for (int j = 0; j < MLP_H; ++j) {
             const float dz = sD2[j * SP + lane];
-            const float4 q0 = *reinterpret_cast<const float4*>(sm + L.oW2 + j * MLP_H + 8 * w);
-            const float4 q1 = *reinterpret_cast<const float4*>(sm + L.oW2 + j * MLP_H + 8 * w + 4);
-            s[0] += q0.x * dz;
-            s[1] += q0.y * dz;
-            s[2] += q0.z * dz;
-            s[3] += q0.w * dz;
-            s[4] += q1.x * dz;
-            s[5] += q1.y * dz;
-            s[6] += q1.z * dz;
-            s[7] += q1.w * dz;
+            const float4 q = *reinterpret_cast<const float4*>(sm + L.oW2 + j * MLP_H + HW * w);
+            s[0] += q.x * dz;
+            s[1] += q.y * dz;
+            s[2] += q.z * dz;
+            s[3] += q.w * dz;
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) sD1[(8 * w + k) * SP + lane] = s[k] * gelu_prime_f(z1[k]);
+        for (int k = 0; k < HW; ++k) sD1[(HW * w + k) * SP + lane] = s[k] * gelu_prime_f(z1[k]);
     }
     __syncthreads();
     float2* out = part + (size_t)blockIdx.x * (L.P + 1);
@@ -214,28 +215,30 @@ __global__ void __launch_bounds__(256) k_mlp_pass(const float* __restrict__ W, c
             for (int j = 0; j < C; ++j) o[i * IS * ldo + j * JS] = make_float2(acc[i][j].s, acc[i][j].c);
     };
     using std::integral_constant;
-    {
+    if (tid < 256) {
         const int j = tid >> 4, k = tid & 15;
         tile(integral_constant<int, 4>{}, integral_constant<int, 4>{}, integral_constant<int, 16>{},
              integral_constant<int, 16>{}, sD2 + j * SP, sA1 + k * SP, out + L.oW2 + j * MLP_H + k, MLP_H);
+        return;
     }
+    const int t2 = tid - 256;
     {
-        const int j = tid / M::CG, d = tid % M::CG;
+        const int j = t2 / M::CG, d = t2 % M::CG;
         tile(integral_constant<int, M::TR>{}, integral_constant<int, M::TC>{}, integral_constant<int, 256 / M::CG>{},
              integral_constant<int, M::CG>{}, sD1 + j * SP, sX + d * SP, out + L.oW1 + j * D + d, D);
     }
     // biases, the last layer and the loss: one entry per thread
-    if (tid < 3 * MLP_H + 2) {
-        const int j = tid & (MLP_H - 1), g = tid / MLP_H;
+    if (t2 < 3 * MLP_H + 2) {
+        const int j = t2 & (MLP_H - 1), g = t2 / MLP_H;
         const float* a = g == 0 ? sD1 + j * SP : g == 1 ? sD2 + j * SP : g == 2 ? sA2 + j * SP : sR;
         Pair acc;
         for (int s = 0; s < MLP_SB; ++s) {
-            if (g < 2 || tid == 3 * MLP_H)
+            if (g < 2 || t2 == 3 * MLP_H)
                 acc.add(a[s], 0.f);
             else
                 acc.add_prod(a[s], sR[s]);
         }
-        const int p = g == 0 ? L.ob1 + j : g == 1 ? L.ob2 + j : g == 2 ? L.oW3 + j : tid == 3 * MLP_H ? L.ob3 : L.P;
+        const int p = g == 0 ? L.ob1 + j : g == 1 ? L.ob2 + j : g == 2 ? L.oW3 + j : t2 == 3 * MLP_H ? L.ob3 : L.P;
         out[p] = make_float2(acc.s, acc.c);
     }
 }
