@@ -27,8 +27,7 @@ cudaError_t adi_vol(const Launch& L, const AArgs<T>& a)
     long g = (long)occ * L.nsm;
     if (g > ntile) g = ntile;
     if (g > kMaxGrid) g = kMaxGrid;
-    k_sfa_vol<T, K, MODE, FORCE, PROJ><<<(int)g, C::NT, sm, L.st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_sfa_vol<T, K, MODE, FORCE, PROJ>, (unsigned)g, C::NT, sm, L.st, a);
 }
 
 template <typename T, int K, int RS, bool STAGE>
@@ -39,8 +38,7 @@ cudaError_t adi_faces(const Launch& L, const AArgs<T>& a)
                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (ready != cudaSuccess) return ready;
     const int nb = (L.N + 3) / 4, g = nb * nb * ((L.N + 1) / 2);  // bricks of 4 x 4 x 2 cells
-    k_sfa_faces<T, K, RS, STAGE><<<g, 128, sm, L.st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_sfa_faces<T, K, RS, STAGE>, g, 128, sm, L.st, a);
 }
 
 template <typename T, int K>

@@ -18,8 +18,8 @@ static cudaError_t train_pass_d(cudaStream_t st, const float* W, const float* X,
     const int nb = (n + MLP_SB - 1) / MLP_SB;
     float2* part = reinterpret_cast<float2*>(work);
     k_mlp_pass<D><<<nb, MLP_NT, sm, st>>>(W, X, Y, n, part);
-    k_mlp_reduce<D><<<(L.P + 1 + 63) / 64, 256, 0, st>>>(part, nb, n, G, loss);
-    return cudaGetLastError();
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return launch_dependent(k_mlp_reduce<D>, (L.P + 1 + 63) / 64, 256, 0, st, part, nb, n, G, loss);
 }
 
 cudaError_t mlp_train_pass(cudaStream_t st, int D, const float* W, const float* X, const float* Y, int n, float* work,

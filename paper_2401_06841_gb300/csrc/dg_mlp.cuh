@@ -246,9 +246,10 @@ __global__ void __launch_bounds__(MLP_NT) k_mlp_pass(const float* __restrict__ W
 // gradient and loss from the blocks' sums: four threads per entry take the blocks
 // in quarters, added in order
 template <int D>
-__global__ void __launch_bounds__(256) k_mlp_reduce(const float2* __restrict__ part, int nb, int n,
-                                                    float* __restrict__ G, double* __restrict__ loss)
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float2* part, int nb, int n,
+                                                    float* G, double* loss)
 {
+    grid_dependency();
     constexpr MlpLayout L = MlpLayout::make(D);
     __shared__ float2 s[4][64];
     const int e = threadIdx.x & 63, q = threadIdx.x >> 6, p = blockIdx.x * 64 + e;
@@ -257,7 +258,7 @@ __global__ void __launch_bounds__(256) k_mlp_reduce(const float2* __restrict__ p
     if (p <= L.P) {
 #pragma unroll 8
         for (int b = b0; b < b1; ++b) {
-            const float2 v = part[(size_t)b * (L.P + 1) + p];
+            const float2 v = __ldcg(part + (size_t)b * (L.P + 1) + p);
             acc.add(v.x, v.y);
         }
     }

@@ -493,6 +493,7 @@ template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
 __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL ? 3 : 4) : K == 2 ? 4 : 8) : 1)
     k_sf_vol(const __grid_constant__ Args<T> a)
 {
+    grid_dependency();
     using C = VolCfg<T, K, VOL, FORCE, PROJ, VABS>;
     constexpr int b = C::b, n = C::n, NT = C::NT, NP = C::NP, NPD = C::NPD, LDU = C::LDU, LDA = C::LDA;
     constexpr G1<K> G{};
@@ -1026,6 +1027,7 @@ template <typename T, int K, int RS, bool STAGE>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? 4 : 3) : 1)
     k_sf_faces(const __grid_constant__ Args<T> a)
 {
+    grid_dependency();
     using C = FaceCfg<T, K>;
     constexpr int b = C::b, n = K + 1, NP = C::NP, NT = C::NT, LD = C::LD, nq = n * n * n, nf = 6 * n * n;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -84,6 +84,7 @@ template <typename T, int K, int MODE, bool FORCE, bool PROJ>
 __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K == 2 ? 4 : 8) : 1)
     k_sfa_vol(const __grid_constant__ AArgs<T> a)
 {
+    grid_dependency();
     using C = AVolCfg<T, K, MODE, FORCE, PROJ>;
     constexpr bool VOL = C::VOL, SRC = C::SRC;
     constexpr int b = C::b, n = C::n, NT = C::NT, NP = C::NP, NPD = C::NPD, LDU = C::LDU, LDA = C::LDA, LDH = C::LDH;
@@ -527,6 +528,7 @@ template <typename T, int K, int RS, bool STAGE>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 5 : K == 2 ? 3 : 2) : 1)
     k_sfa_faces(const __grid_constant__ AArgs<T> a)
 {
+    grid_dependency();
     using C = AFaceCfg<T, K>;
     constexpr int b = C::b, n = K + 1, NP = C::NP, LD = C::LD, nq = n * n * n, nf = 6 * n * n;
     extern __shared__ __align__(16) unsigned char smem_raw[];

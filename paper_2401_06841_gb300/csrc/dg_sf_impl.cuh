@@ -60,8 +60,7 @@ static cudaError_t go_vol(const Launch& L, const Args<T>& a, int occ)
     long g = (long)(occ < 1 ? 1 : occ) * L.nsm;
     if (g > ntile) g = ntile;
     if (g > kMaxGrid) g = kMaxGrid;
-    k_sf_vol<T, K, VOL, FORCE, PROJ, VABS><<<(int)g, C::NT, sizeof(T) * C::total, L.st>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(k_sf_vol<T, K, VOL, FORCE, PROJ, VABS>, (unsigned)g, C::NT, sizeof(T) * C::total, L.st, a);
 }
 
 template <typename T, int K, bool STAGE>
@@ -70,12 +69,9 @@ static cudaError_t go_faces(const Launch& L, const Args<T>& a)
     const size_t sm = sizeof(T) * FaceCfg<T, K>::total;
     const int nb = (L.N + 3) / 4, g = nb * nb * ((L.N + 1) / 2);  // bricks of 4 x 4 x 2 cells
     if (L.ph.riemann == 2)
-        k_sf_faces<T, K, 2, STAGE><<<g, 128, sm, L.st>>>(a);
-    else if (L.ph.riemann == 1)
-        k_sf_faces<T, K, 1, STAGE><<<g, 128, sm, L.st>>>(a);
-    else
-        k_sf_faces<T, K, 0, STAGE><<<g, 128, sm, L.st>>>(a);
-    return cudaGetLastError();
+        return launch_dependent(k_sf_faces<T, K, 2, STAGE>, g, 128, sm, L.st, a);
+    if (L.ph.riemann == 1) return launch_dependent(k_sf_faces<T, K, 1, STAGE>, g, 128, sm, L.st, a);
+    return launch_dependent(k_sf_faces<T, K, 0, STAGE>, g, 128, sm, L.st, a);
 }
 
 // the projection launch (mode 0), or the volume and face launches of a
