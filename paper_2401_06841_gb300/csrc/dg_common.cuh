@@ -15,6 +15,8 @@ namespace dg {
 
 // largest mesh: N^3 cell indices fit in 32 bits
 constexpr int kMaxN = 1024;
+// most blocks of a launch that leaves per-block partial sums
+constexpr int kMaxGrid = 8192;
 
 template <int K>
 struct Dims {

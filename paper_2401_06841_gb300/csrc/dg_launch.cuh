@@ -17,14 +17,12 @@ struct Launch {
     const void* tab;     // tables of the element type in use (auxiliary kernels)
     const void* ttab;    // tables of the tile kernels
     Ctl* ctl;
-    double* partials;    // [kMaxGrid][16]
+    double* partials;    // [16][kMaxGrid]
     int nsm;             // multiprocessors on the device
     int bk;              // 0: CUDA-core products, 1: split-BF16 x3 tensor-core products
     Rule1 r1;            // the 1D Gauss rule
     void* gtab;          // forcing: 1D factors [N][17][k+1][2] of the element type
 };
-
-constexpr int kMaxGrid = 8192;
 
 template <typename T>
 cudaError_t setup_kernels(int K);

@@ -891,8 +891,8 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL 
         __syncthreads();
         double* s_buf = reinterpret_cast<double*>(smem_raw);
         if (!VOL && a.dtf) {
-            const double sp = (double)smax + 3.0 * a.cs_d;
-            atomicMax(&s_smax, (unsigned long long)__double_as_longlong(sp));
+            const double sp = (double)warp_max(smax) + 3.0 * a.cs_d;
+            if (lane == 0) atomicMax(&s_smax, (unsigned long long)__double_as_longlong(sp));
             __syncthreads();
             if (tid == 0) atomicMax(&a.ctl->smax, s_smax);
         }

@@ -454,7 +454,8 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
     __syncthreads();
     double* s_buf = reinterpret_cast<double*>(smem_raw);
     if (MODE == SFA_PROJECT && a.dtf) {
-        atomicMax(&s_smax, (unsigned long long)__double_as_longlong((double)smax));
+        const double sp = (double)warp_max(smax);
+        if (lane == 0) atomicMax(&s_smax, (unsigned long long)__double_as_longlong(sp));
         __syncthreads();
         if (tid == 0) atomicMax(&a.ctl->smax, s_smax);
     }
@@ -474,7 +475,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
             double d[n];
             reduce(diss, d, n);
             if (tid == 0) mine[0] = d[0];  // component 0 is warp 0's
-            if (last_block_reduce<NT>(a.partials + 8, mine, 1, &a.ctl->cnt_diag, s_tot) && tid == 0)
+            if (last_block_reduce<NT>(a.partials + 8 * kMaxGrid, mine, 1, &a.ctl->cnt_diag, s_tot) && tid == 0)
                 a.ctl->work[1] += s_tot[0] * a.h3;
         } else {
             // 0-2 <rho a_h>, 3 <rho>, 4 <m.a_h>, 5-7 <m>
