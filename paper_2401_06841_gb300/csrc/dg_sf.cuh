@@ -489,8 +489,10 @@ struct VolCfg {
 //
 // Bound: FP32 instruction issue (about 8.8 thousand instructions per cell at
 // degree 3 with PROJ, 880 bytes of HBM traffic); FP64 by the FP64 pipe.
+// Blocks per SM in FP32: as many as the registers allow without spilling more than a few
+// (degree 2: 5 blocks 128^3 7.12 ms for 2 steps, 4 blocks 7.19, 6 blocks 7.23).
 template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
-__global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL ? 3 : 4) : K == 2 ? 4 : 8) : 1)
+__global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL ? 3 : 4) : K == 2 ? 5 : 8) : 1)
     k_sf_vol(const __grid_constant__ Args<T> a)
 {
     grid_dependency();
@@ -1023,8 +1025,10 @@ __device__ __forceinline__ void hll_normal(T cs, T cs2, const T* WL, const T* WR
 }
 
 // Bound: FP32 instruction issue (about 8 thousand instructions per cell at degree 3).
+// Blocks per SM in FP32, likewise: degree 1 8 blocks (96^3: 0.377 ms a step; 6: 0.394),
+// degree 2 4 (128^3, 2 steps: 7.19 ms; 5: 7.28), degree 3 3.
 template <typename T, int K, int RS, bool STAGE>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? 4 : 3) : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4 : 3) : 1)
     k_sf_faces(const __grid_constant__ Args<T> a)
 {
     grid_dependency();

@@ -525,8 +525,11 @@ struct AFaceCfg {
 // The brick layout of k_sf_faces; boundary faces take a ghost trace: the cell's own
 // (outflow), with the normal velocity negated (reflective), or the prescribed inflow
 // state at the faces at coordinate 0.
+// Blocks per SM in FP32: degree 1 6 (96^3: 0.440 ms a step; 5: 0.458), degree 2 4 with
+// HLLC (48^3 with reset, 2 steps: 0.81 ms; 3: 0.83) and 3 with Rusanov, whose flux
+// spills at 4 (88^3: 1.42 ms a step; 4: 1.45), degree 3 2 (64^3, 2 steps: 2.53 ms; 3: 2.85).
 template <typename T, int K, int RS, bool STAGE>
-__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 5 : K == 2 ? 3 : 2) : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (RS == 2 ? 4 : 3) : 2) : 1)
     k_sfa_faces(const __grid_constant__ AArgs<T> a)
 {
     grid_dependency();
