@@ -17,8 +17,9 @@ velocity projection for the next stage.  L2 is flushed (a 256 MB write)
 before every timed step, outside the timed interval (the state, 5.4 GB, is
 larger than L2 as well).
 
-Variants: plain FP32, split-BF16 x3 tensor-core products ("x3": tcgen05
-kernels), and the learned viscosity sensor (learned-f32, learned-x3; network
+Variants: plain FP32, the x3 mode (on the same sum-factorised FP32 kernels by
+default; split-BF16 tensor-core products with --x3-backend mma), and the learned
+viscosity sensor (learned-f32, learned-x3; network
 trained here, untimed, on plain-sensor pairs of separate driven runs at Mach 3
 and Mach 10, seeds 2 and 3, never the evaluation seeds).
 
@@ -123,9 +124,7 @@ def peaks():
 
 
 # committed ncu summaries of the stage kernels, per variant: (file, kernel sources)
-PROFILE = {"x3": ("k5_stage_x3_64c_k3.md", ("dg_tc5_kernels.cuh", "dg_tc5.cuh", "dg_tc5.cu", "dg_common.cuh")),
-           "f32": ("k_tile_f32_stage_64c_k3.md", ("dg_tile.cuh", "dg_mma.cuh", "dg_common.cuh",
-                                                   "dg_launch_impl.cuh"))}
+PROFILE = {"x3": ("k_sf_stage_x3_64c_k3.md", ("dg_sf.cuh", "dg_sf_impl.cuh", "dg_kernels.cuh", "dg_common.cuh"))}
 
 
 def profiled_traffic(variant, N):
@@ -645,7 +644,8 @@ def main():
     ap.add_argument("--train-epochs", dest="train_epochs", type=int, default=20)
     ap.add_argument("--diffusion", type=float, default=0.0, help="eps of an added div(eps grad u)")
     ap.add_argument("--x3-backend", dest="x3_backend", default="tcgen05", choices=["tcgen05", "mma"],
-                    help="order-3 x3 stage: the tcgen05 kernels or the fused mma.sync kernel")
+                    help="x3 stage: the FP32 kernels (tcgen05, the name of the default since it chose the tensor-core "
+                         "kernels that they replaced) or the fused mma.sync kernel")
     ap.add_argument("--c3-N", dest="c3_N", type=int, default=128, help="mesh of the strong-shock configuration")
     ap.add_argument("--c3-steps", dest="c3_steps", type=int, default=100)
     ap.add_argument("--no-c3", dest="no_c3", action="store_true")
@@ -739,8 +739,9 @@ def main():
     hbm, bf16, src = peaks()
     achieved = bytes_per_stage / (r["stage_ms"] * 1e-3) / 1e9
     tr = profiled_traffic(head, N)
-    kern = ("k5_volume + k5_faces + k5_project (tcgen05)" if head.endswith("x3")
-            else "k_tile stage (RHS + SSP-RK stage + positivity + next projection)")
+    mma = head.endswith("x3") and args.x3_backend == "mma"
+    kern = ("k_tile stage (RHS + SSP-RK stage + positivity + next projection)" if mma or args.diffusion > 0
+            else "k_sf_vol + k_sf_faces (+ the step's projection)")
     roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
             "traffic": tr, "kernel": "%s, %s; one launch = one RK stage" % (kern, head), "peak_source": src,
             "stage_ms": r["stage_ms"], "bytes_per_stage": bytes_per_stage}
@@ -767,7 +768,7 @@ def main():
     line = {"metric": METRIC, "value": r["value"], "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": r["ms_per_step"], "higher_is_better": True,
             "scaling": "weak", "vs_baseline": None,
-            "dtype": {"f32": "f32", "x3": "bf16x3+f32"}[head.split("-")[-1]], "data": "synthetic",
+            "dtype": "bf16x3+f32" if mma else "f32", "data": "synthetic",
             "config": dict(workload(args), variant=head), "roofline": roof, "clocks": clk,
             "gpu_launches": int(r["launches"]),
             "e2e": {"value": e2e_v, "unit": UNIT, "h2d_bytes_per_step": nbytes, "d2h_bytes_per_step": nbytes},

@@ -1027,7 +1027,7 @@ int dg_init(dg_ctx** out, const dg_mesh* mesh, int order, double cs, const dg_nu
     ctx->marks_dirty = true;
     // x3 by default runs on the same kernels as FP32: axis by axis in FP32 registers
     // the transforms take less time than as split-BF16 products on the tensor cores
-    // (64^3 P3, one driven step: 1.1 ms against 2.9 ms on tcgen05 products and 3.4 ms in
+    // (64^3 P3, one driven step: 1.0 ms against 2.9 ms on tcgen05 products and 3.4 ms in
     // the fused mma.sync kernel; the tensor pipe was 22-24 % busy, the rest of the time
     // went into splitting operands, staging them and waiting for products)
     ctx->sf = nu->diffusion == 0.0 && (ctx->prec != DG_PREC_X3 || opts->x3_backend == 0);

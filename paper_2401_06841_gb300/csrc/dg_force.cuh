@@ -88,7 +88,9 @@ struct ForceCfg {
 
 // block: rows iy0 .. iy0 + rpb - 1 of the plane iz = blockIdx.y, RB of them at a time
 // (their sums over ky are short chains of dependent loads: several rows in flight
-// cover the latency), 64 cells at a time
+// cover the latency), 64 cells at a time.  128^3 cells of degree 3 in FP32, 61 modes:
+// 190 us (2.7 TB/s of coefficients); 474 us row by row, 2060 us mode by mode at the
+// points.
 template <typename T, int K>
 __global__ void __launch_bounds__(192) k_force(const T* __restrict__ G, int N, int rpb, ForceModes fm,
                                                const int* __restrict__ modes, const double* __restrict__ amp,

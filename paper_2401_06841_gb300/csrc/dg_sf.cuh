@@ -21,10 +21,15 @@
 // owns the plane c of Gauss points along z (K+1 warps): it contracts the modes
 // along z with its plane's basis values, then walks the rows of points, whose
 // fields, fluxes and partial sums along x and y stay in registers; the sums along
-// z go through shared memory once per tile.  In k_sf_faces warp f owns face f of
-// the 32 cells (6 warps): the traces of both sides, the Riemann fluxes and the
-// lifted coefficients of a face stay in its thread's registers, and the six faces
-// meet in shared memory once per tile.
+// z go through shared memory once per tile.  In k_sf_faces a thread owns a face of a
+// brick of 4 x 4 x 2 cells (4 warps): the traces of both sides, the Riemann fluxes and
+// their projection stay in its registers, and the faces of a cell meet in shared
+// memory once per brick.
+//
+// A driven SSP-RK3 step of 64^3 cells of degree 3 in FP32 takes 0.99 ms (volume 117 to
+// 169, faces 130 us a stage, projection 66), where the dense products of the fused stage
+// kernel (dg_tile.cuh) took 5.07; 128^3 of degree 2 3.56 ms for 19.8; one FP64
+// right-hand side of 24^3 of degree 3 0.56 ms for 1.79.
 #pragma once
 
 #include "dg_kernels.cuh"
@@ -487,8 +492,9 @@ struct VolCfg {
 // velocity projection -> vh_out (VABS: and of |v|), with the forcing sums when
 // FORCE.  !VOL: the projection launch (CFL bound with a.dtf).
 //
-// Bound: FP32 instruction issue (about 8.8 thousand instructions per cell at
-// degree 3 with PROJ, 880 bytes of HBM traffic); FP64 by the FP64 pipe.
+// Bound: FP32 instruction issue and its latency: 13.7 thousand instructions per cell at
+// degree 3 with FORCE and PROJ go out in 58 % of the issue slots (FMA pipe 42 %, HBM
+// 18 %), with the 12 warps per SM that 168 registers leave.  FP64 by the FP64 pipe.
 // Blocks per SM in FP32: as many as the registers allow without spilling more than a few
 // (degree 2: 5 blocks 128^3 7.12 ms for 2 steps, 4 blocks 7.19, 6 blocks 7.23).
 template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
@@ -944,6 +950,12 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL 
 // have 192, and 96 operand rows where those would read 224.  Bricks past the end of
 // the mesh hold the periodic images of its cells, which are the neighbours the
 // last cells need.
+// Bound: latency between the phases of a brick (rows in, traces and fluxes, rows of the
+// stage in, combine), with the 12 warps per SM that 168 registers and 67 KB leave at
+// degree 3: issue slots 45 %, FMA pipe 31 %, HBM 35 %, no pipe near its limit.  64^3 of
+// degree 3 FP32: 130 us (2.3 TB/s; 212 us with the six faces of 32 consecutive cells),
+// 256^3 8.3 ms.  Four blocks with the traces in shared memory were slower
+// (0.83-0.9x), packed pairs of FP32 and a prefetch of the next bricks to L2 no faster.
 template <typename T, int K>
 struct FaceCfg {
     static constexpr int b = Dims<K>::b, NP = npair(K), NT = 128;
