@@ -944,12 +944,10 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL 
 // ---------------------------------------------------------------------------
 // face kernel
 // ---------------------------------------------------------------------------
-// A block takes a brick of 4 x 4 x 2 cells (lane = cell, x fastest) with 4 warps:
-// warps 0-2 own the + faces of the 32 cells along x, y, z, warp 3 the 8 + 8 + 16
-// - faces of the brick's lower sides: 128 faces where 32 cells taken one by one
-// have 192, and 96 operand rows where those would read 224.  Bricks past the end of
-// the mesh hold the periodic images of its cells, which are the neighbours the
-// last cells need.
+// A block takes a brick of 4 x 4 x 2 cells (lane = cell, x fastest) with 4 warps, a
+// thread per face (BrickFaces): 128 faces where 32 cells taken one by one have 192, and
+// 96 operand rows where those would read 224.  Bricks past the end of the mesh hold the
+// periodic images of its cells, which are the neighbours the last cells need.
 // Bound: latency between the phases of a brick (rows in, traces and fluxes, rows of the
 // stage in, combine), with the 12 warps per SM that 168 registers and 67 KB leave at
 // degree 3: issue slots 45 %, FMA pipe 31 %, HBM 35 %, no pipe near its limit.  64^3 of
@@ -966,6 +964,50 @@ struct FaceCfg {
     // 32-63: rvol, 64-95: u^n
     static constexpr int oFlux = 3 * REG;  // [variable][pair][face]
     static constexpr int total = oFlux + 4 * NP * 128;
+};
+
+// The faces of a brick by thread.  Warps 0 and 1 own the + faces of the cells along x
+// and y; warps 2 and 3 the three layers of z faces (0 below the brick, 1 between its
+// planes, 2 above) and the 8 + 8 faces of its lower x and y sides:
+//   warp 2 layer 1 of cells 0-7, lower x, layer 2; warp 3 lower y, layer 1 of cells 8-15,
+//   layer 0.
+// The traces along the directions are different code: no warp runs more than two of the
+// three while the others wait (with all lower faces in warp 3, 64^3 of degree 3 took 3.94
+// ms for 4 steps, 3.90 so; 256^3 51.0 and 50.5).
+struct BrickFaces {
+    int d, rowL, rowR;  // direction, rows of the lower (L) and upper (R) cell
+    __device__ __forceinline__ BrickFaces(int w, int lane)
+    {
+        const int i = lane & 3, j = (lane >> 2) & 3, k = lane >> 4, k8 = j & 1;
+        if (w < 2) {
+            d = w;
+            rowL = lane;
+            rowR = w == 0 ? (i < 3 ? lane + 1 : 40 + 4 * k + j) : (j < 3 ? lane + 4 : 56 + 4 * k + i);
+        } else if (k == 0 && (lane >= 8) == (w == 2)) {  // lower x of (j, k) = (i, k8), lower y of (i, k8)
+            d = w - 2;
+            rowL = 32 + 16 * d + (lane & 7);
+            rowR = d == 0 ? 16 * k8 + 4 * i : 16 * k8 + i;
+        } else {
+            const bool low = w == 3 && k == 1;
+            d = 2;
+            rowL = low ? 64 + lane - 16 : lane;
+            rowR = low ? lane - 16 : (k < 1 ? lane + 16 : 80 + 4 * j + i);
+        }
+    }
+    // the face of cell c of the brick on its + / - side along Dd
+    template <int Dd>
+    __device__ static __forceinline__ int above(int c)
+    {
+        return 32 * Dd + c + (Dd == 2 && (c & 24) == 8 ? 32 : 0);
+    }
+    template <int Dd>
+    __device__ static __forceinline__ int below(int c)
+    {
+        const int i = c & 3, j = (c >> 2) & 3, k = c >> 4;
+        if constexpr (Dd == 0) return i > 0 ? c - 1 : 72 + 4 * k + j;
+        if constexpr (Dd == 1) return j > 0 ? 32 + c - 4 : 96 + 4 * k + i;
+        return k > 0 ? above<2>(c - 16) : 112 + c;
+    }
 };
 
 // 2D coefficients of a field's trace on the + (SIDE 1) or - face along Dd
@@ -1089,27 +1131,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
         copy_row(sm + (64 + rs) * LD, cell_of(ri, rj, rk ? 2 : -1));
         cp_async_commit();
     }
-    // the thread's face: direction, rows of its lower (L) and upper (R) cell
-    int d, rowL, rowR;
-    {
-        const int i = lane & 3, j = (lane >> 2) & 3, k = lane >> 4;
-        if (w < 3) {
-            d = w;
-            rowL = lane;
-            rowR = w == 0 ? (i < 3 ? lane + 1 : 40 + 4 * k + j)
-                          : (w == 1 ? (j < 3 ? lane + 4 : 56 + 4 * k + i) : (k < 1 ? lane + 16 : 80 + 4 * j + i));
-        } else if (lane < 16) {
-            // lanes 0-7: -x faces of (j, k); 8-15: -y faces of (i, k)
-            d = lane >> 3;
-            const int e0 = lane & 3, e1 = (lane >> 2) & 1;
-            rowL = 32 + 16 * d + (lane & 7);
-            rowR = d == 0 ? 16 * e1 + 4 * e0 : 16 * e1 + e0;
-        } else {
-            d = 2;
-            rowL = 64 + lane - 16;
-            rowR = lane - 16;
-        }
-    }
+    const BrickFaces face(w, lane);
+    const int d = face.d;
     const T dt = STAGE ? T(a.ctl->dt) : T(0);
     const bool fix = a.ahat != nullptr;
     cp_async_wait<0>();
@@ -1118,8 +1141,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
     // rho, v_n, v_t1, v_t2 ----
     T c2[8][NP];
     {
-        const T* Lp = sm + rowL * LD;
-        const T* Rp = sm + rowR * LD;
+        const T* Lp = sm + face.rowL * LD;
+        const T* Rp = sm + face.rowR * LD;
         auto traces = [&](auto D_) {
             constexpr int Dd = decltype(D_)::value;
             constexpr int t1 = Dd == 0 ? 1 : 0, t2 = Dd == 2 ? 1 : 2;
@@ -1222,10 +1245,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
     static_for<0, 3>([&](auto D_) {
         constexpr int Dd = decltype(D_)::value;
         const T* X = sm + C::oFlux + w * NP * 128;
-        const T* Xp = X + 32 * Dd + lane;
-        const T* Xm = X + (Dd == 0 ? (ci > 0 ? lane - 1 : 96 + 4 * ck + cj)
-                                   : (Dd == 1 ? (cj > 0 ? 32 + lane - 4 : 104 + 4 * ck + ci)
-                                              : (ck > 0 ? 64 + lane - 16 : 112 + 4 * cj + ci)));
+        const T *Xp = X + BrickFaces::above<Dd>(lane), *Xm = X + BrickFaces::below<Dd>(lane);
         static_for<0, K + 1>([&](auto I) {
             constexpr int p = decltype(I)::value;
             static_for<0, K - p + 1>([&](auto J) {

@@ -525,8 +525,10 @@ struct AFaceCfg {
     static constexpr int total = oFlux + 5 * NP * 128;
 };
 
-// The brick layout of k_sf_faces; boundary faces take a ghost trace: the cell's own
-// (outflow), with the normal velocity negated (reflective), or the prescribed inflow
+// The bricks of k_sf_faces, with warps 0-2 on the + faces along x, y, z and warp 3 on the
+// lower faces (BrickFaces here took degree 2 with HLLC from 0.81 to 0.80 ms and degree 3
+// from 2.53 to 2.60).  Boundary faces take a ghost trace: the cell's own (outflow), with
+// the normal velocity negated (reflective), or the prescribed inflow
 // state at the faces at coordinate 0.
 // Blocks per SM in FP32: degree 1 6 (96^3: 0.440 ms a step; 5: 0.458), degree 2 4 with
 // HLLC (48^3 with reset, 2 steps: 0.81 ms; 3: 0.83) and 3 with Rusanov, whose flux
