@@ -790,6 +790,7 @@ cudaError_t tile(dg_ctx* c, const TileLaunch& t)
 {
     const Launch L = make_launch(c);
     Timed tm(c, t.mode == TM_PROJECT ? KIND_PROJECT : KIND_RHS);
+    if (c->sf && t.mode != TM_PROJECT) c->counts.launches += 1;  // a volume and a face kernel
     return (c->prec == DG_PREC_F64) ? launch_tile<double>(L, t) : launch_tile<float>(L, t);
 }
 
