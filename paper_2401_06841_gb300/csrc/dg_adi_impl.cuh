@@ -37,7 +37,7 @@ cudaError_t adi_faces(const Launch& L, const AArgs<T>& a)
     static const cudaError_t ready = cudaFuncSetAttribute(k_sfa_faces<T, K, RS, STAGE>,
                                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (ready != cudaSuccess) return ready;
-    const int nb = (L.N + 3) / 4, g = nb * nb * ((L.N + 1) / 2);  // bricks of 4 x 4 x 2 cells
+    const int g = Brick::count(L.N);
     return launch_dependent(k_sfa_faces<T, K, RS, STAGE>, g, 128, sm, L.st, a);
 }
 

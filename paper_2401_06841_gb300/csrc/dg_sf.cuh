@@ -32,6 +32,7 @@
 // right-hand side of 24^3 of degree 3 0.56 ms for 1.79.
 #pragma once
 
+#include "dg_brick.cuh"
 #include "dg_kernels.cuh"
 #include "dg_tile.cuh"
 
@@ -1092,27 +1093,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
     T* sm = reinterpret_cast<T*>(smem_raw);
     __shared__ T s_th[TCELL];
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int N = a.N, nbx = (N + 3) >> 2;
-    int x0, y0, z0;
-    {
-        const unsigned q = blockIdx.x / (unsigned)nbx;
-        x0 = 4 * (int)(blockIdx.x - q * nbx);
-        y0 = 4 * (int)(q % (unsigned)nbx);
-        z0 = 2 * (int)(q / (unsigned)nbx);
-    }
-    // cell of brick coordinates (-1..4, -1..4, -1..2), periodic
-    auto cell_of = [&](int i, int j, int k) -> long {
-        int x = x0 + i, y = y0 + j, z = z0 + k;
-        x = x < 0 ? N - 1 : (x < N ? x : x % N);
-        y = y < 0 ? N - 1 : (y < N ? y : y % N);
-        z = z < 0 ? N - 1 : (z < N ? z : z % N);
-        return ((long)z * N + y) * N + x;
-    };
+    const Brick brick(blockIdx.x, a.N);
     // ---- operand rows (rho, v), four lanes per row ----
     const int rs = tid >> 2, sub = tid & 3;  // row within a group of 32, lane of it
     const int ri = rs & 3, rj = (rs >> 2) & 3, rk = rs >> 4;
-    const long rcell = cell_of(ri, rj, rk);
-    const bool rvalid = x0 + ri < N && y0 + rj < N && z0 + rk < N;
+    const long rcell = brick.cell(ri, rj, rk), own = brick.own(rs);
     {
         constexpr int CH = chunk<T, b>(), V = CH / (int)sizeof(T), NB = b / V;  // chunks of rho; 3 NB of v
         auto copy_row = [&](T* dst, long c) {
@@ -1127,8 +1112,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
         copy_row(sm + rs * LD, rcell);
         // -x, +x: (j, k) = (rs & 3, (rs >> 2) & 1); -y, +y: (i, k) the same
         const int hs = rs >> 3, h0 = rs & 3, h1 = (rs >> 2) & 1;
-        copy_row(sm + (32 + rs) * LD, hs < 2 ? cell_of(hs ? 4 : -1, h0, h1) : cell_of(h0, hs == 3 ? 4 : -1, h1));
-        copy_row(sm + (64 + rs) * LD, cell_of(ri, rj, rk ? 2 : -1));
+        copy_row(sm + (32 + rs) * LD, hs < 2 ? brick.cell(hs ? 4 : -1, h0, h1) : brick.cell(h0, hs == 3 ? 4 : -1, h1));
+        copy_row(sm + (64 + rs) * LD, brick.cell(ri, rj, rk ? 2 : -1));
         cp_async_commit();
     }
     const BrickFaces face(w, lane);
@@ -1164,13 +1149,15 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
             traces(std::integral_constant<int, 2>{});
     }
     __syncthreads();
-    // the operand rows are free: the epilogue's inputs arrive during the fluxes
+    // the operand rows are free: the epilogue's inputs arrive during the fluxes, those of
+    // the brick's own cells alone (rows past the end of the mesh keep what they hold: no
+    // result uses them)
     constexpr int CHU = chunk<T, 4 * b>(), VU = CHU / (int)sizeof(T), NCU = 4 * b / VU;
     static_assert(CHU == 16, "state rows in 16-byte chunks");
     const bool out16 = (reinterpret_cast<uintptr_t>(a.out) & 15u) == 0;
-    {
+    if (own >= 0) {
         auto copy_state = [&](T* dst, const T* src) {
-            const T* s = src + rcell * 4 * b;
+            const T* s = src + own * 4 * b;
             T* q = dst + rs * LD;
 #pragma unroll
             for (int k = 0; k < (NCU + 3) / 4; ++k)
@@ -1180,11 +1167,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
         if (out16) {
             copy_state(sm + C::REG, a.out);
         } else {
-            for (int e = sub; e < 4 * b; e += 4) sm[C::REG + rs * LD + e] = a.out[rcell * 4 * b + e];
+            for (int e = sub; e < 4 * b; e += 4) sm[C::REG + rs * LD + e] = a.out[own * 4 * b + e];
         }
         if (STAGE && a.rk_a != T(0)) copy_state(sm + 2 * C::REG, a.u_n);
-        cp_async_commit();
     }
+    cp_async_commit();
     // ---- Riemann fluxes at the face points, lifted row by row ----
     {
         T fx[4][NP];
@@ -1238,7 +1225,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
     T r[b];
     unsigned int st = 0u;
     const int ci = lane & 3, cj = (lane >> 2) & 3, ck = lane >> 4;
-    const bool valid = x0 + ci < N && y0 + cj < N && z0 + ck < N;
+    const bool valid = brick.inside(ci, cj, ck);
     T* const row = sm + lane * LD + w * b;  // u^(s), later the result
 #pragma unroll
     for (int l = 0; l < b; ++l) r[l] = T(0);
@@ -1321,7 +1308,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
                         mn = other < mn ? other : mn;
                     }
                     if (a.trouble && mn < T(0)) {
-                        if (lane == c) a.trouble[cell_of(ci, cj, ck)] |= DG_MARK_NEGATIVE;
+                        if (lane == c) a.trouble[brick.own(lane)] |= DG_MARK_NEGATIVE;
                         st |= DG_ST_TROUBLED_;
                     }
                     if (mn < a.eps) {
@@ -1351,8 +1338,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4
     }
     st_row<T, b>(row, r);
     __syncthreads();
-    if (rvalid) {
-        T* g = a.out + rcell * 4 * b;
+    if (own >= 0) {
+        T* g = a.out + own * 4 * b;
         const T* q = sm + rs * LD;
         if (out16) {
 #pragma unroll

@@ -544,25 +544,12 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
     T* sm = reinterpret_cast<T*>(smem_raw);
     __shared__ T s_bound[5][2][TCELL];  // mean and bound of the higher modes per variable and cell
     const int tid = threadIdx.x, w = tid >> 5, lane = tid & 31;
-    const int N = a.N, nbx = (N + 3) >> 2;
-    int x0, y0, z0;
-    {
-        const unsigned q = blockIdx.x / (unsigned)nbx;
-        x0 = 4 * (int)(blockIdx.x - q * nbx);
-        y0 = 4 * (int)(q % (unsigned)nbx);
-        z0 = 2 * (int)(q / (unsigned)nbx);
-    }
-    auto cell_of = [&](int i, int j, int k) -> long {
-        int x = x0 + i, y = y0 + j, z = z0 + k;
-        x = x < 0 ? N - 1 : (x < N ? x : x % N);
-        y = y < 0 ? N - 1 : (y < N ? y : y % N);
-        z = z < 0 ? N - 1 : (z < N ? z : z % N);
-        return ((long)z * N + y) * N + x;
-    };
+    const int N = a.N;
+    const Brick brick(blockIdx.x, N);
+    const int x0 = brick.x0, y0 = brick.y0, z0 = brick.z0;
     const int rs = tid >> 2, sub = tid & 3;
     const int ri = rs & 3, rj = (rs >> 2) & 3, rk = rs >> 4;
-    const long rcell = cell_of(ri, rj, rk);
-    const bool rvalid = x0 + ri < N && y0 + rj < N && z0 + rk < N;
+    const long rcell = brick.cell(ri, rj, rk), own = brick.own(rs);
     {
         constexpr int CH = chunk<T, b>(), V = CH / (int)sizeof(T), NB = b / V, NR = 5 * NB;
         auto copy_row = [&](T* dst, long c) {
@@ -576,8 +563,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
         };
         copy_row(sm + rs * LD, rcell);
         const int hs = rs >> 3, h0 = rs & 3, h1 = (rs >> 2) & 1;
-        copy_row(sm + (32 + rs) * LD, hs < 2 ? cell_of(hs ? 4 : -1, h0, h1) : cell_of(h0, hs == 3 ? 4 : -1, h1));
-        copy_row(sm + (64 + rs) * LD, cell_of(ri, rj, rk ? 2 : -1));
+        copy_row(sm + (32 + rs) * LD, hs < 2 ? brick.cell(hs ? 4 : -1, h0, h1) : brick.cell(h0, hs == 3 ? 4 : -1, h1));
+        copy_row(sm + (64 + rs) * LD, brick.cell(ri, rj, rk ? 2 : -1));
         cp_async_commit();
     }
     int d, rowL, rowR;
@@ -652,9 +639,10 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
     __syncthreads();
     constexpr int CHU = chunk<T, 5 * b>(), VU = CHU / (int)sizeof(T), NCU = 5 * b / VU;
     const bool out16 = (reinterpret_cast<uintptr_t>(a.out) & (CHU - 1)) == 0;
-    {
+    // the rows of the brick's own cells (see k_sf_faces)
+    if (own >= 0) {
         auto copy_state = [&](T* dst, const T* src) {
-            const T* s = src + rcell * 5 * b;
+            const T* s = src + own * 5 * b;
             T* q = dst + rs * LD;
 #pragma unroll
             for (int k = 0; k < (NCU + 3) / 4; ++k)
@@ -664,11 +652,11 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
         if (out16) {
             copy_state(sm + C::REG, a.out);
         } else {
-            for (int e = sub; e < 5 * b; e += 4) sm[C::REG + rs * LD + e] = a.out[rcell * 5 * b + e];
+            for (int e = sub; e < 5 * b; e += 4) sm[C::REG + rs * LD + e] = a.out[own * 5 * b + e];
         }
         if (STAGE && a.rk_a != T(0)) copy_state(sm + 2 * C::REG, a.u_n);
-        cp_async_commit();
     }
+    cp_async_commit();
     {
         T fx[5][NP];
 #pragma unroll
@@ -807,7 +795,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
     if constexpr (STAGE) {
         // ---- positivity of density and pressure (Sec. 3.1) ----
         const T eps = a.eps, g1 = a.gas.g1;
-        const bool valid = x0 + ci < N && y0 + cj < N && z0 + ck < N;
+        const bool valid = brick.inside(ci, cj, ck);
         bool check = false;
         if (valid) {
             T ub[5], dl[5];
@@ -908,7 +896,7 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
             }
         }
         __syncthreads();
-        if (rvalid) {
+        if (own >= 0) {
             bool bad = false;
             for (int e = sub; e < 5 * b; e += 4) bad |= !isfinite(sm[rs * LD + e]);
             if (bad) st |= DG_ST_NONFINITE_;
@@ -916,8 +904,8 @@ __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 6 : K == 2 ? (
         st = __reduce_or_sync(0xffffffffu, st);
         if (lane == 0 && st) atomicOr(&a.ctl->status, st);
     }
-    if (rvalid) {
-        T* g = a.out + rcell * 5 * b;
+    if (own >= 0) {
+        T* g = a.out + own * 5 * b;
         const T* q = sm + rs * LD;
         if (out16) {
 #pragma unroll

@@ -67,7 +67,7 @@ template <typename T, int K, bool STAGE>
 static cudaError_t go_faces(const Launch& L, const Args<T>& a)
 {
     const size_t sm = sizeof(T) * FaceCfg<T, K>::total;
-    const int nb = (L.N + 3) / 4, g = nb * nb * ((L.N + 1) / 2);  // bricks of 4 x 4 x 2 cells
+    const int g = Brick::count(L.N);
     if (L.ph.riemann == 2)
         return launch_dependent(k_sf_faces<T, K, 2, STAGE>, g, 128, sm, L.st, a);
     if (L.ph.riemann == 1) return launch_dependent(k_sf_faces<T, K, 1, STAGE>, g, 128, sm, L.st, a);
