@@ -1049,19 +1049,25 @@ __device__ __forceinline__ void rusanov_normal(T cs, T cs2, const T* WL, const T
     F[2] = qL * WL[2] + qR * WR[2];
     F[3] = qL * WL[3] + qR * WR[3];
 }
-// HLL, F = (S_R F_L - S_L F_R + S_L S_R (U_R - U_L))/(S_R - S_L) with the Davis bounds;
-// bounds of one sign are clamped at zero, which leaves the upwind flux:
-//   w_R = -S_L/(S_R - S_L), w_L = 1 - w_R, q_L = w_L rho_L (v_n,L - S_L),
+// HLL, F = (S_R F_L - S_L F_R + S_L S_R (U_R - U_L))/(S_R - S_L) with the Davis bounds,
+// clamped at zero where both have one sign:
+//   w_L = S_R/(S_R - S_L), w_R = -S_L/(S_R - S_L), q_L = w_L rho_L (v_n,L - S_L),
 //   q_R = w_R rho_R (v_n,R - S_R), p* = cs^2 (w_L rho_L + w_R rho_R).
+// The smaller weight is formed from its own bound and the larger one as the rest: a clamped
+// bound then leaves the upwind flux exactly, on either side, and a bound near zero lets no
+// rounding of the other weight carry a dense side's flux into a thin one.
 // CONTACT (HLLC for p = cs^2 rho): the tangential momenta cross with the mass flux at the
-// tangential velocity of the side the contact S_M = m*/rho* leaves behind
+// tangential velocity of the side the contact S_M = m*/rho* leaves behind (the upwind side
+// outside the bounds)
 template <typename T, bool CONTACT>
 __device__ __forceinline__ void hll_normal(T cs, T cs2, const T* WL, const T* WR, T* F)
 {
     const T vl = WL[1], vr = WR[1];
     const T SL = fmin(vl, vr) - cs, SR = fmax(vl, vr) + cs;
     const T sl = fmin(SL, T(0)), sr = fmax(SR, T(0));
-    const T wr = -sl * rcp<T>(sr - sl), wl = T(1) - wr;
+    const bool nearer = sr < -sl;  // of the two bounds S_R
+    const T ws = (nearer ? sr : -sl) * rcp<T>(sr - sl), wb = T(1) - ws;
+    const T wl = nearer ? ws : wb, wr = nearer ? wb : ws;
     const T rl = wl * WL[0], rr = wr * WR[0];
     const T qL = rl * (vl - sl), qR = rr * (vr - sr);
     F[0] = (rl * vl + rr * vr) - wr * sr * (WR[0] - WL[0]);
@@ -1070,7 +1076,7 @@ __device__ __forceinline__ void hll_normal(T cs, T cs2, const T* WL, const T* WR
         // signs of rho* and m* (times S_R - S_L > 0)
         const T aL = WL[0] * (SL - vl), aR = WR[0] * (SR - vr);
         const T ms = aR * vr - aL * vl - cs2 * (WR[0] - WL[0]);
-        const bool left = (aR - aL > T(0)) == (ms >= T(0));
+        const bool left = SL >= T(0) || (SR > T(0) && (aR - aL > T(0)) == (ms >= T(0)));
         F[2] = F[0] * (left ? WL[2] : WR[2]);
         F[3] = F[0] * (left ? WL[3] : WR[3]);
     } else {
