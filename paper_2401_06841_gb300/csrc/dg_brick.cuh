@@ -38,7 +38,7 @@ struct Brick {
     DG_BRICK_FN long own(int r) const
     {
         const int i = r & 3, j = (r >> 2) & 3, k = r >> 4;
-        return inside(i, j, k) ? ((long)(z0 + k) * N + y0 + j) * N + x0 + i : -1;
+        return inside(i, j, k) ? cell(i, j, k) : -1;
     }
 };
 
