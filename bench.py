@@ -64,7 +64,7 @@ def workload(args):
             "state": "synthetic k^-2 velocity (seed 105) relaxed %d driven FP32 steps, taken as the state at t=T"
                      % args.relax,
             "l2": "flushed (256 MB write) before every timed step; state larger than L2",
-            "learned_gate": "learned variants: nu/(cs h/p) < %g -> nu = 0 (tiles of 16 such cells skip div v)"
+            "learned_gate": "learned variants: nu/(cs h/p) < %g -> nu = 0 (blocks of 32 such cells skip div v)"
                             % args.nu_gate}
 
 
@@ -655,7 +655,7 @@ def main():
     ap.add_argument("--no-start", dest="no_start", action="store_true")
     ap.add_argument("--nu-gate", dest="nu_gate", type=float, default=1.0,
                     help="learned variants: cells with nu/(cs h/p) below this get no viscous pressure, and "
-                         "tiles of 16 such cells skip div v")
+                         "blocks of 32 such cells skip div v")
     ap.add_argument("--no-adiabatic", dest="no_adiabatic", action="store_true",
                     help="skip the timing of the five-variable adiabatic system")
     args = ap.parse_args()

@@ -94,9 +94,11 @@ typedef struct {
  * nu_gate (>= 0): in DG_AV_LEARNED mode a cell whose predicted coefficient
  * nu/(cs h/p) is below nu_gate gets nu = 0, i.e. no viscous pressure at any of
  * its points (the sensor's "no shock here" decision); 0 disables the gate.
- * A tile of 16 consecutive cells whose coefficients are all zero skips the
- * gradient evaluation and div v at its points (the result is the same as
- * with the work done: Pi = 0 there); dg_prof counts those tiles.
+ * Cells that a block of the volume kernel takes together (32 consecutive
+ * ones; 16, at k = 1 32, in the fused kernel of x3_backend 1 and of the
+ * diffusion operator) skip the gradient evaluation and div v at their points
+ * where all their coefficients are zero (the result is the same as with the
+ * work done: Pi = 0 there); dg_prof counts the skipped tiles.
  * diffusion (>= 0): eps of div(eps grad u).  The interface gradient is the
  * normal derivative at the face of the polynomial recovered over the face's
  * two cells (degree 2K+1 in the normal direction from the K+1 normal
@@ -347,14 +349,16 @@ int dg_av_nu_carried(dg_ctx* ctx, float* nu_out);
 typedef struct {
     int64_t launches;      /* kernels launched since the last reset               */
     int64_t n_project, n_rhs, n_force, n_other;
-    double ms_project;     /* projection kernel (K_A)                             */
-    double ms_rhs;         /* RHS + stage update kernel (K_B)                     */
+    double ms_project;     /* projection kernel                                   */
+    double ms_rhs;         /* volume and face kernels of right-hand sides and
+                              stages (or the fused stage kernel)                  */
     double ms_force;       /* forcing projection                                  */
     double ms_other;       /* diagnostics, L1                                     */
-    /* volume-term tiles (16 consecutive cells each) the stage kernels ran since
-     * the last reset, and those among them that skipped div v and the viscous
-     * pressure because every cell's coefficient was zero (DG_AV_LEARNED with
-     * nu_gate, or DG_AV_OFF); counted whether or not profiling is on */
+    /* volume-term tiles (16 consecutive cells each, 32 at k = 1) the stage
+     * kernels ran since the last reset, and those among them that skipped div v
+     * and the viscous pressure because the coefficient of every cell their block
+     * takes (dg_nu_params) was zero (DG_AV_LEARNED with nu_gate, or DG_AV_OFF);
+     * counted whether or not profiling is on */
     int64_t tiles_volume, tiles_gated;
 } dg_prof;
 int dg_profile(dg_ctx* ctx, int enable);          /* enable/disable; resets counts */

@@ -578,21 +578,17 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL 
         if constexpr (VOL) {
             if (a.av_mode == 2) {
                 // learned sensor: Pi = rho nu |div v|; no gradients where every cell of the
-                // tile has a zero coefficient
+                // block has a zero coefficient
                 b1 = valid ? T(a.nu[c0 + lane]) : T(0);
                 a2 = T(0);
-                const unsigned nz = __ballot_sync(0xffffffffu, b1 != T(0));
-                need_div = nz != 0u;
-                if (tid == 0) {
-                    for (int t0 = 0; t0 < nvalid; t0 += a.tcount) {
-                        const unsigned m = a.tcount >= 32 ? nz : (nz >> t0) & ((1u << a.tcount) - 1u);
-                        gated += m == 0u;
-                    }
-                }
-            } else if (tid == 0 && !need_div) {
-                gated += (nvalid + a.tcount - 1) / a.tcount;
+                need_div = __ballot_sync(0xffffffffu, b1 != T(0)) != 0u;
             }
-            if (tid == 0) ntiles += (nvalid + a.tcount - 1) / a.tcount;
+            if (tid == 0) {
+                // a block's cells skip together: a tile beside one that needs div v has not
+                const unsigned int nt = (nvalid + a.tcount - 1) / a.tcount;
+                ntiles += nt;
+                gated += need_div ? 0u : nt;
+            }
         }
         T A[4][NP];
         static_for<0, 4>([&](auto F) {
