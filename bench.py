@@ -155,6 +155,15 @@ def profiled_traffic(variant, N):
     return int(m_t.group(1)) * (N / 64) ** 3
 
 
+def stage_kernels(head, args):
+    """(description, DRAM bytes per stage or None) of the kernels that a stage of
+    variant `head` runs: the committed summary is that of the sum-factorised
+    kernels, which neither the mma.sync products nor the diffusion operator take."""
+    if args.diffusion > 0 or (head.endswith("x3") and args.x3_backend == "mma"):
+        return "k_tile stage (RHS + SSP-RK stage + positivity + next projection)", None
+    return "k_sf_vol + k_sf_faces (+ the step's projection)", profiled_traffic(head, args.N)
+
+
 def adiabatic_arm(args, dev, seed, flush, world, near_isothermal=False):
     """The five-variable adiabatic system (Sec. 2.1) on the same mesh and
     degree, FP32, steps timed like the main variants (L2 flushed before each,
@@ -738,10 +747,9 @@ def main():
     bytes_per_stage = dof * 4 * (1 + 2.0 / 3.0 + 1)
     hbm, bf16, src = peaks()
     achieved = bytes_per_stage / (r["stage_ms"] * 1e-3) / 1e9
-    tr = profiled_traffic(head, N)
-    mma = head.endswith("x3") and args.x3_backend == "mma"
-    kern = ("k_tile stage (RHS + SSP-RK stage + positivity + next projection)" if mma or args.diffusion > 0
-            else "k_sf_vol + k_sf_faces (+ the step's projection)")
+    kern, tr = stage_kernels(head, args)
+    # split products: x3 on the mma.sync back end, and with the diffusion operator
+    mma = head.endswith("x3") and (args.x3_backend == "mma" or args.diffusion > 0)
     roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s", "frac": achieved / hbm,
             "traffic": tr, "kernel": "%s, %s; one launch = one RK stage" % (kern, head), "peak_source": src,
             "stage_ms": r["stage_ms"], "bytes_per_stage": bytes_per_stage}
