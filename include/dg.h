@@ -49,10 +49,10 @@ extern "C" {
 #define DG_PREC_F64 0      /* everything in FP64 (parity mode)                   */
 #define DG_PREC_F32 1      /* FP32 state and arithmetic; FP64 global sums        */
 #define DG_PREC_X3 2       /* FP32 state; basis<->quadrature transforms in FP32
-                              (the kernels of DG_PREC_F32) or, by x3_backend or
-                              with the diffusion operator, on the tensor cores as
-                              split-BF16 x3 products with FP32 accumulation; FP64
-                              global sums                                        */
+                              (the kernels of DG_PREC_F32) or, by x3_backend, with
+                              the diffusion operator and in dg_rhs_noalloc, on the
+                              tensor cores as split-BF16 x3 products with FP32
+                              accumulation; FP64 global sums                     */
 
 /* ---- artificial viscosity modes ------------------------------------------ */
 #define DG_AV_OFF 0
@@ -383,8 +383,10 @@ int dg_set_meta(dg_ctx* ctx, const dg_meta* in);
  * plus a 1,180,160-byte head must fit in 64 MiB (N <= 65 at k = 3 in FP32,
  * N <= 51 in FP64); larger meshes return DG_ENOMEM and nothing runs.  Artificial
  * viscosity modes DG_AV_OFF and DG_AV_VNR only, no diffusion operator (nu->diffusion
- * must be 0), Rusanov face fluxes only (it equals dg_rhs of a context created
- * with riemann = DG_RIEMANN_RUSANOV).  Every call looks up the array's device
+ * must be 0), Rusanov face fluxes only: bit for bit dg_rhs of a context created
+ * with riemann = DG_RIEMANN_RUSANOV and, for DG_PREC_X3, x3_backend = 1 (here that
+ * precision is the split products; a context's default, x3_backend = 0, is FP32
+ * arithmetic, as DG_PREC_F32 is here).  Every call looks up the array's device
  * address (cudaGetSymbolAddress, a host-side query); the first call for a
  * given order and precision at that address uploads the tables (again after a
  * device reset): make that first call before any stream capture.  All calls share the array and it keeps the
