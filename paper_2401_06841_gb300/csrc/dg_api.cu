@@ -225,11 +225,13 @@ struct Driver {
     bool have_spare = false;
     double spare = 0;
     // the modes and amplitudes of the present x as the forcing projection takes them
+    // (fixed arrays: nothing is allocated between two steps)
     struct Pack {
         ForceModes fm{};
-        std::vector<int> ints;
-        std::vector<double> amp;
-    } pack;
+        int ints[3 * kMaxModes];
+        double amp[6 * kMaxModes];
+    } pack[2];     // [ip]: of the present x, [ip ^ 1]: of the next update
+    int ip = 0;
     bool packed = false;
     // the next update, made while the device works on a step
     struct Next {
@@ -238,7 +240,6 @@ struct Driver {
         uint64_t rng;
         bool have_spare;
         double spare;
-        Pack pack;
     } nx;
 
     // SplitMix64 (Steele, Lea & Flood 2014)
@@ -332,7 +333,7 @@ struct Driver {
                 rng = nx.rng;
                 have_spare = nx.have_spare;
                 spare = nx.spare;
-                std::swap(pack, nx.pack);
+                ip ^= 1;
                 packed = true;
                 nx.ready = false;
             } else {
@@ -354,7 +355,7 @@ struct Driver {
         const bool have0 = have_spare;
         const double spare0 = spare;
         advance();
-        make_pack(nx.pack);
+        make_pack(pack[ip ^ 1]);
         std::memcpy(nx.x, x, sizeof(double) * 6 * nm);
         nx.rng = rng;
         nx.have_spare = have_spare;
@@ -368,9 +369,9 @@ struct Driver {
     void make_pack(Pack& p) const;
     const Pack& packs()
     {
-        if (!packed) make_pack(pack);
+        if (!packed) make_pack(pack[ip]);
         packed = true;
-        return pack;
+        return pack[ip];
     }
     void advance()
     {
@@ -380,10 +381,9 @@ struct Driver {
                 for (int r = 0; r < 2; ++r) x[m][i][r] = f * x[m][i][r] + c * normal();
     }
     // amplitudes A_k = P_zeta(k) x_k, P_zeta = zeta (I - kk^T/k^2) + (1-zeta) kk^T/k^2
-    void amplitudes(std::vector<double>& amp, std::vector<int>& kvec) const
+    // amp [nm][3][2], kvec [nm][3]
+    void amplitudes(double* amp, int* kvec) const
     {
-        amp.assign(nm * 6, 0.0);
-        kvec.assign(nm * 3, 0);
         for (int m = 0; m < nm; ++m) {
             double k2 = 0;
             for (int i = 0; i < 3; ++i) {
@@ -403,47 +403,46 @@ struct Driver {
     }
 };
 
-// the modes in the order and packing of the forcing projection (dg_force.cuh):
-// packed, pair starts and group starts into ints [3 kMaxModes], the amplitudes
-// (conjugated where kx is flipped) into amp_out [nm][3][2]
-ForceModes pack_modes(int nm, const int* kvec, const double* amp, std::vector<int>& ints, std::vector<double>& amp_out)
+// the modes in the order and packing of the forcing projection (dg_force.cuh): packed
+// modes, pair starts and group starts, and the amplitudes (conjugated where kx is flipped);
+// modes of equal k in the order given
+void pack_modes(int nm, const int* kvec, const double* amp, Driver::Pack& p)
 {
-    std::vector<int> order(nm), sgn(nm);
+    int order[kMaxModes], sgn[kMaxModes];
     for (int m = 0; m < nm; ++m) {
         order[m] = m;
         sgn[m] = kvec[3 * m] < 0 ? -1 : 1;
     }
     auto key = [&](int m, int d) { return sgn[m] * kvec[3 * m + d]; };
-    std::stable_sort(order.begin(), order.end(), [&](int p, int q) {
+    std::sort(order, order + nm, [&](int i, int j) {
         for (int d = 0; d < 3; ++d)
-            if (key(p, d) != key(q, d)) return key(p, d) < key(q, d);
-        return false;
+            if (key(i, d) != key(j, d)) return key(i, d) < key(j, d);
+        return i < j;
     });
-    ints.assign(3 * kMaxModes, 0);
-    amp_out.assign(6 * (size_t)nm, 0.0);
+    std::memset(p.ints, 0, sizeof(p.ints));
     ForceModes fm{nm, 0, 0};
     for (int i = 0; i < nm; ++i) {
         const int m = order[i], kx = key(m, 0), ky = key(m, 1), kz = key(m, 2);
-        ints[i] = kx | (ky + kForceKM) << 8 | (kz + kForceKM) << 16;
+        p.ints[i] = kx | (ky + kForceKM) << 8 | (kz + kForceKM) << 16;
         for (int v = 0; v < 3; ++v) {
-            amp_out[(i * 3 + v) * 2] = amp[(m * 3 + v) * 2];
-            amp_out[(i * 3 + v) * 2 + 1] = sgn[m] * amp[(m * 3 + v) * 2 + 1];
+            p.amp[(i * 3 + v) * 2] = amp[(m * 3 + v) * 2];
+            p.amp[(i * 3 + v) * 2 + 1] = sgn[m] * amp[(m * 3 + v) * 2 + 1];
         }
-        const bool newpair = i == 0 || (ints[i] ^ ints[i - 1]) & 0xffff;
+        const bool newpair = i == 0 || (p.ints[i] ^ p.ints[i - 1]) & 0xffff;
         if (newpair) {
-            if (i == 0 || (ints[i] ^ ints[i - 1]) & 0xff) ints[kForceGroups + fm.ngroup++] = fm.npair;
-            ints[kForcePairs + fm.npair++] = i;
+            if (i == 0 || (p.ints[i] ^ p.ints[i - 1]) & 0xff) p.ints[kForceGroups + fm.ngroup++] = fm.npair;
+            p.ints[kForcePairs + fm.npair++] = i;
         }
     }
-    return fm;
+    p.fm = fm;
 }
 
 void Driver::make_pack(Pack& p) const
 {
-    std::vector<double> a;
-    std::vector<int> k;
+    double a[6 * kMaxModes];
+    int k[3 * kMaxModes];
     amplitudes(a, k);
-    p.fm = pack_modes(nm, k.data(), a.data(), p.ints, p.amp);
+    pack_modes(nm, k, a, p);
 }
 
 // Pinned host memory of a context, for what dg_step and dg_adi_step exchange with
@@ -484,13 +483,11 @@ struct MailBox {
     cudaError_t wait() { return cudaEventSynchronize(done); }
     cudaError_t modes(const Driver::Pack& p, int* d_kvec, double* d_amp, cudaStream_t st)
     {
-        std::memcpy(m->kvec, p.ints.data(), sizeof(int) * p.ints.size());
-        std::memcpy(m->amp, p.amp.data(), sizeof(double) * p.amp.size());
-        const cudaError_t e =
-            cudaMemcpyAsync(d_kvec, m->kvec, sizeof(int) * p.ints.size(), cudaMemcpyHostToDevice, st);
-        return e != cudaSuccess
-                   ? e
-                   : cudaMemcpyAsync(d_amp, m->amp, sizeof(double) * p.amp.size(), cudaMemcpyHostToDevice, st);
+        const size_t na = sizeof(double) * 6 * p.fm.nm;
+        std::memcpy(m->kvec, p.ints, sizeof(p.ints));
+        std::memcpy(m->amp, p.amp, na);
+        const cudaError_t e = cudaMemcpyAsync(d_kvec, m->kvec, sizeof(p.ints), cudaMemcpyHostToDevice, st);
+        return e != cudaSuccess ? e : cudaMemcpyAsync(d_amp, m->amp, na, cudaMemcpyHostToDevice, st);
     }
     ~MailBox()
     {
@@ -562,6 +559,7 @@ struct dg_ctx {
     void* gtab = nullptr;  // forcing: 1D factors (of the mesh and the rule: built by the first projection)
     bool gtab_ready = false;
     double* ana = nullptr; // turbulence statistics accumulators
+    unsigned long long bins[4 * DG_MAX_BINS];  // the density histogram's counts, read back
     cufftHandle fft = 0;   // power-spectrum plan (created on first use)
     int fft_ng = 0;
     Rule1 r1{};            // 1D Gauss rule
@@ -1190,7 +1188,7 @@ int dg_forcing_from_modes(dg_ctx* ctx, int nmodes, const int32_t* kvec, const do
     for (int i = 0; i < 3 * nmodes; ++i) kmaxc = std::max(kmaxc, std::abs((int)kvec[i]));
     if (kmaxc > 8) return fail(ctx, DG_EINVAL, "dg_forcing_from_modes: |k_d| > 8");
     Driver::Pack p;
-    p.fm = pack_modes(nmodes, kvec, amp, p.ints, p.amp);
+    pack_modes(nmodes, kvec, amp, p);
     CK(force_project(ctx, p));
     CK(cudaStreamSynchronize(ctx->st));
     ctx->drv.on = false;
@@ -1674,8 +1672,8 @@ int dg_density_pdf(dg_ctx* ctx, double lo, double hi, int nbins, double* hist)
         CK(ctx->prec == DG_PREC_F64 ? launch_density_pdf<double>(L, (const double*)u, lo, hi, nbins, mean, cnt, weight)
                                     : launch_density_pdf<float>(L, (const float*)u, lo, hi, nbins, mean, cnt, weight));
     }
-    std::vector<unsigned long long> h(4 * (size_t)nbins);
-    CK(cudaMemcpyAsync(h.data(), cnt, sizeof(unsigned long long) * h.size(), cudaMemcpyDeviceToHost, ctx->st));
+    unsigned long long* h = ctx->bins;
+    CK(cudaMemcpyAsync(h, cnt, sizeof(unsigned long long) * 4 * nbins, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
     for (int i = 0; i < nbins; ++i) {
         hist[i] = 0.0;
