@@ -21,6 +21,31 @@ namespace dg {
 // 2 M pairs of the structure function 2.07 -> 1.15 ms, a sampled component 0.52 -> 0.38,
 // its shell sums 0.36 -> 0.13.
 
+// A thread's part of a cell's (K+1)^3 points: all of them, or one row along x
+// (rows: item = (cell, z, y)), whose expansion along z the n threads of a plane repeat.
+template <int K>
+struct CellPart {
+    long c;
+    int z0, z1, y0, y1;
+    __device__ __forceinline__ CellPart(long it, bool rows)
+    {
+        constexpr int n = K + 1;
+        c = rows ? it / (n * n) : it;
+        const int q = rows ? (int)(it - c * n * n) : 0;
+        z0 = rows ? q / n : 0;
+        z1 = rows ? z0 + 1 : n;
+        y0 = rows ? q - z0 * n : 0;
+        y1 = rows ? y0 + 1 : n;
+    }
+};
+// Rows on meshes whose cells are too few to fill the multiprocessors: there a thread's
+// chain through its whole cell is the kernel's time.  Below 64 cells per multiprocessor
+// (21^3): degree 3, 200 bins, rows against cells 8^3 44 and 69 us, 16^3 53 and 77, 28^3 78
+// and 78, 40^3 128 and 114; spectrum 8^3 242 and 319 us, 16^3 300 and 351, 32^3 1103 and
+// 1074; degree 1 8^3 194 and 204, 24^3 226 and 218.
+constexpr long kRowCells = 64;
+static bool cell_rows(const Launch& L) { return L.ncell < kRowCells * (long)L.nsm; }
+
 // sqrt(2m+1) P_m(x), m = 0..K (K <= 3)
 template <int K>
 __device__ __forceinline__ void pnorm_all(double x, double* p)
@@ -186,34 +211,44 @@ __global__ void __launch_bounds__(256) k_mean_rho(const T* __restrict__ u, long 
 // floor((log10(rho/mean) - lo)/ds) comes from single precision, and from FP64 where
 // that lands within tol of a bin edge (tol above its error: same bins).
 // One thread per cell (64 points of degree 3: 16 M points in 6.2 ms with a thread
-// and a full evaluation per point).
+// and a full evaluation per point) or per row of points, see cell_rows.  A block whose
+// samples are fewer than the bins adds to the counters in global memory.  The last
+// block to finish weights the counts and leaves the histogram in their place.
 template <int K>
 __host__ __device__ constexpr int inner(int a)
 {
     return K == 3 ? (a == 1 || a == 2) : (K == 2 ? a == 1 : 0);
 }
 static __device__ __noinline__ bool positive(double x) { return x > 0.0; }
+struct ClassWeights {
+    double w[4];
+};
 
 template <typename T, int K>
 __global__ void __launch_bounds__(128) k_density_pdf(const T* __restrict__ u, long ncell,
                                                      const __grid_constant__ Line t, const double* mean, double lo,
-                                                     double ds, float tol, int nbins,
-                                                     unsigned long long* __restrict__ cnt)
+                                                     double ds, float tol, int nbins, bool rows, bool shared,
+                                                     ClassWeights weight, unsigned int* counter, double* acc)
 {
     constexpr int n = K + 1, b = Dims<K>::b, NP = sf::npair(K);
     extern __shared__ unsigned int s_cnt[];
-    for (int i = threadIdx.x; i < 4 * nbins; i += blockDim.x) s_cnt[i] = 0u;
-    __syncthreads();
+    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(acc);  // [nbins][4]
+    if (shared) {
+        for (int i = threadIdx.x; i < 4 * nbins; i += blockDim.x) s_cnt[i] = 0u;
+        __syncthreads();
+    }
     const double rm = *mean;
     const float irm = (float)(1.0 / rm), lof = (float)lo, ids = (float)(1.0 / ds);
-    for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell; c += (long)gridDim.x * blockDim.x) {
+    const long items = rows ? ncell * n * n : ncell;
+    for (long it = blockIdx.x * (long)blockDim.x + threadIdx.x; it < items; it += (long)gridDim.x * blockDim.x) {
+        const CellPart<K> part(it, rows);
         double r[b], A[NP];
-        load_field<T, K>(u + c * 4 * b, 0, r);
+        load_field<T, K>(u + part.c * 4 * b, 0, r);
 #pragma unroll 1
-        for (int z = 0; z < n; ++z) {
+        for (int z = part.z0; z < part.z1; ++z) {
             sf::plane_eval<double, K>(r, t.P[z], A);
 #pragma unroll 1
-            for (int y = 0; y < n; ++y) {
+            for (int y = part.y0; y < part.y1; ++y) {
                 double q[n], f[n];
                 sf::row_eval<double, K>(A, t.P[y], q);
                 line_values<K>(t, q, f);
@@ -231,14 +266,57 @@ __global__ void __launch_bounds__(128) k_density_pdf(const T* __restrict__ u, lo
                     } else if (fl >= 0.0f && fl < (float)nbins) {
                         bin = (int)fl;
                     }
-                    if (bin >= 0) atomicAdd(&s_cnt[4 * bin + c2 + inner<K>(x)], 1u);
+                    if (bin < 0) continue;
+                    const int at = 4 * bin + c2 + inner<K>(x);
+                    if (shared)
+                        atomicAdd(&s_cnt[at], 1u);
+                    else
+                        atomicAdd(&cnt[at], 1ull);
                 }
             }
         }
     }
+    if (shared) {
+        __syncthreads();
+        for (int i = threadIdx.x; i < 4 * nbins; i += blockDim.x)
+            if (s_cnt[i]) atomicAdd(&cnt[i], (unsigned long long)s_cnt[i]);
+    }
+    __shared__ bool s_last;
+    __threadfence();
     __syncthreads();
-    for (int i = threadIdx.x; i < 4 * nbins; i += blockDim.x)
-        if (s_cnt[i]) atomicAdd(&cnt[i], (unsigned long long)s_cnt[i]);
+    if (threadIdx.x == 0) s_last = atomicAdd(counter, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // bin i is written over the counts of bin i / 4, which its own pass or an earlier one
+    // has read; eight bins of a thread at a time, their loads in flight together.  (Most of
+    // many bins are empty: no FP64 conversions there.)
+    constexpr int NB = 8;
+    for (int i0 = 0; i0 < nbins; i0 += NB * blockDim.x) {
+        ulonglong2 q[NB][2];
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            const int i = i0 + j * blockDim.x + threadIdx.x;
+            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(cnt + 4 * i);
+            q[j][0] = q[j][1] = make_ulonglong2(0ull, 0ull);
+            if (i < nbins) q[j][0] = __ldcg(p), q[j][1] = __ldcg(p + 1);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < NB; ++j) {
+            const int i = i0 + j * blockDim.x + threadIdx.x;
+            double h = 0.0;
+            if (q[j][0].x | q[j][0].y | q[j][1].x | q[j][1].y) {
+                h += (double)q[j][0].x * weight.w[0];
+                h += (double)q[j][0].y * weight.w[1];
+                h += (double)q[j][1].x * weight.w[2];
+                h += (double)q[j][1].y * weight.w[3];
+            }
+            if (i < nbins) acc[i] = h;
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) *counter = 0u;
 }
 
 // structure-function pairs: item = j * npairs + p, five uniforms per item
@@ -293,26 +371,28 @@ __global__ void __launch_bounds__(256) k_structure(const T* __restrict__ u, int 
 
 // velocity component d on the Ng = (K+1) N grid, x_g = (g + 1/2)/Ng:
 // out[(gz Ng + gy) Ng + gx]
-// one thread per cell: rho and m_d axis by axis at the cell's (K+1)^3 grid points
+// one thread per cell, or per row of points on small meshes: rho and m_d axis by axis at
+// the cell's (K+1)^3 grid points
 template <typename T, int K>
 __global__ void __launch_bounds__(128) k_sample(const T* __restrict__ u, int N, int d, const __grid_constant__ Line t,
-                                                double* __restrict__ out)
+                                                bool rows, double* __restrict__ out)
 {
     constexpr int p = K + 1, b = Dims<K>::b, NP = sf::npair(K);
-    const long Ng = (long)p * N, ncell = (long)N * N * N;
-    for (long c = blockIdx.x * (long)blockDim.x + threadIdx.x; c < ncell; c += (long)gridDim.x * blockDim.x) {
+    const long Ng = (long)p * N, ncell = (long)N * N * N, items = rows ? ncell * p * p : ncell;
+    for (long it = blockIdx.x * (long)blockDim.x + threadIdx.x; it < items; it += (long)gridDim.x * blockDim.x) {
+        const CellPart<K> part(it, rows);
         int ix, iy, iz;
-        cell_xyz(c, N, ix, iy, iz);
+        cell_xyz(part.c, N, ix, iy, iz);
         double r[b], m[b], A[NP], M[NP];
-        load_field<T, K>(u + c * 4 * b, 0, r);
-        load_field<T, K>(u + c * 4 * b, 1 + d, m);
+        load_field<T, K>(u + part.c * 4 * b, 0, r);
+        load_field<T, K>(u + part.c * 4 * b, 1 + d, m);
         double* o = out + ((long)iz * p * Ng + (long)iy * p) * Ng + (long)ix * p;
 #pragma unroll 1
-        for (int z = 0; z < p; ++z) {
+        for (int z = part.z0; z < part.z1; ++z) {
             sf::plane_eval<double, K>(r, t.P[z], A);
             sf::plane_eval<double, K>(m, t.P[z], M);
 #pragma unroll 1
-            for (int y = 0; y < p; ++y) {
+            for (int y = part.y0; y < part.y1; ++y) {
                 double q[p], f[p], g[p];
                 sf::row_eval<double, K>(A, t.P[y], q);
                 line_values<K>(t, q, f);
@@ -467,25 +547,33 @@ static Line line_of(const double* x, int n)
     return t;
 }
 
-// cnt [nbins][4]: samples per bin and weight class; the weights of the classes in
-// weight[4] (products of three 1D weights / 8, over the cells)
+// acc: zeroed room of [nbins][4] counts (samples per bin and weight class), the histogram
+// [nbins] when the kernel is through; a class's weight: a product of three 1D weights / 8,
+// over the cells
 template <typename T, int K>
-static cudaError_t pdf_k(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean,
-                         unsigned long long* cnt, double* weight)
+static cudaError_t pdf_k(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean, double* acc)
 {
     k_mean_rho<T, K><<<grid_of(L.ncell, L.nsm), 256, 0, L.st>>>(u, L.ncell, mean);
     const double ds = (hi - lo) / nbins;
     // error of the single-precision bin coordinate: the logarithm's (below 1e-6 of
     // its size) over ds and the rounding of the coordinate
     const double tol = 1e-6 * (2.0 + std::fabs(lo) + std::fabs(hi)) / ds + 1e-6 * nbins;
-    long g = (L.ncell + 127) / 128;
+    constexpr int n = K + 1;
+    const bool rows = cell_rows(L);
+    const long items = rows ? L.ncell * n * n : L.ncell;
+    long g = (items + 127) / 128;
     if (g > 16L * L.nsm) g = 16L * L.nsm;
-    const size_t sm = sizeof(unsigned int) * 4 * nbins;
-    k_density_pdf<T, K><<<(int)g, 128, sm, L.st>>>(u, L.ncell, line_of(L.r1.x, K + 1), mean, lo, ds,
-                                                   (float)std::min(tol, 1.0), nbins, cnt);
     const double wo = L.r1.w[0], wi = K >= 2 ? L.r1.w[1] : wo;
-    for (int c = 0; c < 4; ++c)
-        weight[c] = std::pow(wi, c) * std::pow(wo, 3 - c) / 8.0 / (double)L.ncell;
+    ClassWeights w;
+    for (int c = 0; c < 4; ++c) w.w[c] = std::pow(wi, c) * std::pow(wo, 3 - c) / 8.0 / (double)L.ncell;
+    // counters of the block's own where its samples are no fewer than the bins: 16^3 of degree
+    // 3 by rows, 200 bins 53 us so, 109 on the common ones; 8^3, 2000 bins 54 us on the common
+    // ones, 108 by cells on the block's own
+    const bool shared = (items + g - 1) / g * (rows ? n : n * n * n) >= nbins;
+    const size_t sm = shared ? sizeof(unsigned int) * 4 * nbins : 0;
+    k_density_pdf<T, K><<<(int)g, 128, sm, L.st>>>(u, L.ncell, line_of(L.r1.x, n), mean, lo, ds,
+                                                   (float)std::min(tol, 1.0), nbins, rows, shared,
+                                                   w, &L.ctl->cnt_diag, acc);
     return cudaGetLastError();
 }
 
@@ -503,17 +591,17 @@ static cudaError_t sample_k(const Launch& L, const T* u, int d, double* out)
 {
     double x[4];
     for (int a = 0; a <= K; ++a) x[a] = (2.0 * a + 1.0) / (K + 1) - 1.0;
-    long g = (L.ncell + 127) / 128;
+    const bool rows = cell_rows(L);
+    long g = (L.ncell * (rows ? (K + 1) * (K + 1) : 1) + 127) / 128;
     if (g > 16L * L.nsm) g = 16L * L.nsm;
-    k_sample<T, K><<<(int)g, 128, 0, L.st>>>(u, L.N, d, line_of(x, K + 1), out);
+    k_sample<T, K><<<(int)g, 128, 0, L.st>>>(u, L.N, d, line_of(x, K + 1), rows, out);
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t launch_density_pdf(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean,
-                               unsigned long long* cnt, double* weight)
+cudaError_t launch_density_pdf(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean, double* acc)
 {
-    DG_DISPATCH(pdf_k, u, lo, hi, nbins, mean, cnt, weight);
+    DG_DISPATCH(pdf_k, u, lo, hi, nbins, mean, acc);
 }
 
 template <typename T>
@@ -539,8 +627,7 @@ cudaError_t launch_shell(const Launch& L, const void* F, int Ng, int nbins, doub
 }
 
 #define DG_ANALYSIS_INSTANTIATE(T)                                                                               \
-    template cudaError_t launch_density_pdf<T>(const Launch&, const T*, double, double, int, double*,           \
-                                               unsigned long long*, double*);                                   \
+    template cudaError_t launch_density_pdf<T>(const Launch&, const T*, double, double, int, double*, double*);  \
     template cudaError_t launch_structure<T>(const Launch&, const T*, int, long, unsigned long long, double*);   \
     template cudaError_t launch_sample<T>(const Launch&, const T*, int, double*);
 DG_ANALYSIS_INSTANTIATE(float)

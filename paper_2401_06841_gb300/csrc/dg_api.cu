@@ -559,7 +559,6 @@ struct dg_ctx {
     void* gtab = nullptr;  // forcing: 1D factors (of the mesh and the rule: built by the first projection)
     bool gtab_ready = false;
     double* ana = nullptr; // turbulence statistics accumulators
-    unsigned long long bins[4 * DG_MAX_BINS];  // the density histogram's counts, read back
     cufftHandle fft = 0;   // power-spectrum plan (created on first use)
     int fft_ng = 0;
     Rule1 r1{};            // 1D Gauss rule
@@ -1661,24 +1660,17 @@ int dg_density_pdf(dg_ctx* ctx, double lo, double hi, int nbins, double* hist)
     if (!hist || nbins < 1 || nbins > DG_MAX_BINS || !(hi > lo))
         return fail(ctx, DG_EINVAL, "dg_density_pdf: bad bins or null buffer");
     if (!ctx->state_set) return fail(ctx, DG_ESTATE, "dg_density_pdf: no state set");
-    unsigned long long* cnt = reinterpret_cast<unsigned long long*>(ctx->ana);  // [nbins][4 weight classes]
     double* mean = ctx->ana + 4 * DG_MAX_BINS;
-    double weight[4];
     CK(cudaMemsetAsync(ctx->ana, 0, sizeof(double) * (4 * DG_MAX_BINS + 1), ctx->st));
     Launch L = make_launch(ctx);
     {
         Timed tm(ctx, KIND_OTHER);
         const void* u = ctx->reg[ctx->cur];
-        CK(ctx->prec == DG_PREC_F64 ? launch_density_pdf<double>(L, (const double*)u, lo, hi, nbins, mean, cnt, weight)
-                                    : launch_density_pdf<float>(L, (const float*)u, lo, hi, nbins, mean, cnt, weight));
+        CK(ctx->prec == DG_PREC_F64 ? launch_density_pdf<double>(L, (const double*)u, lo, hi, nbins, mean, ctx->ana)
+                                    : launch_density_pdf<float>(L, (const float*)u, lo, hi, nbins, mean, ctx->ana));
     }
-    unsigned long long* h = ctx->bins;
-    CK(cudaMemcpyAsync(h, cnt, sizeof(unsigned long long) * 4 * nbins, cudaMemcpyDeviceToHost, ctx->st));
+    CK(cudaMemcpyAsync(hist, ctx->ana, sizeof(double) * nbins, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));
-    for (int i = 0; i < nbins; ++i) {
-        hist[i] = 0.0;
-        for (int c = 0; c < 4; ++c) hist[i] += (double)h[4 * i + c] * weight[c];
-    }
     return DG_OK;
 }
 

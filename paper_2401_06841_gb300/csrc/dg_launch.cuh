@@ -103,8 +103,7 @@ cudaError_t launch_adi_shift(const Launch& L, void* u, double d);
 
 // turbulence statistics (dg_analysis.cu)
 template <typename T>
-cudaError_t launch_density_pdf(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean,
-                               unsigned long long* cnt, double* weight);
+cudaError_t launch_density_pdf(const Launch& L, const T* u, double lo, double hi, int nbins, double* mean, double* acc);
 template <typename T>
 cudaError_t launch_structure(const Launch& L, const T* u, int nbins, long npairs, unsigned long long seed, double* acc);
 template <typename T>
