@@ -7,7 +7,8 @@
  * ------------------------------------------------------------------------
  * Data layout (all device buffers are owned by the caller, e.g. torch
  * tensors; the library never allocates or frees device memory; a context holds
- * 32 KB of pinned host memory for what a step exchanges with the device):
+ * 32 KB of pinned host memory, in whole pages, for what a step exchanges with the
+ * device):
  *   N cells per axis, unit box, h = 1/N; cell c = (iz*N + iy)*N + ix.
  *   degree k in {1,2,3}; b = (k+1)(k+2)(k+3)/6 modes; n = k+1 Gauss points
  *   per axis.  Basis phi_{ijl}(xi) = Pn_i(xi_x) Pn_j(xi_y) Pn_l(xi_z),

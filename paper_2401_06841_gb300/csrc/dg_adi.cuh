@@ -27,10 +27,9 @@ struct AdiGas {
     T gamma;   // gamma
     T g1;      // gamma - 1
     T ig1;     // 1 / (gamma - 1)
-    T cth;     // reset mode: cs^2 / (gamma - 1), the thermal energy per unit mass
     T kap;     // energy offset per unit mass
     T c0;      // (gamma - 1) kap: the pressure of the offset per unit density
-    T cres;    // cth - kap: the thermal energy per unit mass the reset leaves in e_s
+    T cres;    // reset mode: cs^2 / (gamma - 1) - kap, the thermal energy per unit mass it leaves in e_s
 };
 
 constexpr int cmax(int a, int b) { return a > b ? a : b; }

@@ -69,7 +69,6 @@ cudaError_t adi_k(const Launch& L, double gamma, const AdiLaunch& t)
     a.gas.gamma = T(gamma);
     a.gas.g1 = T(gamma - 1.0);
     a.gas.ig1 = T(1.0 / (gamma - 1.0));
-    a.gas.cth = T(t.cs_reset * t.cs_reset / (gamma - 1.0));
     a.gas.kap = T(t.kap);
     a.gas.c0 = T((gamma - 1.0) * t.kap);
     a.gas.cres = T(t.cs_reset * t.cs_reset / (gamma - 1.0) - t.kap);

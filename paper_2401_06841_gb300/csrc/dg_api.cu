@@ -2139,12 +2139,10 @@ int dg_adi_step(dg_adi_ctx* ctx, int nsteps, double fixed_dt, double* t_out, dou
                 t.u_n = ctx->reg[A];
                 t.out = ctx->reg[out[s]];
                 t.pr_in = pr[s & 1];
-                t.pr_out = pr[(s + 1) & 1];
                 // the stages after the first project their own input in their volume kernel
                 t.flags = (s > 0 ? F_SELFPROJ : 0) | (force ? F_FORCE : 0);
                 t.ahat = ctx->ahat;
                 t.abar_in = s & 1;
-                t.abar_out = (s + 1) & 1;
                 t.beta = RW[s];
                 rk_weights(ctx->rk, s, ctx->prec != DG_PREC_F64, t.rk_a, t.rk_b);
                 ACK(adi_go(ctx, t));

@@ -170,8 +170,8 @@ static cudaError_t tile_kb(const Launch& L, const TileLaunch& t)
 // Split-BF16 products (x3_backend 1) and the diffusion operator, whose gradients the
 // sum-factorised kernels don't form, take the fused kernel's dense products; all else the
 // sum-factorised kernels, faster at every size and degree measured (16^3 P1 FP64, 20
-// driven steps: 2.3 ms for 13.1; 64^3 P3 FP32, 4 steps: 3.9 for 20.3; 128^3 P2, 2 steps:
-// 7.1 for 39.6).
+// driven steps: 2.3 ms for 13.1; 64^3 P3 FP32, 4 steps: 3.8 for 20.3; 128^3 P2, 2 steps:
+// 7.0 for 39.6).
 template <typename T, int K>
 cudaError_t tile_k(const Launch& L, const TileLaunch& t)
 {

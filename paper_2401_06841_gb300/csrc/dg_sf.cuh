@@ -26,9 +26,9 @@
 // their projection stay in its registers, and the faces of a cell meet in shared
 // memory once per brick.
 //
-// A driven SSP-RK3 step of 64^3 cells of degree 3 in FP32 takes 0.99 ms (volume 117 to
-// 169, faces 130 us a stage, projection 66), where the dense products of the fused stage
-// kernel (dg_tile.cuh) took 5.07; 128^3 of degree 2 3.56 ms for 19.8; one FP64
+// A driven SSP-RK3 step of 64^3 cells of degree 3 in FP32 takes 0.96 ms (volume 112 to
+// 158, faces 130 us a stage, projection 63), where the dense products of the fused stage
+// kernel (dg_tile.cuh) took 5.07; 128^3 of degree 2 3.50 ms for 19.8; one FP64
 // right-hand side of 24^3 of degree 3 0.56 ms for 1.79.
 #pragma once
 
@@ -493,9 +493,10 @@ struct VolCfg {
 // velocity projection -> vh_out (VABS: and of |v|), with the forcing sums when
 // FORCE.  !VOL: the projection launch (CFL bound with a.dtf).
 //
-// Bound: FP32 instruction issue and its latency: 13.7 thousand instructions per cell at
-// degree 3 with FORCE and PROJ go out in 58 % of the issue slots (FMA pipe 42 %, HBM
-// 18 %), with the 12 warps per SM that 168 registers leave.  FP64 by the FP64 pipe.
+// Bound: FP32 instruction issue and its latency, with the 12 warps per SM that 168
+// registers leave: at degree 3 with FORCE and PROJ 13.5 thousand instructions per cell go
+// out in 60 % of the issue slots (FMA pipe 44 %, HBM 20 %), with PROJ alone in 64 %, the
+// volume term alone in 70 %.  FP64 by the FP64 pipe.
 // Blocks per SM in FP32: as many as the registers allow without spilling more than a few
 // (degree 2: 5 blocks 128^3 7.12 ms for 2 steps, 4 blocks 7.19, 6 blocks 7.23).
 template <typename T, int K, bool VOL, bool FORCE, bool PROJ, bool VABS>
@@ -946,8 +947,8 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? (VOL 
 // 96 operand rows where those would read 224.  Bricks past the end of the mesh hold the
 // periodic images of its cells, which are the neighbours the last cells need.
 // Bound: latency between the phases of a brick (rows in, traces and fluxes, rows of the
-// stage in, combine), with the 12 warps per SM that 168 registers and 67 KB leave at
-// degree 3: issue slots 45 %, FMA pipe 31 %, HBM 35 %, no pipe near its limit.  64^3 of
+// stage in, combine), with the 12 warps per SM that 168 registers and 53 KB leave at
+// degree 3: issue slots 47 %, FMA pipe 32 %, HBM 37 %, no pipe near its limit.  64^3 of
 // degree 3 FP32: 130 us (2.3 TB/s; 212 us with the six faces of 32 consecutive cells),
 // 256^3 8.3 ms.  Four blocks with the traces in shared memory were slower
 // (0.83-0.9x), packed pairs of FP32 and a prefetch of the next bricks to L2 no faster.
@@ -1081,8 +1082,8 @@ __device__ __forceinline__ void hll_normal(T cs, T cs2, const T* WL, const T* WR
     }
 }
 
-// Bound: FP32 instruction issue (about 8 thousand instructions per cell at degree 3).
-// Blocks per SM in FP32, likewise: degree 1 8 blocks (96^3: 0.377 ms a step; 6: 0.394),
+// 9.1 thousand instructions per cell at degree 3, bound as above.
+// Blocks per SM in FP32: degree 1 8 blocks (96^3: 0.377 ms a step; 6: 0.394),
 // degree 2 4 (128^3, 2 steps: 7.19 ms; 5: 7.28), degree 3 3.
 template <typename T, int K, int RS, bool STAGE>
 __global__ void __launch_bounds__(128, sizeof(T) == 4 ? (K == 1 ? 8 : K == 2 ? 4 : 3) : 1)

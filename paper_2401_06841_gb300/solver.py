@@ -20,6 +20,8 @@ class Solver:
 
     N cells per axis, degree k (1..3), sound speed cs; precision 'f64', 'f32'
     or 'x3'; av 'off' | 'vnr' | 'learned'; face flux riemann 'rusanov' | 'hll' | 'hllc';
+    x3_backend (precision 'x3' alone): 'tcgen05', the default's name since its kernels
+    were tensor-core ones, selects the FP32 kernels, 'mma' the split-BF16 products;
     positivity 'scale' (rescale stage outputs) | 'repeat' (also repeat the step
     with troubled cells of u^n flattened, Sec. 3.1)."""
 
