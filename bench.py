@@ -124,7 +124,8 @@ def peaks():
 
 
 # committed ncu summaries of the stage kernels, per variant: (file, kernel sources)
-PROFILE = {"x3": ("k_sf_stage_x3_64c_k3.md", ("dg_sf.cuh", "dg_sf_impl.cuh", "dg_kernels.cuh", "dg_common.cuh"))}
+PROFILE = {"x3": ("k_sf_stage_x3_64c_k3.md", ("dg_sf.cuh", "dg_brick.cuh", "dg_sf_impl.cuh", "dg_kernels.cuh",
+                                                "dg_common.cuh"))}
 
 
 def profiled_traffic(variant, N):
