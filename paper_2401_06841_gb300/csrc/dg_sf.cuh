@@ -1052,15 +1052,21 @@ __device__ __forceinline__ void rusanov_normal(T cs, T cs2, const T* WL, const T
 //   q_R = w_R rho_R (v_n,R - S_R), p* = cs^2 (w_L rho_L + w_R rho_R).
 // The smaller weight is formed from its own bound and the larger one as the rest: a clamped
 // bound then leaves the upwind flux exactly, on either side, and a bound near zero lets no
-// rounding of the other weight carry a dense side's flux into a thin one.
+// rounding of the other weight carry a dense side's flux into a thin one.  Outside the bounds
+// the upwind state stands on both sides: a downwind vacuum or NaN does not enter.
 // CONTACT (HLLC for p = cs^2 rho): the tangential momenta cross with the mass flux at the
-// tangential velocity of the side the contact S_M = m*/rho* leaves behind (the upwind side
-// outside the bounds)
+// tangential velocity of the side the contact S_M = m*/rho* leaves behind
 template <typename T, bool CONTACT>
-__device__ __forceinline__ void hll_normal(T cs, T cs2, const T* WL, const T* WR, T* F)
+__device__ __forceinline__ void hll_normal(T cs, T cs2, const T* L, const T* R, T* F)
 {
+    const T SL = fmin(L[1], R[1]) - cs, SR = fmax(L[1], R[1]) + cs;
+    T WL[4], WR[4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v) {
+        WL[v] = SR <= T(0) ? R[v] : L[v];
+        WR[v] = SL >= T(0) ? L[v] : R[v];
+    }
     const T vl = WL[1], vr = WR[1];
-    const T SL = fmin(vl, vr) - cs, SR = fmax(vl, vr) + cs;
     const T sl = fmin(SL, T(0)), sr = fmax(SR, T(0));
     const bool nearer = sr < -sl;  // of the two bounds S_R
     const T ws = (nearer ? sr : -sl) * rcp<T>(sr - sl), wb = T(1) - ws;
@@ -1073,7 +1079,7 @@ __device__ __forceinline__ void hll_normal(T cs, T cs2, const T* WL, const T* WR
         // signs of rho* and m* (times S_R - S_L > 0)
         const T aL = WL[0] * (SL - vl), aR = WR[0] * (SR - vr);
         const T ms = aR * vr - aL * vl - cs2 * (WR[0] - WL[0]);
-        const bool left = SL >= T(0) || (SR > T(0) && (aR - aL > T(0)) == (ms >= T(0)));
+        const bool left = (aR - aL > T(0)) == (ms >= T(0));
         F[2] = F[0] * (left ? WL[2] : WR[2]);
         F[3] = F[0] * (left ? WL[3] : WR[3]);
     } else {

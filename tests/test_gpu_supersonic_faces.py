@@ -57,3 +57,24 @@ def test_upwind_flux_of_a_thin_gas_beside_a_dense_one(k, riemann, prec):
             got = s.rhs(u, None, 0.0).cpu().numpy().astype(np.float64)
             err = np.abs(got - O.rhs(cfg, u, None, 0.0))[inner].max(axis=(1, 2)) / scale[inner]
             assert err.max() < TOL[prec], (axis, sign, err.max())
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["f64", "f32"])
+@pytest.mark.parametrize("riemann", ["hll", "hllc"])
+@pytest.mark.parametrize("bad", ["nan", "vacuum"])
+def test_a_downwind_vacuum_or_nan_does_not_enter(bad, riemann, prec):
+    # uniform flow at 3 cs along an axis past one cell of NaN or of nothing (its velocity is
+    # 0/0): the cell upwind of it has the right-hand side of the undisturbed flow
+    k, n = 2, 8
+    s = Solver(n, k, precision=prec, riemann=riemann, av="off")
+    for axis in range(3):
+        for sign in (-1, 1):
+            u = I.random_state(n, k, seed=95, v_rms=0.1)
+            u[:, 1 + axis] += 3.0 * sign * u[:, 0]
+            c = (3 * n + 4) * n + 5
+            up = c - sign * (1, n, n * n)[axis]
+            ref = s.rhs(u, None, 0.0)
+            u[c] = np.nan if bad == "nan" else 0.0
+            got = s.rhs(u, None, 0.0)
+            assert torch.equal(got[up], ref[up]), (axis, sign)
