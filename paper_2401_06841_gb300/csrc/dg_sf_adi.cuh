@@ -22,7 +22,7 @@
 // integral of the energy source), [1] dissipated energy (the thermal energy the
 // reset takes out).
 // Bound as in dg_sf.cuh.  64^3 of degree 3 FP32: an SSP-RK3 step takes 1.27 ms (volume
-// 106 to 148, faces 238 us a stage, projection 73), on dense products 5.4; 48^3 of degree
+// 107 to 148, faces 236 us a stage, projection 79), on dense products 5.4; 48^3 of degree
 // 2, driven with HLLC and the reset, 0.40 ms for 2.1.
 #pragma once
 
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(32 * (K + 1), sizeof(T) == 4 ? (K == 3 ? 3 : K
                         f[3][i] = vz;
                         f[NF - 1][i] = pd;
                         if (MODE == SFA_PROJECT && a.dtf && valid) {
-                            const T cs = fast_sqrt<T>(a.gas.gamma * (pd + c0g * rho) * ir);
+                            const T cs = rounded_sqrt<T>(a.gas.gamma * (pd + c0g * rho) * ir);
                             const T sp = fabs(f[1][i]) + fabs(f[2][i]) + fabs(f[3][i]) + T(3) * cs;
                             smax = sp > smax ? sp : smax;
                         }
